@@ -256,11 +256,7 @@ int higgs_dequantize(const higgs_desc* d, const void* packed, const void* scales
     if (!packed || !scales || !grid || !W_out || !workspace) return HIGGS_ERR_INVALID_ARG;
     if (!aligned(packed, 16) || !aligned(scales, 16) || !aligned(W_out, 16) || !aligned(workspace, 256)) return HIGGS_ERR_INVALID_ARG;
     if (workspace_bytes < higgs_workspace_bytes(d, HIGGS_OP_QUANTIZE, 0)) return HIGGS_ERR_WORKSPACE;
-    cudaStream_t st = as_stream(stream);
-    uint8_t* canonical = static_cast<uint8_t*>(workspace);
-    rc = launch_unpack(*d, packed, canonical, st);
-    if (rc != HIGGS_OK) return rc;
-    return launch_dequantize(*d, canonical, scales, grid, W_out, w_dtype, st);
+    return launch_dequantize(*d, packed, scales, grid, W_out, w_dtype, as_stream(stream));
 }
 
 int higgs_layer_error(const higgs_desc* d, const void* W, int w_dtype, const void* packed, const void* scales,
@@ -273,12 +269,9 @@ int higgs_layer_error(const higgs_desc* d, const void* W, int w_dtype, const voi
     if (!W || !packed || !scales || !grid || !workspace) return HIGGS_ERR_INVALID_ARG;
     if (!aligned(W, 16) || !aligned(packed, 16) || !aligned(scales, 16) || !aligned(workspace, 256)) return HIGGS_ERR_INVALID_ARG;
     if (workspace_bytes < higgs_workspace_bytes(d, HIGGS_OP_QUANTIZE, 0)) return HIGGS_ERR_WORKSPACE;
-    cudaStream_t st = as_stream(stream);
-    uint8_t* canonical = static_cast<uint8_t*>(workspace);
-    rc = launch_unpack(*d, packed, canonical, st);
-    if (rc != HIGGS_OK) return rc;
-    rc = launch_layer_error(*d, canonical, scales, grid, W, w_dtype, sums_out, st);
-    return rc != HIGGS_OK ? rc : launch_error_ratio(sums_out, st);
+    // (the workspace is at least the 8 KB of canonical codes of one 16 x 1024 tile: room for the partial sums)
+    static_assert(kErrorPartials * 2 * sizeof(double) <= 16 * 512, "partial sums fit the smallest workspace");
+    return launch_layer_error(*d, packed, scales, grid, W, w_dtype, sums_out, static_cast<double*>(workspace), as_stream(stream));
 }
 
 int higgs_allocate_bits(int32_t num_layers, int32_t num_options, const double* alpha, const double* t2, const int32_t* bits64,

@@ -172,6 +172,54 @@ __device__ __forceinline__ void apply_signs1024(float (&v)[32], uint64_t xi, int
     }
 }
 
+// The 1024-point transform with one exchange through shared memory instead of five shuffle stages.  A warp owns one
+// group; before, lane l holds v[c*8 + e] = element c*256 + l*8 + e (the mapping above: index bits 0-2, 8, 9 in
+// registers, bits 3-7 across lanes); after, lane c*8 + e holds v[j] = element c*256 + j*8 + e (bits 3-7 in registers).
+// Same butterflies in the same order of stages as fwht1024_warp, so the values are bit-identical to it.  160 shuffles and
+// 160 fused multiply-adds become 8 vector stores, 32 loads and 160 additions: 64 shared-memory wavefronts instead of
+// 160.  `ex`: this warp's exchange buffer, kFwhtExchange floats, 16-byte aligned; rows of 36 floats keep the vector
+// stores (lane l writes row l) and the loads (lane l reads column l) free of bank conflicts.
+constexpr int kFwhtRow = 36;
+constexpr int kFwhtExchange = 32 * kFwhtRow;
+__device__ __forceinline__ void butterflies32(float (&v)[32]) {
+#pragma unroll
+    for (int h = 1; h < 32; h <<= 1) {
+#pragma unroll
+        for (int r = 0; r < 32; ++r) {
+            if ((r & h) == 0) {
+                const float a = v[r], b = v[r | h];
+                v[r] = a + b;
+                v[r | h] = a - b;
+            }
+        }
+    }
+}
+__device__ __forceinline__ void fwht1024_to_columns(float (&v)[32], float* ex, int lane) {
+    butterflies32(v);
+    __syncwarp();            // (the buffer's previous readers)
+#pragma unroll
+    for (int r = 0; r < 32; r += 4)
+        *reinterpret_cast<float4*>(ex + lane * kFwhtRow + r) = make_float4(v[r], v[r + 1], v[r + 2], v[r + 3]);
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = ex[j * kFwhtRow + lane];
+    butterflies32(v);
+}
+// The inverse direction (H is symmetric: the same transform, columns in, rows out).
+__device__ __forceinline__ void fwht1024_from_columns(float (&v)[32], float* ex, int lane) {
+    butterflies32(v);
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 32; ++j) ex[j * kFwhtRow + lane] = v[j];
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < 32; r += 4) {
+        const float4 q = *reinterpret_cast<const float4*>(ex + lane * kFwhtRow + r);
+        v[r] = q.x; v[r + 1] = q.y; v[r + 2] = q.z; v[r + 3] = q.w;
+    }
+    butterflies32(v);
+}
+
 // element index inside the group of register r of lane l (see above)
 __device__ __forceinline__ int fwht_index(int lane, int r) { return (r >> 3) * 256 + lane * 8 + (r & 7); }
 
@@ -188,7 +236,7 @@ int launch_encode(const higgs_desc& d, const void* W, int w_dtype, const float* 
                   uint8_t* canonical, void* packed, void* scales, bool* packed_done, cudaStream_t st);
 int launch_pack(const higgs_desc& d, const uint8_t* canonical, void* packed, cudaStream_t st);
 int launch_unpack(const higgs_desc& d, const void* packed, uint8_t* canonical, cudaStream_t st);
-int launch_dequantize(const higgs_desc& d, const uint8_t* canonical, const void* scales, const float* grid, void* W_out,
+int launch_dequantize(const higgs_desc& d, const void* packed, const void* scales, const float* grid, void* W_out,
                       int w_dtype, cudaStream_t st);
 // Further destinations of a product's output - the all-gather of a row-sharded layer fused into the epilogue: the same
 // [B][ldy] window in the memory of other devices (peer-mapped pointers), written with plain stores.
@@ -218,8 +266,10 @@ int launch_convert_out(const float* y32, void* y, int y_dtype, size_t count, cud
 size_t make_grid_workspace(int p, int n, int64_t m);
 int launch_make_grid(int p, int n, const float* samples, int64_t m, int max_iters, float* grid_out, float* mse_out,
                      int32_t* iters_out, void* ws, cudaStream_t st);
-int launch_layer_error(const higgs_desc& d, const uint8_t* canonical, const void* scales, const float* grid, const void* W,
-                       int w_dtype, double* sums, cudaStream_t st);
+// partials: scratch of at least kErrorPartials pairs of doubles
+constexpr int kErrorPartials = 512;
+int launch_layer_error(const higgs_desc& d, const void* packed, const void* scales, const float* grid, const void* W,
+                       int w_dtype, double* sums, double* partials, cudaStream_t st);
 int allocate_bits(int L, int J, const double* alpha, const double* t2, const int32_t* bits64, const int64_t* sizes,
                   int64_t budget64, int32_t* choice_out, double* objective_out);
 int launch_encode_general(int p, int n, int64_t N, int64_t K, uint64_t xi, const void* W, int w_dtype, const float* grid,

@@ -1,153 +1,303 @@
 // Dequantisation to the original space (Appendix F, "Dequantization"): for every (row, group)
-//   r = scale * G[codes]  (the layer in the rotated space),   w^ = diag(sign) (H / sqrt(g)) r.
-// Validation / export path, not on the decode hot path (which never leaves the rotated space).
+//   r = scale * G[codes]  (the layer in the rotated space),   w^ = diag(sign) (H / sqrt(g)) r,
+// and the layer's relative error t^2 (Section 5, "Measuring Grid Parameters").  Both read the packed stream directly.
 #include "common.cuh"
 
 namespace higgs {
 
 namespace {
 
-// The dequantised group (row, gi) in registers: lane l gets the 32 elements idx = c*256 + l*8 + e of the group (the
-// mapping of fwht1024_warp), so its codes are 4 runs of 8/p consecutive canonical codes.
-template <int P>
-__device__ __forceinline__ void dequantize_group(const uint8_t* __restrict__ canonical, const __half* __restrict__ scales,
-                                                 const float* __restrict__ grid, int64_t K, uint64_t xi, int64_t row, int64_t gi,
-                                                 int lane, float (&v)[32]) {
-    const int64_t groups = K / kGroup;
-    const float scale = __half2float(scales[((row / kRowTile) * groups + gi) * kRowTile + (row % kRowTile)]);   // tile-major
-    const uint8_t* crow = canonical + row * (K / P) + gi * (kGroup / P);
+constexpr int kDqWarps = 8;            // a block takes one row tile (16 rows) x one group per turn; warp w rows w and w + 8
+
+// The table indices of rows w (low halves) and w + 8 of one (row tile, group), as this lane needs them after
+// fwht1024_to_columns: lane c*8 + e holds elements c*256 + j*8 + e, j = 0..31, i.e. pair (e >> 1) of every second
+// 4-pair step of the 64-input blocks 4c .. 4c + 3.  In every packed format the indices of one such pair position for
+// the two rows are one contiguous run of packed lane L = 4 w + (e >> 1): the lanes of a warp read whole 64-byte runs.
+template <int FMT>
+struct ColumnCodes {
+    static constexpr bool SIX = FMT == 1, NIB = FMT == 2, B8 = FMT == 3;
+    uint32_t w[SIX ? 12 : NIB ? 8 : B8 ? 32 : 16];
+    __device__ __forceinline__ void load(const uint8_t* __restrict__ packed, int64_t first_block, int warp, int lane) {
+        const int c = lane >> 3, L = warp * 4 + ((lane & 7) >> 1);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const int e0 = c * 256 + lane * 8;                 // first element of the chunk inside the group
-        if (P == 2) {
-            const uint32_t w = *reinterpret_cast<const uint32_t*>(crow + e0 / 2);      // 4 codes = 8 elements
+        for (int jj = 0; jj < 4; ++jj) {
+            const int64_t blk = first_block + 4 * c + jj;
+            if (SIX) {
+                if (jj & 1) continue;                                    // a super-block covers blocks jj and jj + 1
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const float2 gp = __ldg(reinterpret_cast<const float2*>(grid) + ((w >> (8 * t)) & 0xffu));
-                v[c * 8 + 2 * t] = scale * gp.x;
-                v[c * 8 + 2 * t + 1] = scale * gp.y;
-            }
-        } else {
-            const uint2 w = *reinterpret_cast<const uint2*>(crow + e0);               // 8 codes = 8 elements
+                for (int pl = 0; pl < 3; ++pl) {
+                    const uint2 q = __ldg(reinterpret_cast<const uint2*>(packed + (blk >> 1) * 768 + pl * 256 + L * 8));
+                    w[jj * 3 + pl] = q.x;
+                    w[jj * 3 + 3 + pl] = q.y;
+                }
+            } else if (NIB) {
+                const uint2 q = __ldg(reinterpret_cast<const uint2*>(packed + blk * 256 + L * 8));
+                w[jj * 2] = q.x; w[jj * 2 + 1] = q.y;
+            } else {
 #pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                const uint32_t code = ((t < 4 ? w.x : w.y) >> (8 * (t & 3))) & 0xffu;
-                v[c * 8 + t] = scale * __ldg(grid + code);
+                for (int h = 0; h < (B8 ? 2 : 1); ++h) {
+                    const uint4 q = __ldg(reinterpret_cast<const uint4*>(packed + blk * (B8 ? 1024 : 512) + h * 512 + L * 16));
+                    uint32_t* o = w + jj * (B8 ? 8 : 4) + h * 4;
+                    o[0] = q.x; o[1] = q.y; o[2] = q.z; o[3] = q.w;
+                }
             }
         }
     }
-    fwht1024_warp(v, lane);
-#pragma unroll
-    for (int r = 0; r < 32; ++r) v[r] *= 0.03125f;          // H / sqrt(1024)
-    apply_signs1024(v, xi, gi * kGroup, lane);
+    // table row of element j (jj = j >> 3, m = (j & 7) >> 1, ah = j & 1) for row half rh; see the slot layout in quantize.cu
+    __device__ __forceinline__ uint32_t index(int j, int rh, int lane) const {
+        const int jj = j >> 3, m = (j & 7) >> 1, ah = j & 1, a = rh + 2 * ah;
+        if (SIX) {
+            const uint32_t lo = (w[jj * 3 + (m >> 1)] >> (8 * a + 4 * (m & 1))) & 15u;
+            return lo | (((w[jj * 3 + 2] >> (8 * a + 2 * m)) & 3u) << 4);
+        }
+        if (NIB) return (w[jj * 2 + ((j & 7) >> 2)] >> (8 * (j & 3) + 4 * rh)) & 15u;
+        if (B8) return (w[jj * 8 + (j & 7)] >> (16 * rh + 8 * (lane & 1))) & 255u;
+        return (w[jj * 4 + m] >> (8 * a)) & 255u;
+    }
+};
+
+// Lookup table in shared memory: row idx holds, 16 times over, the two coordinates an index stands for (one p = 2 code
+// or two p = 1 codes; 8-bit scalar codes: the value, twice), so that lane l reads word l of its row - the coordinate of
+// its parity - and the 32 lookups of a warp never meet in a bank.
+template <int FMT>
+__device__ __forceinline__ void fill_pair_table(float* table, const float* __restrict__ grid, int p, int n, int bits) {
+    constexpr int ROWS = FMT == 1 ? 64 : FMT == 2 ? 16 : 256;
+    for (int i = threadIdx.x; i < ROWS * 32; i += blockDim.x) {
+        const int idx = i >> 5, k = i & 1;
+        table[i] = FMT == 3 ? grid[idx] : p == 2 ? grid[2 * idx + k] : grid[(idx >> (k * bits)) & (n - 1)];
+    }
 }
 
-// One warp per (row, group of 1024).
-template <int P, typename OutT>
-__global__ void __launch_bounds__(256) dequantize_kernel(const uint8_t* __restrict__ canonical, const __half* __restrict__ scales,
-                                                         const float* __restrict__ grid, OutT* __restrict__ W_out,
-                                                         int64_t N, int64_t K, uint64_t xi) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int64_t groups = K / kGroup;
-    if (warp >= N * groups) return;
-    const int64_t row = warp / groups, gi = warp % groups;
-    float v[32];
-    dequantize_group<P>(canonical, scales, grid, K, xi, row, gi, lane, v);
-    OutT* dst = W_out + row * K + gi * kGroup;
+// Sign bits of this lane's 32 elements c*256 + l*8 + e of the group at input k0: byte c of the result.
+__device__ __forceinline__ uint32_t lane_sign_bits(uint64_t xi, int64_t k0, int lane) {
+    const uint64_t word = sign_word(xi, ((uint64_t)k0 >> 6) + (uint64_t)(lane & 15));
+    const uint32_t lo = (uint32_t)word, hi = (uint32_t)(word >> 32);
+    uint32_t bits = 0u;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-        if (sizeof(OutT) == 4) {
-            float* d = reinterpret_cast<float*>(dst) + c * 256 + lane * 8;
-            *reinterpret_cast<float4*>(d) = make_float4(v[c * 8], v[c * 8 + 1], v[c * 8 + 2], v[c * 8 + 3]);
-            *reinterpret_cast<float4*>(d + 4) = make_float4(v[c * 8 + 4], v[c * 8 + 5], v[c * 8 + 6], v[c * 8 + 7]);
-        } else {
-            uint32_t w4[4];
+        const int src = 4 * c + (lane >> 3);
+        const uint32_t from_lo = __shfl_sync(0xffffffffu, lo, src), from_hi = __shfl_sync(0xffffffffu, hi, src);
+        bits |= ((((lane & 4) ? from_hi : from_lo) >> ((lane & 3) * 8)) & 0xffu) << (8 * c);
+    }
+    return bits;
+}
+__device__ __forceinline__ float with_sign(float v, uint32_t bits, int r) {
+    return __uint_as_float(__float_as_uint(v) ^ ((bits << (31 - r)) & 0x80000000u));
+}
+
+template <typename T>
+struct RawRow;
+template <>
+struct RawRow<__nv_bfloat16> {
+    uint4 q[4];
+    __device__ __forceinline__ void load(const __nv_bfloat16* __restrict__ src, int lane) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) q[c] = __ldg(reinterpret_cast<const uint4*>(src + c * 256 + lane * 8));
+    }
+    __device__ __forceinline__ void get(float (&v)[32]) const {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const uint32_t w[4] = {q[c].x, q[c].y, q[c].z, q[c].w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                __nv_bfloat162 h = __floats2bfloat162_rn(v[c * 8 + 2 * e], v[c * 8 + 2 * e + 1]);
-                w4[e] = *reinterpret_cast<uint32_t*>(&h);
+                v[c * 8 + 2 * e] = __uint_as_float(w[e] << 16);
+                v[c * 8 + 2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
             }
-            *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(dst) + c * 256 + lane * 8) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+        }
+    }
+};
+template <>
+struct RawRow<float> {
+    float4 q[8];
+    __device__ __forceinline__ void load(const float* __restrict__ src, int lane) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) q[c] = __ldg(reinterpret_cast<const float4*>(src + (c >> 1) * 256 + lane * 8 + (c & 1) * 4));
+    }
+    __device__ __forceinline__ void get(float (&v)[32]) const {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) { v[4 * c] = q[c].x; v[4 * c + 1] = q[c].y; v[4 * c + 2] = q[c].z; v[4 * c + 3] = q[c].w; }
+    }
+};
+
+template <typename OutT>
+__device__ __forceinline__ void store_row(OutT* __restrict__ dst, int lane, const float (&v)[32]);
+template <>
+__device__ __forceinline__ void store_row<float>(float* __restrict__ dst, int lane, const float (&v)[32]) {
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+        *reinterpret_cast<float4*>(dst + (c >> 1) * 256 + lane * 8 + (c & 1) * 4) = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+}
+template <>
+__device__ __forceinline__ void store_row<__nv_bfloat16>(__nv_bfloat16* __restrict__ dst, int lane, const float (&v)[32]) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        uint32_t w4[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const __nv_bfloat162 h = __floats2bfloat162_rn(v[c * 8 + 2 * e], v[c * 8 + 2 * e + 1]);
+            w4[e] = *reinterpret_cast<const uint32_t*>(&h);
+        }
+        *reinterpret_cast<uint4*>(dst + c * 256 + lane * 8) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+    }
+}
+
+// ERROR = false: W_out[row][k] = the dequantised matrix.  ERROR = true: the two sums of t^2 = ||W^ - W||^2 / ||W||^2,
+// taken in the rotated space (the transform is orthonormal): W is rotated as the encoder rotates it and compared with
+// scale * G[code].  A block writes its pair of partial sums; launch_layer_error's second kernel adds them in block order.
+// Bound: instruction issue (75-79 % of the slots; 810 instructions per row and group, 360 of them the transform), next to 2 or 4 + b/8
+// bytes per weight from HBM.  14336 x 4096 bf16 at 4 bits: error 185 + 47 us (canonical codes unpacked to memory byte by
+// byte, then one warp per row and group adding to two global doubles) -> 59 us; the 147 MB it reads take 22 us.
+template <int FMT, typename T, bool ERROR>
+__global__ void __launch_bounds__(kDqWarps * 32, 2) packed_rows_kernel(const uint8_t* __restrict__ packed, const __half* __restrict__ scales,
+                                                                       const float* __restrict__ grid, int p, int n, int bits,
+                                                                       const T* __restrict__ W, T* __restrict__ W_out, int64_t N,
+                                                                       int64_t K, uint64_t xi, double* __restrict__ partials) {
+    extern __shared__ __align__(16) float dq_smem[];
+    constexpr int ROWS = FMT == 1 ? 64 : FMT == 2 ? 16 : 256;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float* ex = dq_smem + ROWS * 32 + warp * kFwhtExchange;
+    fill_pair_table<FMT>(dq_smem, grid, p, n, bits);
+    __syncthreads();
+    const float* table_lane = dq_smem + lane;
+    const int64_t groups = K / kGroup, kblocks = K / kBlockK, turns = (N / kRowTile) * groups;
+    int64_t rt = (int64_t)blockIdx.x / groups, gi = (int64_t)blockIdx.x % groups;
+    const int64_t step_tiles = (int64_t)gridDim.x / groups, step_groups = (int64_t)gridDim.x % groups;
+    double num = 0.0, den = 0.0;
+    for (int64_t turn = blockIdx.x; turn < turns; turn += gridDim.x, rt += step_tiles, gi += step_groups) {
+        if (gi >= groups) { gi -= groups; ++rt; }
+        ColumnCodes<FMT> codes;
+        codes.load(packed, rt * kblocks + gi * 16, warp, lane);
+        const __half* sc = scales + (rt * groups + gi) * kRowTile + warp;
+        const float scale[2] = {__half2float(sc[0]), __half2float(sc[8])};
+        const uint32_t sign = lane_sign_bits(xi, gi * kGroup, lane);
+        RawRow<T> raw[2];
+        if (ERROR) {
+#pragma unroll
+            for (int rh = 0; rh < 2; ++rh) raw[rh].load(W + (rt * 16 + warp + 8 * rh) * K + gi * kGroup, lane);
+        }
+#pragma unroll
+        for (int rh = 0; rh < 2; ++rh) {
+            float v[32];
+            if (ERROR) {
+                raw[rh].get(v);
+                float dsum = 0.f, nsum = 0.f;
+#pragma unroll
+                for (int r = 0; r < 32; ++r) {
+                    dsum = fmaf(v[r], v[r], dsum);
+                    v[r] = with_sign(v[r], sign, r);
+                }
+                fwht1024_to_columns(v, ex, lane);
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    const float d = fmaf(scale[rh], table_lane[codes.index(j, rh, lane) * 32], -0.03125f * v[j]);
+                    nsum = fmaf(d, d, nsum);
+                }
+#pragma unroll
+                for (int m = 16; m > 0; m >>= 1) {
+                    nsum += __shfl_xor_sync(0xffffffffu, nsum, m);
+                    dsum += __shfl_xor_sync(0xffffffffu, dsum, m);
+                }
+                num += (double)nsum;
+                den += (double)dsum;
+            } else {
+                const float s = scale[rh] * 0.03125f;          // H / sqrt(1024)
+#pragma unroll
+                for (int j = 0; j < 32; ++j) v[j] = s * table_lane[codes.index(j, rh, lane) * 32];
+                fwht1024_from_columns(v, ex, lane);
+#pragma unroll
+                for (int r = 0; r < 32; ++r) v[r] = with_sign(v[r], sign, r);
+                store_row<T>(W_out + (rt * 16 + warp + 8 * rh) * K + gi * kGroup, lane, v);
+            }
+        }
+    }
+    if (ERROR) {
+        __syncthreads();                                       // (the table and exchange buffers are free: reuse them)
+        double* red = reinterpret_cast<double*>(dq_smem);
+        if (lane == 0) { red[2 * warp] = num; red[2 * warp + 1] = den; }
+        __syncthreads();
+        if (threadIdx.x < 2) {
+            double s = 0.0;
+            for (int w = 0; w < kDqWarps; ++w) s += red[2 * w + threadIdx.x];
+            partials[2 * blockIdx.x + threadIdx.x] = s;
         }
     }
 }
 
-// The "database" entry of the dynamic bit-width problem (Section 5, "Measuring Grid Parameters"): the layer's relative
-// quantisation error t^2 = ||W^ - W||_F^2 / ||W||_F^2, accumulated as the two sums without materialising W^.
-template <int P, typename T>
-__global__ void __launch_bounds__(256) layer_error_kernel(const uint8_t* __restrict__ canonical, const __half* __restrict__ scales,
-                                                          const float* __restrict__ grid, const T* __restrict__ W,
-                                                          int64_t N, int64_t K, uint64_t xi, double* __restrict__ sums) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int64_t groups = K / kGroup;
-    if (warp >= N * groups) return;
-    const int64_t row = warp / groups, gi = warp % groups;
-    float v[32];
-    dequantize_group<P>(canonical, scales, grid, K, xi, row, gi, lane, v);
-    const T* src = W + row * K + gi * kGroup;
-    float num = 0.f, den = 0.f;
+__global__ void __launch_bounds__(64) error_total_kernel(const double* __restrict__ partials, int blocks, double* __restrict__ sums) {
+    __shared__ double total[2];
+    const int which = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double s = 0.0;
+    for (int i = lane; i < blocks; i += 32) s += partials[2 * i + which];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const float w = (float)src[c * 256 + lane * 8 + e];
-            const float dlt = v[c * 8 + e] - w;
-            num = fmaf(dlt, dlt, num);
-            den = fmaf(w, w, den);
-        }
-    }
-#pragma unroll
-    for (int m = 16; m > 0; m >>= 1) {
-        num += __shfl_xor_sync(0xffffffffu, num, m);
-        den += __shfl_xor_sync(0xffffffffu, den, m);
-    }
-    if (lane == 0) {
-        atomicAdd(sums, (double)num);
-        atomicAdd(sums + 1, (double)den);
+    for (int m = 16; m > 0; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
+    if (lane == 0) { total[which] = s; sums[which] = s; }
+    __syncthreads();
+    if (threadIdx.x == 0) sums[2] = total[1] > 0.0 ? total[0] / total[1] : 0.0;
+}
+
+int sm_count() {
+    static int cached[64] = {0};
+    return device_once(cached, [] {
+        int dev = 0, v = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
+            v = 148;
+        return v;
+    });
+}
+
+template <int FMT, typename T, bool ERROR>
+int launch_rows(const higgs_desc& d, const void* packed, const void* scales, const float* grid, const void* W, void* W_out,
+                double* partials, int* blocks_out, cudaStream_t st) {
+    constexpr int ROWS = FMT == 1 ? 64 : FMT == 2 ? 16 : 256;
+    constexpr int smem = (ROWS * 32 + kDqWarps * kFwhtExchange) * (int)sizeof(float);
+    static int per_sm[64] = {0};
+    const int resident = device_once(per_sm, [] {
+        int b = 0;
+        if (cudaFuncSetAttribute(packed_rows_kernel<FMT, T, ERROR>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, packed_rows_kernel<FMT, T, ERROR>, kDqWarps * 32, smem) != cudaSuccess || b < 1)
+            return -1;
+        return b;
+    });
+    if (resident < 1) return HIGGS_ERR_CUDA;
+    const int64_t turns = (d.N / kRowTile) * (d.K / kGroup);
+    int64_t blocks = (int64_t)resident * sm_count();
+    if (ERROR && blocks > kErrorPartials) blocks = kErrorPartials;
+    if (blocks > turns) blocks = turns;
+    if (blocks_out) *blocks_out = (int)blocks;
+    packed_rows_kernel<FMT, T, ERROR><<<(unsigned)blocks, kDqWarps * 32, smem, st>>>(
+        static_cast<const uint8_t*>(packed), static_cast<const __half*>(scales), grid, d.p, d.n, code_bits(d.n), static_cast<const T*>(W),
+        static_cast<T*>(W_out), d.N, d.K, d.rht_seed, partials);
+    return cuda_status(cudaGetLastError());
+}
+
+template <typename T, bool ERROR>
+int launch_format(const higgs_desc& d, const void* packed, const void* scales, const float* grid, const void* W, void* W_out,
+                  double* partials, int* blocks, cudaStream_t st) {
+    switch (format_of(d.p, d.n)) {
+        case Format::kByteLut: return launch_rows<0, T, ERROR>(d, packed, scales, grid, W, W_out, partials, blocks, st);
+        case Format::kSixBit: return launch_rows<1, T, ERROR>(d, packed, scales, grid, W, W_out, partials, blocks, st);
+        case Format::kNibble: return launch_rows<2, T, ERROR>(d, packed, scales, grid, W, W_out, partials, blocks, st);
+        case Format::kByte8: return launch_rows<3, T, ERROR>(d, packed, scales, grid, W, W_out, partials, blocks, st);
+        default: return HIGGS_ERR_UNSUPPORTED;
     }
 }
 
 }  // namespace
 
-int launch_layer_error(const higgs_desc& d, const uint8_t* canonical, const void* scales, const float* grid, const void* W,
-                       int w_dtype, double* sums, cudaStream_t st) {
-    if (cudaMemsetAsync(sums, 0, 2 * sizeof(double), st) != cudaSuccess) return HIGGS_ERR_CUDA;
-    const int64_t warps = d.N * (d.K / kGroup);
-    if (warps == 0) return HIGGS_OK;
-    const unsigned blocks = (unsigned)((warps + 7) / 8);
-    const __half* sc = static_cast<const __half*>(scales);
-    if (d.p == 2 && w_dtype == HIGGS_F32)
-        layer_error_kernel<2, float><<<blocks, 256, 0, st>>>(canonical, sc, grid, static_cast<const float*>(W), d.N, d.K, d.rht_seed, sums);
-    else if (d.p == 2 && w_dtype == HIGGS_BF16)
-        layer_error_kernel<2, __nv_bfloat16><<<blocks, 256, 0, st>>>(canonical, sc, grid, static_cast<const __nv_bfloat16*>(W), d.N, d.K, d.rht_seed, sums);
-    else if (d.p == 1 && w_dtype == HIGGS_F32)
-        layer_error_kernel<1, float><<<blocks, 256, 0, st>>>(canonical, sc, grid, static_cast<const float*>(W), d.N, d.K, d.rht_seed, sums);
-    else if (d.p == 1 && w_dtype == HIGGS_BF16)
-        layer_error_kernel<1, __nv_bfloat16><<<blocks, 256, 0, st>>>(canonical, sc, grid, static_cast<const __nv_bfloat16*>(W), d.N, d.K, d.rht_seed, sums);
-    else
-        return HIGGS_ERR_UNSUPPORTED;
+int launch_layer_error(const higgs_desc& d, const void* packed, const void* scales, const float* grid, const void* W,
+                       int w_dtype, double* sums, double* partials, cudaStream_t st) {
+    int blocks = 0;
+    const int rc = w_dtype == HIGGS_F32 ? launch_format<float, true>(d, packed, scales, grid, W, nullptr, partials, &blocks, st)
+                                        : launch_format<__nv_bfloat16, true>(d, packed, scales, grid, W, nullptr, partials, &blocks, st);
+    if (rc != HIGGS_OK) return rc;
+    error_total_kernel<<<1, 64, 0, st>>>(partials, blocks, sums);
     return cuda_status(cudaGetLastError());
 }
 
-int launch_dequantize(const higgs_desc& d, const uint8_t* canonical, const void* scales, const float* grid, void* W_out,
+int launch_dequantize(const higgs_desc& d, const void* packed, const void* scales, const float* grid, void* W_out,
                       int w_dtype, cudaStream_t st) {
-    const int64_t warps = d.N * (d.K / kGroup);
-    if (warps == 0) return HIGGS_OK;
-    const unsigned blocks = (unsigned)((warps + 7) / 8);
-    const __half* sc = static_cast<const __half*>(scales);
-    if (d.p == 2 && w_dtype == HIGGS_F32)
-        dequantize_kernel<2, float><<<blocks, 256, 0, st>>>(canonical, sc, grid, static_cast<float*>(W_out), d.N, d.K, d.rht_seed);
-    else if (d.p == 2 && w_dtype == HIGGS_BF16)
-        dequantize_kernel<2, __nv_bfloat16><<<blocks, 256, 0, st>>>(canonical, sc, grid, static_cast<__nv_bfloat16*>(W_out), d.N, d.K, d.rht_seed);
-    else if (d.p == 1 && w_dtype == HIGGS_F32)
-        dequantize_kernel<1, float><<<blocks, 256, 0, st>>>(canonical, sc, grid, static_cast<float*>(W_out), d.N, d.K, d.rht_seed);
-    else if (d.p == 1 && w_dtype == HIGGS_BF16)
-        dequantize_kernel<1, __nv_bfloat16><<<blocks, 256, 0, st>>>(canonical, sc, grid, static_cast<__nv_bfloat16*>(W_out), d.N, d.K, d.rht_seed);
-    else
-        return HIGGS_ERR_UNSUPPORTED;
-    return cuda_status(cudaGetLastError());
+    return w_dtype == HIGGS_F32 ? launch_format<float, false>(d, packed, scales, grid, nullptr, W_out, nullptr, nullptr, st)
+                                : launch_format<__nv_bfloat16, false>(d, packed, scales, grid, nullptr, W_out, nullptr, nullptr, st);
 }
 
 }  // namespace higgs
