@@ -150,8 +150,11 @@ int higgs_make_uniform_grid(int n, float* grid_out, float* step_out, float* mse_
  *                the samples
  *   iters_out    device, optional: iterations run (int32), negative if
  *                max_iters was reached without convergence
- * Distances are fp32, sums fp64; the result is a fixed point of the same
- * iteration the fp64 definition runs but need not be bit-identical to it.
+ * Distances are fp32, sums 64-bit fixed point with a resolution of 2^-62
+ * times num_samples times the largest |coordinate| (exact for N(0, 1) samples
+ * but the tiniest), independent of the order of summation; the result is a fixed
+ * point of the same iteration the fp64 definition runs but need not be
+ * bit-identical to it.
  * 1 <= p <= 4 and 1 <= n <= 4096 (n need not be a power of two), else
  * HIGGS_ERR_UNSUPPORTED.
  */

@@ -1,19 +1,33 @@
 // Grid fit of Algorithm 2 ("CLVQ(n, p), computed once"), run as Lloyd's batch
 // iteration on caller-provided samples of N(0, I_p): the assignment step is the
-// encoder's exhaustive nearest-point search, the update a segmented mean.
+// encoder's exhaustive nearest-point rule, the update a segmented mean.
 #include "common.cuh"
 
 namespace higgs {
 
 namespace {
 
+constexpr int kFitThreads = 1024;
+constexpr int kMaxFitBlocks = 1024;
+constexpr int kNear = 32;              // centres in a cell's neighbour list
+constexpr int kNearRow = 40;           // ... which is 80 bytes in shared memory: the lists of a warp's cells spread over the banks
+constexpr int kLaneScans = 160;        // more listed scans than this in a batch: one per lane instead of one per warp
+constexpr int kMinNearCentres = 65;    // grids with lists: below, a scan is no longer than a list or two ...
+constexpr int kMaxNearCentres = 512;   // ... above, building the lists costs as much as the scans they save
+constexpr int kMaxSharedSums = 1024;   // coordinates whose changes a block collects in shared memory first
+constexpr int kQueueRounds = 4;        // samples a lane tests before the block scans those that need it
+
 struct GridWs {
     float* centres;               // [n][p]
-    double* sums;                 // [n][p]
-    unsigned long long* counts;   // [n]
+    long long* delta;             // [3][n][p] changes of the cells' sums, fixed point
+    int32_t* delta_cnt;           // [3][n]    changes of the cells' sizes
+    double* err;                  // [kMaxFitBlocks] squared error of a block's samples
+    unsigned long long* bar;      // [2] grid barrier: arrivals (low half), blocks with a changed assignment (high half)
+    int32_t* flags;               // [0] done, [1] iterations, [2] bits of the largest |sample|
+    uint16_t* near_idx;           // [kMaxNearCentres][kNear] neighbour lists
+    float* excl;                  // [kMaxNearCentres]
     int32_t* assign;              // [m]
-    double* err;                  // [2]: running, last completed
-    int32_t* flags;               // [0] changed, [1] done, [2] iterations, [3] grid-barrier arrivals (persistent fit)
+    float* lower;                 // [m]
 };
 
 __host__ __device__ inline size_t up256(size_t v) { return (v + 255) / 256 * 256; }
@@ -22,165 +36,450 @@ GridWs carve(void* ws, int p, int n, int64_t m) {
     uint8_t* b = static_cast<uint8_t*>(ws);
     GridWs w;
     w.centres = reinterpret_cast<float*>(b); b += up256(sizeof(float) * n * p);
-    w.sums = reinterpret_cast<double*>(b); b += up256(sizeof(double) * n * p);
-    w.counts = reinterpret_cast<unsigned long long*>(b); b += up256(sizeof(unsigned long long) * n);
-    w.err = reinterpret_cast<double*>(b); b += 256;
-    w.flags = reinterpret_cast<int32_t*>(b); b += 256;
-    w.assign = reinterpret_cast<int32_t*>(b);
-    (void)m;
+    w.delta = reinterpret_cast<long long*>(b); b += up256(sizeof(long long) * 3 * n * p);
+    w.delta_cnt = reinterpret_cast<int32_t*>(b); b += up256(sizeof(int32_t) * 3 * n);
+    w.err = reinterpret_cast<double*>(b); b += up256(sizeof(double) * kMaxFitBlocks);
+    w.bar = reinterpret_cast<unsigned long long*>(b);
+    w.flags = reinterpret_cast<int32_t*>(b + 16); b += 256;
+    w.near_idx = reinterpret_cast<uint16_t*>(b); b += sizeof(uint16_t) * kMaxNearCentres * kNear;
+    w.excl = reinterpret_cast<float*>(b); b += sizeof(float) * kMaxNearCentres;
+    w.assign = reinterpret_cast<int32_t*>(b); b += up256(sizeof(int32_t) * (size_t)m);
+    w.lower = reinterpret_cast<float*>(b);
     return w;
 }
 
-__global__ void grid_init_kernel(GridWs w, const float* __restrict__ samples, int p, int n, int64_t m) {
+__global__ void grid_init_kernel(GridWs w, int p, int n, int64_t m) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < m) w.assign[i] = -1;
-    if (i < (int64_t)n * p) { w.centres[i] = samples[i]; w.sums[i] = 0.0; }
-    if (i < n) w.counts[i] = 0ull;
-    if (i < 2) w.err[i] = 0.0;
-    if (i < 8) w.flags[i] = 0;
+    if (i < (int64_t)3 * n * p) w.delta[i] = 0;
+    if (i < 3 * n) w.delta_cnt[i] = 0;
+    if (i < 2) w.bar[i] = 0;
+    if (i < 4) w.flags[i] = 0;
 }
 
-// Assignment step.  The centres sit in dynamic shared memory ([n][P] floats, at most 64 KB).  SMALL (n <= 256): the
-// per-cell sums are first collected in shared memory and then added to the global ones; otherwise every sample adds
-// to the global sums directly (with thousands of cells the atomics rarely collide).  Distances are the plain
-// sum of (x_k - c_k)^2 in coordinate order, fp32, strict '<' (lowest index wins a tie) - the encoder's rule.
-template <int P, bool SMALL>
-__device__ __forceinline__ void assign_body(const GridWs& w, const float* __restrict__ samples, int n, int64_t m,
-                                            unsigned char* grid_smem) {
-    float* sc = reinterpret_cast<float*>(grid_smem);
-    double* ssum = reinterpret_cast<double*>(grid_smem + up256(sizeof(float) * n * P));
-    unsigned int* scnt = reinterpret_cast<unsigned int*>(ssum + (SMALL ? n * P : 0));
-    __shared__ double serr;
-    __shared__ int schanged;
-    for (int i = threadIdx.x; i < n * P; i += blockDim.x) {
-        sc[i] = __ldcg(&w.centres[i]);       // (bypasses L1: in the persistent fit another block rewrote the centres)
-        if (SMALL) ssum[i] = 0.0;
-    }
-    if (SMALL)
-        for (int i = threadIdx.x; i < n; i += blockDim.x) scnt[i] = 0u;
-    if (threadIdx.x == 0) { serr = 0.0; schanged = 0; }
-    __syncthreads();
-    double err = 0.0;
-    int changed = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-        float x[P];
-#pragma unroll
-        for (int k = 0; k < P; ++k) x[k] = samples[i * P + k];
-        float best = INFINITY;
-        int bi = 0;
-        for (int c = 0; c < n; ++c) {
-            float d = 0.f;
-#pragma unroll
-            for (int k = 0; k < P; ++k) {
-                const float e = x[k] - sc[c * P + k];
-                d = k == 0 ? e * e : fmaf(e, e, d);
-            }
-            if (d < best) { best = d; bi = c; }
-        }
-        if (w.assign[i] != bi) { w.assign[i] = bi; ++changed; }
-        err += (double)best;
-        if (SMALL) {
-#pragma unroll
-            for (int k = 0; k < P; ++k) atomicAdd(&ssum[bi * P + k], (double)x[k]);
-            atomicAdd(&scnt[bi], 1u);
-        } else {
-#pragma unroll
-            for (int k = 0; k < P; ++k) atomicAdd(&w.sums[bi * P + k], (double)x[k]);
-            atomicAdd(&w.counts[bi], 1ull);
-        }
-    }
-    atomicAdd(&serr, err);
-    if (changed) atomicAdd(&schanged, changed);
-    __syncthreads();
-    if (SMALL) {
-        for (int i = threadIdx.x; i < n * P; i += blockDim.x)
-            if (ssum[i] != 0.0) atomicAdd(&w.sums[i], ssum[i]);
-        for (int i = threadIdx.x; i < n; i += blockDim.x)
-            if (scnt[i]) atomicAdd(&w.counts[i], (unsigned long long)scnt[i]);
-    }
-    if (threadIdx.x == 0) {
-        atomicAdd(&w.err[0], serr);
-        if (schanged) atomicAdd(&w.flags[0], schanged);
-    }
-}
-
-template <int P, bool SMALL>
-__global__ void __launch_bounds__(256) grid_assign_kernel(GridWs w, const float* __restrict__ samples, int n, int64_t m) {
-    extern __shared__ __align__(16) unsigned char grid_smem[];
-    if (w.flags[1]) return;
-    assign_body<P, SMALL>(w, samples, n, m, grid_smem);
-}
-
-__device__ __forceinline__ void update_body(const GridWs& w, int p, int n) {
-    const int changed = __ldcg(&w.flags[0]);
-    __syncthreads();
-    for (int i = threadIdx.x; i < n * p; i += blockDim.x) {
-        const unsigned long long cnt = __ldcg(&w.counts[i / p]);
-        if (changed && cnt) w.centres[i] = (float)(__ldcg(&w.sums[i]) / (double)cnt);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < n * p; i += blockDim.x) w.sums[i] = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) w.counts[i] = 0ull;
-    if (threadIdx.x == 0) {
-        w.err[1] = __ldcg(&w.err[0]);
-        w.err[0] = 0.0;
-        w.flags[2] = __ldcg(&w.flags[2]) + 1;
-        w.flags[0] = 0;
-        if (!changed) w.flags[1] = 1;
-    }
-}
-
-__global__ void grid_update_kernel(GridWs w, int p, int n) {
-    if (w.flags[1]) return;
-    update_body(w, p, n);
-}
-
-// ---- the whole iteration in ONE cooperatively launched kernel ---------------------------------------------------
-// Every block is resident (the launch fails otherwise), so the blocks can meet at a barrier between the assignment and
-// the update step: a counter in the workspace that every block's first thread increments and then polls, with a limit
-// on the polls - a barrier that runs out raises the grid-fit status word and every block leaves.
+// Every block is resident (a cooperative launch, or one block), so the blocks can meet at a barrier: a counter in the
+// workspace that every block's first thread adds to and then polls, with a limit on the polls - a barrier that runs out
+// raises the grid-fit status word and every block leaves.  The same addition counts the blocks that report `changed`.
+// Two counters take turns (barrier number `no` uses no % 2), so a block that reads late cannot see the next barrier's.
 __device__ int g_grid_status = 0;
 constexpr unsigned kGridBarrierLimit = 1u << 22;
 
-__device__ __forceinline__ bool grid_barrier(int32_t* counter, int target) {
+// returns whether any block reported a change in this barrier; *ok = false if it ran out
+__device__ __forceinline__ bool grid_barrier(unsigned long long* bar, int no, int blocks, bool changed, unsigned& seen, bool* ok) {
+    __shared__ unsigned s_high;
+    __shared__ int s_ok;
     __syncthreads();
-    int ok = 1;
     if (threadIdx.x == 0) {
+        unsigned long long* counter = bar + (no & 1);
+        const unsigned target = (unsigned)(no / 2 + 1) * (unsigned)blocks;
         __threadfence();
-        atomicAdd(counter, 1);
+        atomicAdd(counter, 1ull | (changed ? 1ull << 32 : 0ull));
         unsigned it = 0;
+        unsigned long long v;
         for (;;) {
-            int v;
-            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
-            if (v >= target) break;
-            if (++it > kGridBarrierLimit) { ok = 0; atomicExch(&g_grid_status, (int)HIGGS_ERR_TIMEOUT); break; }
-            __nanosleep(64);
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(counter) : "memory");
+            if ((unsigned)v >= target || ++it > kGridBarrierLimit) break;
         }
         __threadfence();
+        s_high = (unsigned)(v >> 32);
+        s_ok = (unsigned)v >= target;
+        if ((unsigned)v < target) atomicExch(&g_grid_status, (int)HIGGS_ERR_TIMEOUT);
     }
-    return __syncthreads_and(ok) != 0;
+    __syncthreads();
+    *ok = s_ok != 0;
+    const bool any = s_high != seen;
+    seen = s_high;
+    return any;
 }
 
-template <int P, bool SMALL>
-__global__ void __launch_bounds__(256) grid_fit_kernel(GridWs w, const float* __restrict__ samples, int n, int64_t m, int max_iters) {
+// fp32 squared distance, plain sum of (x_k - c_k)^2 in coordinate order: the encoder's rule
+template <int P>
+__device__ __forceinline__ float centre_distance(const float (&x)[P], const float* c) {
+    float d = 0.f;
+#pragma unroll
+    for (int k = 0; k < P; ++k) {
+        const float e = x[k] - c[k];
+        d = k == 0 ? e * e : fmaf(e, e, d);
+    }
+    return d;
+}
+
+__host__ __device__ inline bool fit_lists(int n) { return n >= kMinNearCentres && n <= kMaxNearCentres; }
+inline size_t fit_smem(int p, int n) {
+    return (size_t)n * p * (sizeof(long long) + sizeof(float)) + (size_t)n * sizeof(int) +
+           (n * p <= kMaxSharedSums ? (size_t)n * p * 8 + (size_t)n * 4 : 0) + (fit_lists(n) ? (size_t)n * (kNearRow * 2 + 20) + 16 : 0);
+}
+
+// The whole iteration in ONE cooperatively launched kernel, one barrier per iteration.
+//   * Assignment.  A sample keeps its cell without a scan while a lower bound on its distance to every OTHER centre
+//     exceeds its distance to its own (Hamerly, "Making k-means even faster", 2010).  The bound is the second-best
+//     distance at the last scan minus what the centres have moved since; the movements add up in a running total M, and
+//     a bound is stored once, as bound + M.  Bounds are rounded down, distances up, by more than fp32 rounding of the
+//     squared distances (a few 2^-24 relative), so a skipped scan could not have ended differently - same centre, lowest
+//     index on ties.  The largest movement is that of a few outer centres with few samples, so for grids of 65 to 512
+//     points every cell a has a list of the up to 32 centres nearest to its own, and M counts only their movements: a
+//     centre outside the list is at least D_a from centre a, so it is no rival while the sample is nearer than D_a / 2
+//     to a, with D_a reduced by twice the movement of any centre since the lists were built.  A scan then covers the
+//     list.  When that movement exceeds 0.15 of the smallest D_a the lists are built anew.
+//     The samples that need a scan go through a queue of the block, so that its warps share them evenly, a warp scanning
+//     one at a time; many scans are done one per lane.
+//   * Update.  Only samples that changed cell touch the sums.  The sums are 64-bit fixed point, scaled so that m times the
+//     largest |coordinate| stays below 2^62: for N(0, I) samples all but the tiniest coordinates are represented
+//     exactly, and integer sums do not depend on the order of the atomics.  Every block adds the iteration's changes to
+//     its own copy of the sums and computes the new centres itself, so no second barrier is needed.  Three buffers take
+//     turns: the changes of iteration i are read after its barrier; block 0 clears those of i - 1, which every block has
+//     read before it arrived there, for iteration i + 2.
+// Bound: latency - per iteration about 2.5 us of barrier, 2 us of update, 2.5 us to test the samples and 1 to 2 us of scans.
+// p = 2, n = 256, 2^18 samples: 37 -> 9 us per iteration (before: every sample scanned all centres every time, sums by
+// fp64 atomics in shared memory, two barriers).  One barrier and movement bounds without lists: 12.4 us.
+template <int P>
+__global__ void __launch_bounds__(kFitThreads, 1) grid_fit_kernel(GridWs w, const float* __restrict__ samples, int n, int64_t m, int max_iters) {
     extern __shared__ __align__(16) unsigned char grid_smem[];
-    const int blocks = (int)gridDim.x;
-    int barrier_no = 0;
-    for (int it = 0; it < max_iters; ++it) {
-        assign_body<P, SMALL>(w, samples, n, m, grid_smem);
-        if (!grid_barrier(&w.flags[3], ++barrier_no * blocks)) return;
-        if (blockIdx.x == 0) update_body(w, P, n);
-        if (!grid_barrier(&w.flags[3], ++barrier_no * blocks)) return;
-        if (*reinterpret_cast<volatile int32_t*>(&w.flags[1])) return;       // no assignment changed: a fixed point
+    const bool shared_sums = n * P <= kMaxSharedSums, lists = fit_lists(n);
+    long long* sums = reinterpret_cast<long long*>(grid_smem);         // [n][P]
+    float* sc = reinterpret_cast<float*>(sums + (size_t)n * P);        // [n][P]
+    int* cnt = reinterpret_cast<int*>(sc + (size_t)n * P);             // [n]
+    unsigned* d_lo = reinterpret_cast<unsigned*>(cnt + n);             // [n][P] this block's changes: low and high halves, sizes
+    unsigned* d_hi = d_lo + (shared_sums ? n * P : 0);
+    int* d_cnt = reinterpret_cast<int*>(d_hi + (shared_sums ? n * P : 0));
+    float* excl = reinterpret_cast<float*>(d_cnt + (shared_sums ? n : 0));      // [n] D_a when the lists were built
+    float* near_moved = excl + n;                                      // [n] M of a cell
+    float* went = near_moved + n;                                      // [n] the centre's movement in this iteration
+    float* old_reach = went + n;                                       // [n] D_a of the lists before, now
+    float* old_moved = old_reach + n;                                  // [n] M with the lists before
+    uint16_t* near_idx = reinterpret_cast<uint16_t*>((reinterpret_cast<uintptr_t>(old_moved + n) + 15) & ~(uintptr_t)15);  // [n][kNearRow], padded with the cell itself
+    __shared__ unsigned s_move[2], s_min_excl;
+    __shared__ uint16_t s_queue[kQueueRounds * kFitThreads];            // samples to scan: place in the batch, bit 15 = by list
+    __shared__ int s_queued[2];
+    __shared__ double s_err[kFitThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, blocks = (int)gridDim.x;
+    const int64_t chunks = (m + 31) / 32, chunk0 = (int64_t)warp * blocks + blockIdx.x, chunk_step = (int64_t)blocks * (kFitThreads / 32);
+
+    for (int i = tid; i < n * P; i += kFitThreads) {
+        sc[i] = samples[i];
+        sums[i] = 0;
+        if (shared_sums) d_lo[i] = d_hi[i] = 0u;
     }
+    for (int i = tid; i < n; i += kFitThreads) {
+        cnt[i] = 0;
+        if (shared_sums) d_cnt[i] = 0;
+    }
+    if (tid < 2) s_move[tid] = 0u;
+    if (tid < 2) s_queued[tid] = 0;
+    int qi = 0;
+    // scale of the fixed-point sums
+    unsigned top = 0u;
+    for (int64_t c = chunk0; c < chunks; c += chunk_step) {
+        const int64_t i = c * 32 + lane;
+#pragma unroll
+        for (int k = 0; k < P; ++k)
+            if (i < m) top = max(top, __float_as_uint(fabsf(samples[i * P + k])));
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (lane == 0) atomicMax(reinterpret_cast<unsigned*>(&w.flags[2]), top);
+    int barrier_no = 0;
+    unsigned seen[2] = {0u, 0u};
+    bool ok;
+    grid_barrier(w.bar, barrier_no++, blocks, false, seen[0], &ok);
+    if (!ok) return;
+    top = (unsigned)__ldcg(&w.flags[2]);
+    const int shift = 62 - (m > 1 ? 64 - __clzll(m - 1) : 0) - (max((int)(top >> 23), 1) - 126);       // |sample| < 2^(exponent - 126)
+    const double scale = __hiloint2double((1023 + shift) << 20, 0), unscale = __hiloint2double((1023 - shift) << 20, 0);
+
+    // scanning one sample: n steps of its lane, or ceil(n / 32) steps and a reduction of the whole warp
+    const int scan_all = max(1, 9 * n / (9 * ((n + 31) / 32) + 45));
+    float moved = 0.f, moved_at_build = 0.f;    // sum over the iterations of the largest movement of any centre
+    bool fresh = lists;                         // the lists have to be (have just been) built
+    double err = 0.0;
+    int it = 0;
+    bool done = false;
+    for (; it < max_iters; ++it) {
+        if (fresh) {
+            // one warp per centre, the centres spread over the blocks: the largest set of at most kNear nearest centres that a
+            // threshold can cut off (bisection over the bits of the squared distance)
+            for (int a = warp * blocks + (int)blockIdx.x; a < n; a += blocks * (kFitThreads / 32)) {
+                float x[P], d[kMaxNearCentres / 32];
+#pragma unroll
+                for (int k = 0; k < P; ++k) x[k] = sc[a * P + k];
+#pragma unroll
+                for (int j = 0; j < kMaxNearCentres / 32; ++j)
+                    d[j] = 32 * j + lane < n ? centre_distance<P>(x, sc + (32 * j + lane) * P) : INFINITY;
+                unsigned lo = 0u, hi = 0x7f800000u;
+                for (int round = 0; round < 16; ++round) {
+                    const unsigned mid = (lo + hi) >> 1;
+                    int c = 0;
+#pragma unroll
+                    for (int j = 0; j < kMaxNearCentres / 32; ++j) c += __float_as_uint(d[j]) < mid ? 1 : 0;
+                    if (__reduce_add_sync(0xffffffffu, c) <= kNear) lo = mid; else hi = mid;
+                }
+                int c = 0;
+                unsigned out = 0x7f800000u;
+#pragma unroll
+                for (int j = 0; j < kMaxNearCentres / 32; ++j) {
+                    const bool in = __float_as_uint(d[j]) < lo;
+                    const unsigned mask = __ballot_sync(0xffffffffu, in);
+                    if (in) w.near_idx[a * kNear + c + __popc(mask & ((1u << lane) - 1u))] = (uint16_t)(32 * j + lane);
+                    else out = min(out, __float_as_uint(d[j]));
+                    c += __popc(mask);
+                }
+                if (lane >= c) w.near_idx[a * kNear + lane] = (uint16_t)a;
+                out = __reduce_min_sync(0xffffffffu, out);
+                if (lane == 0) w.excl[a] = __fsqrt_rd(__fmul_rd(__uint_as_float(out), 0.999996f));
+            }
+            if (tid == 0) s_min_excl = 0x7f800000u;
+            grid_barrier(w.bar, barrier_no, blocks, false, seen[barrier_no & 1], &ok);
+            ++barrier_no;
+            if (!ok) return;
+            for (int i = tid; i < n * kNear / 8; i += kFitThreads)
+                *reinterpret_cast<uint4*>(near_idx + (i >> 2) * kNearRow + (i & 3) * 8) = __ldcg(reinterpret_cast<const uint4*>(w.near_idx) + i);
+            for (int i = tid; i < n; i += kFitThreads) {
+                const float e = __ldcg(&w.excl[i]);
+                old_reach[i] = __fsub_rd(excl[i], 2.f * __fsub_ru(moved, moved_at_build));
+                old_moved[i] = near_moved[i];
+                excl[i] = e;
+                near_moved[i] = 0.f;
+                atomicMin(&s_min_excl, __float_as_uint(e));
+            }
+            moved_at_build = moved;
+            __syncthreads();
+        }
+        const float since_build = __fsub_ru(moved, moved_at_build);
+        const int buf = it % 3;
+        const bool last = it == max_iters - 1;
+        long long* delta = w.delta + (size_t)buf * n * P;
+        int32_t* delta_cnt = w.delta_cnt + (size_t)buf * n;
+        int changed = 0;
+        auto add_coord = [&](int cell, int k, long long v) {
+            if (shared_sums) {                  // (two native 32-bit atomics; a 64-bit one would be a loop)
+                const unsigned vl = (unsigned)v;
+                const unsigned carry = atomicAdd(&d_lo[cell * P + k], vl) > ~vl ? 1u : 0u;
+                atomicAdd(&d_hi[cell * P + k], (unsigned)(v >> 32) + carry);
+            } else {
+                atomicAdd(reinterpret_cast<unsigned long long*>(&delta[cell * P + k]), (unsigned long long)v);
+            }
+        };
+        // the outcome of a scan: the bound on every other centre, and the cell if it changed
+        auto settle = [&](int64_t i, const float (&x)[P], int a, int to, float second) {
+            w.lower[i] = __fadd_rd(second, lists ? near_moved[to] : moved);
+            if (to == a) return;
+            w.assign[i] = to;
+            changed = 1;
+#pragma unroll
+            for (int k = 0; k < P; ++k) {
+                const long long v = __double2ll_rn((double)x[k] * scale);
+                add_coord(to, k, v);
+                if (a >= 0) add_coord(a, k, -v);
+            }
+            int32_t* dc = shared_sums ? d_cnt : delta_cnt;
+            atomicAdd(&dc[to], 1);
+            if (a >= 0) atomicAdd(&dc[a], -1);
+        };
+        for (int64_t batch = 0; batch * chunk_step < chunks; batch += kQueueRounds) {
+            for (int r = 0; r < kQueueRounds; ++r) {
+                const int64_t c = chunk0 + (batch + r) * chunk_step;
+                if (c >= chunks) break;
+                const int64_t i = c * 32 + lane;
+                const bool valid = i < m;
+                float x[P];
+#pragma unroll
+                for (int k = 0; k < P; ++k) x[k] = valid ? samples[i * P + k] : 0.f;
+                const int a = valid ? w.assign[i] : 0;
+                const float lower = valid ? w.lower[i] : 0.f;           // (not yet written in the first iteration, and not used)
+                bool need = valid && a < 0, listed = false;
+                float best = 0.f;
+                if (valid && a >= 0) {
+                    best = centre_distance<P>(x, sc + a * P);
+                    const float u = __fsqrt_ru(__fmul_ru(best, 1.000004f));
+                    if (lists) {
+                        listed = u < 0.5f * __fsub_rd(excl[a], 2.f * since_build);
+                        float bound = __fsub_rd(lower, fresh ? old_moved[a] : near_moved[a]);
+                        // the new list may hold centres whose movements M has not counted: those were outside the old list
+                        if (fresh) bound = fminf(bound, __fsub_rd(old_reach[a], u));
+                        need = !listed || !(u < bound);
+                        if (fresh && !need) w.lower[i] = bound;         // (M of the new lists starts at 0)
+                    } else {
+                        need = !(u < __fsub_rd(lower, moved));
+                    }
+                }
+                const unsigned todo = __ballot_sync(0xffffffffu, need), by_list = __ballot_sync(0xffffffffu, need && listed);
+                if (__popc(todo & ~by_list) >= scan_all) {
+                    float b = INFINITY, s2 = INFINITY;
+                    int bi = 0;
+#pragma unroll 4
+                    for (int q = 0; q < n; ++q) {
+                        const float d = centre_distance<P>(x, sc + q * P);
+                        s2 = fminf(s2, fmaxf(b, d));
+                        if (d < b) { b = d; bi = q; }
+                    }
+                    if (need) {
+                        best = b;
+                        settle(i, x, a, bi, __fsqrt_rd(__fmul_rd(s2, 0.999996f)));
+                    }
+                    if (last && valid) err += (double)best;
+                } else {
+                    int at = 0;
+                    if (lane == 0 && todo) at = atomicAdd(&s_queued[qi], __popc(todo));
+                    at = __shfl_sync(0xffffffffu, at, 0);
+                    if (need) s_queue[at + __popc(todo & ((1u << lane) - 1u))] = (uint16_t)((r * kFitThreads + tid) | (listed ? 0x8000u : 0u));
+                    if (last && valid && !need) err += (double)best;
+                }
+            }
+            __syncthreads();
+            const int queued = s_queued[qi];
+            qi ^= 1;
+            if (tid == 0) s_queued[qi] = 0;            // (every thread has read it before this barrier)
+            auto sample_of = [&](unsigned place) {
+                return ((int64_t)((place >> 5) & 31) * blocks + blockIdx.x + (batch + place / kFitThreads) * chunk_step) * 32 + (place & 31);
+            };
+            const bool by_lane = queued > kLaneScans;
+            if (by_lane) {
+                for (int e = tid; e < queued; e += kFitThreads) {
+                    const unsigned entry = s_queue[e];
+                    if (!(entry & 0x8000u)) continue;
+                    const int64_t i = sample_of(entry & 0x7fffu);
+                    float x[P];
+#pragma unroll
+                    for (int k = 0; k < P; ++k) x[k] = samples[i * P + k];
+                    const int a = w.assign[i];
+                    const float u = __fsqrt_ru(__fmul_ru(centre_distance<P>(x, sc + a * P), 1.000004f));
+                    float b = INFINITY, s2 = INFINITY;
+                    int bi = 0;
+#pragma unroll
+                    for (int g = 0; g < kNear / 8; ++g) {
+                        const uint4 idx = *reinterpret_cast<const uint4*>(near_idx + a * kNearRow + g * 8);
+                        const unsigned v[4] = {idx.x, idx.y, idx.z, idx.w};
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            const int q = (int)((v[k >> 1] >> (16 * (k & 1))) & 0xffffu);
+                            const float d = centre_distance<P>(x, sc + q * P);
+                            if (q != bi || b == INFINITY) s2 = fminf(s2, fmaxf(b, d));      // (the padding repeats the cell itself)
+                            if (d < b || (d == b && q < bi)) { b = d; bi = q; }
+                        }
+                    }
+                    settle(i, x, a, bi, fminf(__fsqrt_rd(__fmul_rd(s2, 0.999996f)), __fsub_rd(__fsub_rd(excl[a], 2.f * since_build), u)));
+                    if (last) err += (double)b;
+                }
+            }
+            for (int e = warp; e < queued; e += kFitThreads / 32) {
+                const unsigned entry = s_queue[e];
+                const bool listed = (entry & 0x8000u) != 0;
+                if (listed && by_lane) continue;
+                const int64_t i = sample_of(entry & 0x7fffu);
+                float y[P];
+#pragma unroll
+                for (int k = 0; k < P; ++k) y[k] = samples[i * P + k];
+                const int a = w.assign[i];
+                float b = INFINITY, s2 = INFINITY, beyond = INFINITY;       // beyond: a bound on the distance to centres outside the list
+                int bi = 0x7fffffff;
+                if (listed) {
+                    bi = near_idx[a * kNearRow + lane];
+                    b = centre_distance<P>(y, sc + bi * P);
+                    beyond = __fsub_rd(__fsub_rd(excl[a], 2.f * since_build), __fsqrt_ru(__fmul_ru(centre_distance<P>(y, sc + a * P), 1.000004f)));
+                } else {
+#pragma unroll 4
+                    for (int q = lane; q < n; q += 32) {
+                        const float d = centre_distance<P>(y, sc + q * P);
+                        s2 = fminf(s2, fmaxf(b, d));
+                        if (d < b) { b = d; bi = q; }
+                    }
+                }
+                const unsigned wb = __reduce_min_sync(0xffffffffu, __float_as_uint(b));        // (not negative: ordered as integers)
+                const int to = (int)__reduce_min_sync(0xffffffffu, __float_as_uint(b) == wb ? (unsigned)bi : 0x7fffffffu);
+                const unsigned ws = __reduce_min_sync(0xffffffffu, __float_as_uint(bi == to ? s2 : b));
+                if (lane == 0) {
+                    settle(i, y, a, to, fminf(__fsqrt_rd(__fmul_rd(__uint_as_float(ws), 0.999996f)), beyond));
+                    if (last) err += (double)__uint_as_float(wb);
+                }
+            }
+            if ((batch + kQueueRounds) * chunk_step < chunks) __syncthreads();      // (the queue is written again)
+        }
+        const bool block_changed = __syncthreads_or(changed) != 0;
+        if (shared_sums && block_changed) {
+            for (int q = tid; q < n * P; q += kFitThreads) {
+                const unsigned long long v = (unsigned long long)d_lo[q] | ((unsigned long long)d_hi[q] << 32);
+                if (v) { atomicAdd(reinterpret_cast<unsigned long long*>(&delta[q]), v); d_lo[q] = d_hi[q] = 0u; }
+            }
+            for (int q = tid; q < n; q += kFitThreads)
+                if (d_cnt[q]) { atomicAdd(&delta_cnt[q], d_cnt[q]); d_cnt[q] = 0; }
+        }
+        const bool any = grid_barrier(w.bar, barrier_no, blocks, block_changed, seen[barrier_no & 1], &ok);
+        ++barrier_no;
+        if (!ok) return;
+        if (!any) { done = true; ++it; break; }          // no assignment changed: a fixed point
+        for (int q = tid; q < n; q += kFitThreads) {
+            const int size = cnt[q] + __ldcg(&delta_cnt[q]);
+            cnt[q] = size;
+            float go2 = 0.f;
+#pragma unroll
+            for (int k = 0; k < P; ++k) {
+                const long long s = sums[q * P + k] + __ldcg(&delta[q * P + k]);
+                sums[q * P + k] = s;
+                if (size > 0) {                                                 // (an empty cell keeps its centre)
+                    const float c = (float)((double)s * unscale / (double)size), go = c - sc[q * P + k];
+                    sc[q * P + k] = c;
+                    go2 = __fmaf_ru(go, go, go2);
+                }
+            }
+            const float step = go2 > 0.f ? __fmul_ru(__fsqrt_ru(go2), 1.000001f) : 0.f;
+            if (step > 0.f) atomicMax(&s_move[it & 1], __float_as_uint(step));
+            if (lists) went[q] = step;
+        }
+        if (blockIdx.x == 0) {
+            const int old = (it + 2) % 3;
+            for (int i = tid; i < n * P; i += kFitThreads) w.delta[(size_t)old * n * P + i] = 0;
+            for (int i = tid; i < n; i += kFitThreads) w.delta_cnt[(size_t)old * n + i] = 0;
+        }
+        __syncthreads();
+        moved = __fadd_ru(moved, __uint_as_float(s_move[it & 1]));
+        if (tid == 0) s_move[(it + 1) & 1] = 0u;       // (last read before the barrier of this iteration)
+        if (lists) {
+            fresh = __fsub_ru(moved, moved_at_build) > 0.15f * __uint_as_float(s_min_excl);
+            // four threads per cell: the largest movement among its list
+            for (int q = tid; q < ((4 * n + 31) & ~31); q += kFitThreads) {
+                const int a = min(q >> 2, n - 1);
+                const uint4 idx = *reinterpret_cast<const uint4*>(near_idx + a * kNearRow + (q & 3) * 8);
+                const unsigned v[4] = {idx.x, idx.y, idx.z, idx.w};
+                float far = 0.f;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) far = fmaxf(far, fmaxf(went[v[k] & 0xffffu], went[v[k] >> 16]));
+                far = fmaxf(far, __shfl_xor_sync(0xffffffffu, far, 1));
+                far = fmaxf(far, __shfl_xor_sync(0xffffffffu, far, 2));
+                if (q < 4 * n && (q & 3) == 0) near_moved[a] = __fadd_ru(near_moved[a], far);
+            }
+            __syncthreads();
+        }
+    }
+    if (done && it < max_iters) {                       // (otherwise the last assignment step has added the errors up)
+        for (int64_t c = chunk0; c < chunks; c += chunk_step) {
+            const int64_t i = c * 32 + lane;
+            if (i >= m) continue;
+            float x[P];
+#pragma unroll
+            for (int k = 0; k < P; ++k) x[k] = samples[i * P + k];
+            err += (double)centre_distance<P>(x, sc + w.assign[i] * P);
+        }
+    }
+#pragma unroll
+    for (int k = 16; k > 0; k >>= 1) err += __shfl_xor_sync(0xffffffffu, err, k);
+    if (lane == 0) s_err[warp] = err;
+    __syncthreads();
+    if (tid == 0) {
+        double total = 0.0;
+        for (int i = 0; i < kFitThreads / 32; ++i) total += s_err[i];
+        w.err[blockIdx.x] = total;
+        if (blockIdx.x == 0) { w.flags[0] = done ? 1 : 0; w.flags[1] = it; }
+    }
+    if (blockIdx.x == 0)
+        for (int i = tid; i < n * P; i += kFitThreads) w.centres[i] = sc[i];
 }
 
-__global__ void grid_finalize_kernel(GridWs w, int p, int n, int64_t m, float* __restrict__ grid_out,
-                                     float* __restrict__ mse_out, int32_t* __restrict__ iters_out) {
-    // lexicographic sort by rank counting (coordinate 0 first; equal points keep their index order)
-    for (int c = threadIdx.x; c < n; c += blockDim.x) {
+__global__ void __launch_bounds__(256) grid_finalize_kernel(GridWs w, int p, int n, int64_t m, int blocks, float* __restrict__ grid_out,
+                                                            float* __restrict__ mse_out, int32_t* __restrict__ iters_out) {
+    // lexicographic sort by rank counting, one warp per centre (coordinate 0 first; equal points keep their index order)
+    const int lane = threadIdx.x & 31, c = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
+    if (c < n) {
         int rank = 0;
-        for (int o = 0; o < n; ++o) {
+        for (int o = lane; o < n; o += 32) {
             int cmp = 0;                                   // sign of (centre o) - (centre c)
             for (int k = 0; k < p && cmp == 0; ++k) {
                 const float a = w.centres[c * p + k], b = w.centres[o * p + k];
@@ -188,11 +487,18 @@ __global__ void grid_finalize_kernel(GridWs w, int p, int n, int64_t m, float* _
             }
             rank += (cmp < 0 || (cmp == 0 && o < c)) ? 1 : 0;
         }
-        for (int k = 0; k < p; ++k) grid_out[rank * p + k] = w.centres[c * p + k];
+        rank = __reduce_add_sync(0xffffffffu, rank);
+        if (lane < p) grid_out[rank * p + lane] = w.centres[c * p + lane];
     }
-    if (threadIdx.x == 0) {
-        if (mse_out) *mse_out = (float)(w.err[1] / ((double)m * p));
-        if (iters_out) *iters_out = w.flags[1] ? w.flags[2] : -w.flags[2];
+    if (c == 0) {
+        double e = 0.0;
+        for (int i = lane; i < blocks; i += 32) e += w.err[i];
+#pragma unroll
+        for (int k = 16; k > 0; k >>= 1) e += __shfl_xor_sync(0xffffffffu, e, k);
+        if (lane == 0) {
+            if (mse_out) *mse_out = (float)(e / ((double)m * p));
+            if (iters_out) *iters_out = w.flags[0] ? w.flags[1] : -w.flags[1];
+        }
     }
 }
 
@@ -261,100 +567,64 @@ int launch_uniform_grid(int n, float* grid_out, float* step_out, float* mse_out,
 }
 
 size_t make_grid_workspace(int p, int n, int64_t m) {
-    return up256(sizeof(float) * n * p) + up256(sizeof(double) * n * p) + up256(sizeof(unsigned long long) * n) + 512 +
-           up256(sizeof(int32_t) * (size_t)m);
+    return up256(sizeof(float) * n * p) + up256(sizeof(long long) * 3 * n * p) + up256(sizeof(int32_t) * 3 * n) +
+           up256(sizeof(double) * kMaxFitBlocks) + 256 + (sizeof(uint16_t) * kNear + sizeof(float)) * kMaxNearCentres +
+           up256(sizeof(int32_t) * (size_t)m) + up256(sizeof(float) * (size_t)m);
 }
 
-template <int P, bool SMALL>
-static int assign_step(GridWs w, const float* samples, int n, int64_t m, unsigned blocks, cudaStream_t st) {
-    const size_t smem = up256(sizeof(float) * n * P) + (SMALL ? sizeof(double) * n * P + sizeof(unsigned int) * n : 0);
-    if (smem > 48 * 1024) {
-        static int opted[64] = {0};                        // per instantiation and device: 1 = done, -1 = failed
-        const int ok = device_once(opted, [] {
-            return cudaFuncSetAttribute(grid_assign_kernel<P, SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)(up256(sizeof(float) * kMaxGridPoints * P))) == cudaSuccess ? 1 : -1;
-        });
-        if (ok < 0) return HIGGS_ERR_CUDA;
-    }
-    grid_assign_kernel<P, SMALL><<<blocks, 256, smem, st>>>(w, samples, n, m);
-    return HIGGS_OK;
-}
-
-// One cooperative launch for the whole iteration; returns HIGGS_ERR_UNSUPPORTED when the device or the shape does not
-// allow it (the caller then enqueues one pair of kernels per iteration).
 static int sm_count_of_device() {
     int dev = 0, v = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1) v = 1;
     return v;
 }
 
-template <int P, bool SMALL>
-static int fit_persistent(GridWs w, const float* samples, int n, int64_t m, int max_iters, cudaStream_t st) {
-    const size_t smem = up256(sizeof(float) * n * P) + (SMALL ? sizeof(double) * n * P + sizeof(unsigned int) * n : 0);
-    static int per_sm[64] = {0};          // resident blocks per SM at the largest shared-memory size, -1 = not available
-    const int bps = device_once(per_sm, [] {
+// One cooperative launch for the whole iteration, a block per SM (fewer when there are fewer than 32 samples for each); where
+// the device does not allow it, one ordinary block, whose barriers are trivial.
+template <int P>
+static int launch_fit(GridWs w, const float* samples, int n, int64_t m, int max_iters, int* blocks_out, cudaStream_t st) {
+    constexpr size_t kMaxSmem = (P * (sizeof(long long) + sizeof(float)) + sizeof(int)) * kMaxGridPoints;     // (n = 4096: no lists)
+    static int state[64] = {0};           // 1 = cooperative launch possible, 2 = not, -1 = failed
+    const int how = device_once(state, [] {
         int dev = 0, coop = 0, v = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop)
+        if (cudaFuncSetAttribute(grid_fit_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxSmem > 73728 ? kMaxSmem : 73728)) != cudaSuccess)
             return -1;
-        const size_t max_smem = up256(sizeof(float) * kMaxGridPoints * P) + (SMALL ? (sizeof(double) * P + sizeof(unsigned int)) * 256 : 0);
-        if (cudaFuncSetAttribute(grid_fit_kernel<P, SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem) != cudaSuccess) return -1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, grid_fit_kernel<P, SMALL>, 256, max_smem) != cudaSuccess || v < 1) return -1;
-        return v;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, grid_fit_kernel<P>, kFitThreads, kMaxSmem) != cudaSuccess || v < 1)
+            return 2;
+        return 1;
     });
-    if (bps < 1) return HIGGS_ERR_UNSUPPORTED;
-    int64_t blocks = (m + 255) / 256;
-    const int64_t cap = (int64_t)bps * sm_count_of_device();
-    if (blocks > cap) blocks = cap;
-    if (blocks > 592) blocks = 592;
-    void* args[] = {&w, &samples, &n, &m, &max_iters};
-    const cudaError_t e = cudaLaunchCooperativeKernel((const void*)grid_fit_kernel<P, SMALL>, dim3((unsigned)blocks), dim3(256), args, smem, st);
-    if (e != cudaSuccess) { (void)cudaGetLastError(); return HIGGS_ERR_UNSUPPORTED; }
-    return HIGGS_OK;
+    if (how < 0) return HIGGS_ERR_CUDA;
+    const size_t smem = fit_smem(P, n);
+    if (how == 1) {
+        int64_t blocks = (m + 31) / 32;
+        if (blocks > sm_count_of_device()) blocks = sm_count_of_device();
+        if (blocks > kMaxFitBlocks) blocks = kMaxFitBlocks;
+        void* args[] = {&w, &samples, &n, &m, &max_iters};
+        if (cudaLaunchCooperativeKernel((const void*)grid_fit_kernel<P>, dim3((unsigned)blocks), dim3(kFitThreads), args, smem, st) == cudaSuccess) {
+            *blocks_out = (int)blocks;
+            return HIGGS_OK;
+        }
+        (void)cudaGetLastError();
+    }
+    grid_fit_kernel<P><<<1, kFitThreads, smem, st>>>(w, samples, n, m, max_iters);
+    *blocks_out = 1;
+    return cuda_status(cudaGetLastError());
 }
 
 int launch_make_grid(int p, int n, const float* samples, int64_t m, int max_iters, float* grid_out, float* mse_out,
                      int32_t* iters_out, void* ws, cudaStream_t st) {
     GridWs w = carve(ws, p, n, m);
-    const int64_t init_threads = m > (int64_t)n * p ? m : (int64_t)n * p;
-    grid_init_kernel<<<(unsigned)((init_threads + 255) / 256), 256, 0, st>>>(w, samples, p, n, m);
-    int64_t blocks = (m + 255) / 256;
-    if (blocks > 592) blocks = 592;
-    const bool small = n <= 256;
-    {
-        int rc = HIGGS_ERR_UNSUPPORTED;
-        switch (p * 2 + (small ? 1 : 0)) {
-            case 3: rc = fit_persistent<1, true>(w, samples, n, m, max_iters, st); break;
-            case 2: rc = fit_persistent<1, false>(w, samples, n, m, max_iters, st); break;
-            case 5: rc = fit_persistent<2, true>(w, samples, n, m, max_iters, st); break;
-            case 4: rc = fit_persistent<2, false>(w, samples, n, m, max_iters, st); break;
-            case 7: rc = fit_persistent<3, true>(w, samples, n, m, max_iters, st); break;
-            case 6: rc = fit_persistent<3, false>(w, samples, n, m, max_iters, st); break;
-            case 9: rc = fit_persistent<4, true>(w, samples, n, m, max_iters, st); break;
-            case 8: rc = fit_persistent<4, false>(w, samples, n, m, max_iters, st); break;
-            default: return HIGGS_ERR_UNSUPPORTED;
-        }
-        if (rc == HIGGS_OK) {
-            grid_finalize_kernel<<<1, 256, 0, st>>>(w, p, n, m, grid_out, mse_out, iters_out);
-            return cuda_status(cudaGetLastError());
-        }
+    const int64_t init_threads = m > (int64_t)3 * n * p ? m : (int64_t)3 * n * p;
+    grid_init_kernel<<<(unsigned)((init_threads + 255) / 256), 256, 0, st>>>(w, p, n, m);
+    int blocks = 0, rc = HIGGS_ERR_UNSUPPORTED;
+    switch (p) {
+        case 1: rc = launch_fit<1>(w, samples, n, m, max_iters, &blocks, st); break;
+        case 2: rc = launch_fit<2>(w, samples, n, m, max_iters, &blocks, st); break;
+        case 3: rc = launch_fit<3>(w, samples, n, m, max_iters, &blocks, st); break;
+        case 4: rc = launch_fit<4>(w, samples, n, m, max_iters, &blocks, st); break;
     }
-    for (int it = 0; it < max_iters; ++it) {
-        int rc;
-        switch (p * 2 + (small ? 1 : 0)) {
-            case 3: rc = assign_step<1, true>(w, samples, n, m, (unsigned)blocks, st); break;
-            case 2: rc = assign_step<1, false>(w, samples, n, m, (unsigned)blocks, st); break;
-            case 5: rc = assign_step<2, true>(w, samples, n, m, (unsigned)blocks, st); break;
-            case 4: rc = assign_step<2, false>(w, samples, n, m, (unsigned)blocks, st); break;
-            case 7: rc = assign_step<3, true>(w, samples, n, m, (unsigned)blocks, st); break;
-            case 6: rc = assign_step<3, false>(w, samples, n, m, (unsigned)blocks, st); break;
-            case 9: rc = assign_step<4, true>(w, samples, n, m, (unsigned)blocks, st); break;
-            case 8: rc = assign_step<4, false>(w, samples, n, m, (unsigned)blocks, st); break;
-            default: return HIGGS_ERR_UNSUPPORTED;
-        }
-        if (rc != HIGGS_OK) return rc;
-        grid_update_kernel<<<1, 256, 0, st>>>(w, p, n);
-    }
-    grid_finalize_kernel<<<1, 256, 0, st>>>(w, p, n, m, grid_out, mse_out, iters_out);
+    if (rc != HIGGS_OK) return rc;
+    grid_finalize_kernel<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(w, p, n, m, blocks, grid_out, mse_out, iters_out);
     return cuda_status(cudaGetLastError());
 }
 

@@ -1,0 +1,54 @@
+"""The grid fit against the plain iteration in the same arithmetic (fp32 distances in coordinate order, lowest index on
+ties, fp64 means): skipped scans, moved samples and the split over blocks and warps must not show."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2411_17525_b200 as hb
+from tests import gpu_util as U
+
+pytestmark = pytest.mark.gpu
+
+
+def plain_lloyd(p, n, x, max_iters):
+    c = x[:n].copy()
+    old = np.full(len(x), -1)
+    for it in range(1, max_iters + 1):
+        a = np.empty(len(x), dtype=np.int64)
+        err = 0.0
+        for i in range(0, len(x), 4096):
+            e = (x[i:i + 4096, None, :] - c[None]).astype(np.float64)          # fp32 differences, widened
+            d = (e[..., 0] ** 2).astype(np.float32)
+            for k in range(1, p):
+                d = (e[..., k] ** 2 + d).astype(np.float32)                    # one rounding, as a fused multiply-add
+            a[i:i + 4096] = d.argmin(1)
+            err += float(d.min(1).astype(np.float64).sum())
+        if np.array_equal(a, old):
+            return c, err, it
+        old = a
+        size = np.bincount(a, minlength=n)
+        for k in range(p):
+            s = np.bincount(a, weights=x[:, k].astype(np.float64), minlength=n)
+            c[size > 0, k] = (s[size > 0] / size[size > 0]).astype(np.float32)
+    return c, err, -max_iters
+
+
+@pytest.mark.parametrize("p,n,m,max_iters", [
+    (1, 1, 1, 5), (1, 4, 31, 50), (2, 16, 33, 50),          # a part of a warp, one sample more than a warp
+    (2, 256, 257, 50),                                      # cells of one sample
+    (2, 65, 151559, 40), (1, 80, 40000, 60), (2, 300, 30000, 80), (3, 512, 20000, 30),                                   # more than one sample per lane on some warps
+    (1, 16, 8192, 400), (3, 830, 4000, 60), (4, 33, 20000, 60), (4, 4096, 5000, 4),
+])
+def test_fit_follows_the_plain_iteration(p, n, m, max_iters):
+    x = np.random.default_rng(7 * n + m).standard_normal((m, p)).astype(np.float32)
+    x[m // 2:m // 2 + 2] = x[0]                             # (equal samples: equal centres when both are among the first n)
+    c, err, iters = plain_lloyd(p, n, x, max_iters)
+    t = torch.from_numpy(x).to(U.dev())
+    grid, mse, it = hb.higgs_make_grid(p, n, t, max_iters=max_iters)
+    again, _, _ = hb.higgs_make_grid(p, n, t, max_iters=max_iters)
+    assert hb.higgs_device_status() == hb.HIGGS_OK
+    assert int(it) == iters
+    want = c[np.lexsort(c.T[::-1])]
+    assert np.max(np.abs(grid.cpu().numpy() - want)) <= 2.0 ** -22              # an fp32 rounding of a mean of size <= 4
+    assert abs(float(mse) - err / (m * p)) <= 1e-6 * err / (m * p) + 1e-30
+    assert torch.equal(grid, again)
