@@ -278,11 +278,14 @@ int higgs_linear_share(const higgs_desc* desc, const void* x, int64_t B, const v
  * independent per output row, so matrices with the same K, grid, group size and seed are one layer over their
  * concatenated rows - the activations are rotated once and, for batches up to 16 (the small-batch kernel, K ranges
  * not meeting in atomics), one kernel launch per 16 tokens streams all of them; for one or two tokens that launch also
- * does the rotation.  Other shapes and batches run as one higgs_linear per matrix (same results, no gain).
+ * does the rotation.  On the tensor-core path sets of at least 2 M weights whose matrices have multiples of 128 rows are
+ * one rotation and one product launch.  Other shapes and batches run as one higgs_linear per matrix (same results, no
+ * gain).
  *   count <= 4; descs[i], packed[i], scales[i], ys[i] (device [B][descs[i]->N] of y_dtype) belong to matrix i;
  *   descs must agree in p, n, g, K, rht_seed (else HIGGS_ERR_INVALID_ARG); grid and x are common;
  *   workspace: higgs_linear_multi_workspace_bytes(count, descs, B) bytes.  The arrays are HOST arrays.
- * Results equal those of higgs_linear on each matrix (bit for bit where neither uses atomics).
+ * Results equal those of higgs_linear on each matrix (bit for bit where neither uses atomics and K is cut alike; the
+ * tensor-core path cuts K by the number of row tiles, see higgs_linear_k_splits).
  * higgs_linear_multi_launch_count: kernels the call enqueues.
  */
 int higgs_linear_multi(int32_t count, const higgs_desc* const* descs, const void* x, int64_t B,

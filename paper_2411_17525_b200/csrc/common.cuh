@@ -177,10 +177,10 @@ __device__ __forceinline__ void apply_signs1024(float (&v)[32], uint64_t xi, int
 // registers, bits 3-7 across lanes); after, lane c*8 + e holds v[j] = element c*256 + j*8 + e (bits 3-7 in registers).
 // Same butterflies in the same order of stages as fwht1024_warp, so the values are bit-identical to it.  160 shuffles and
 // 160 fused multiply-adds become 8 vector stores, 32 loads and 160 additions: 64 shared-memory wavefronts instead of
-// 160.  `ex`: this warp's exchange buffer, kFwhtExchange floats, 16-byte aligned; rows of 36 floats keep the vector
-// stores (lane l writes row l) and the loads (lane l reads column l) free of bank conflicts.
-constexpr int kFwhtRow = 36;
-constexpr int kFwhtExchange = 32 * kFwhtRow;
+// 160.  `ex`: this warp's exchange buffer, 32 rows of 32 floats, 16-byte aligned; row l holds lane l's values, its
+// four-float chunks permuted by l % 8, which keeps the vector stores (lane l writes row l) and the loads (lane l reads
+// column l) free of bank conflicts.
+constexpr int kFwhtExchange = 1024;
 __device__ __forceinline__ void butterflies32(float (&v)[32]) {
 #pragma unroll
     for (int h = 1; h < 32; h <<= 1) {
@@ -198,11 +198,11 @@ __device__ __forceinline__ void fwht1024_to_columns(float (&v)[32], float* ex, i
     butterflies32(v);
     __syncwarp();            // (the buffer's previous readers)
 #pragma unroll
-    for (int r = 0; r < 32; r += 4)
-        *reinterpret_cast<float4*>(ex + lane * kFwhtRow + r) = make_float4(v[r], v[r + 1], v[r + 2], v[r + 3]);
+    for (int q = 0; q < 8; ++q)
+        *reinterpret_cast<float4*>(ex + lane * 32 + ((q ^ (lane & 7)) << 2)) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
     __syncwarp();
 #pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] = ex[j * kFwhtRow + lane];
+    for (int j = 0; j < 32; ++j) v[j] = ex[j * 32 + (lane ^ ((j & 7) << 2))];
     butterflies32(v);
 }
 // The inverse direction (H is symmetric: the same transform, columns in, rows out).
@@ -210,14 +210,32 @@ __device__ __forceinline__ void fwht1024_from_columns(float (&v)[32], float* ex,
     butterflies32(v);
     __syncwarp();
 #pragma unroll
-    for (int j = 0; j < 32; ++j) ex[j * kFwhtRow + lane] = v[j];
+    for (int j = 0; j < 32; ++j) ex[j * 32 + (lane ^ ((j & 7) << 2))] = v[j];
     __syncwarp();
 #pragma unroll
-    for (int r = 0; r < 32; r += 4) {
-        const float4 q = *reinterpret_cast<const float4*>(ex + lane * kFwhtRow + r);
-        v[r] = q.x; v[r + 1] = q.y; v[r + 2] = q.z; v[r + 3] = q.w;
+    for (int q = 0; q < 8; ++q) {
+        const float4 f = *reinterpret_cast<const float4*>(ex + lane * 32 + ((q ^ (lane & 7)) << 2));
+        v[4 * q] = f.x; v[4 * q + 1] = f.y; v[4 * q + 2] = f.z; v[4 * q + 3] = f.w;
     }
     butterflies32(v);
+}
+
+// Sign bits of this lane's 32 elements c*256 + l*8 + e of the group at input k0, bit c*8 + e of the result; and a value
+// with its sign flipped where bit r is set.
+__device__ __forceinline__ uint32_t lane_sign_bits(uint64_t xi, int64_t k0, int lane) {
+    const uint64_t word = sign_word(xi, ((uint64_t)k0 >> 6) + (uint64_t)(lane & 15));
+    const uint32_t lo = (uint32_t)word, hi = (uint32_t)(word >> 32);
+    uint32_t bits = 0u;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const int src = 4 * c + (lane >> 3);
+        const uint32_t from_lo = __shfl_sync(0xffffffffu, lo, src), from_hi = __shfl_sync(0xffffffffu, hi, src);
+        bits |= ((((lane & 4) ? from_hi : from_lo) >> ((lane & 3) * 8)) & 0xffu) << (8 * c);
+    }
+    return bits;
+}
+__device__ __forceinline__ float with_sign(float v, uint32_t bits, int r) {
+    return __uint_as_float(__float_as_uint(v) ^ ((bits << (31 - r)) & 0x80000000u));
 }
 
 // element index inside the group of register r of lane l (see above)
@@ -285,7 +303,7 @@ int tc_k_split(const higgs_desc& d, int64_t B);
 int launch_rht_tc(const higgs_desc& d, const void* x, int64_t B, __half* xdag_tc, cudaStream_t st);
 int launch_linear_tc(const higgs_desc& d, const __half* xdag_tc, int64_t B, const void* packed, const void* scales,
                      const float* grid, void* y, int y_mode, cudaStream_t st, int64_t ldy = 0,
-                     const GatherTargets* more = nullptr);
+                     const GatherTargets* more = nullptr, const MultiSegments* segs = nullptr);
 int read_tc_status(int clear);
 int launch_error_ratio(double* sums, cudaStream_t st);
 int read_grid_status(int clear);

@@ -68,23 +68,6 @@ __device__ __forceinline__ void fill_pair_table(float* table, const float* __res
     }
 }
 
-// Sign bits of this lane's 32 elements c*256 + l*8 + e of the group at input k0: byte c of the result.
-__device__ __forceinline__ uint32_t lane_sign_bits(uint64_t xi, int64_t k0, int lane) {
-    const uint64_t word = sign_word(xi, ((uint64_t)k0 >> 6) + (uint64_t)(lane & 15));
-    const uint32_t lo = (uint32_t)word, hi = (uint32_t)(word >> 32);
-    uint32_t bits = 0u;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const int src = 4 * c + (lane >> 3);
-        const uint32_t from_lo = __shfl_sync(0xffffffffu, lo, src), from_hi = __shfl_sync(0xffffffffu, hi, src);
-        bits |= ((((lane & 4) ? from_hi : from_lo) >> ((lane & 3) * 8)) & 0xffu) << (8 * c);
-    }
-    return bits;
-}
-__device__ __forceinline__ float with_sign(float v, uint32_t bits, int r) {
-    return __uint_as_float(__float_as_uint(v) ^ ((bits << (31 - r)) & 0x80000000u));
-}
-
 template <typename T>
 struct RawRow;
 template <>

@@ -47,7 +47,15 @@ struct TcParams {
     int B, BN, n, p, y_mode; // y_mode 0: fp32, 1: bf16
     int bits;                // log2(n)
     int ksplit;              // K slices (= cluster size along z); each a multiple of 256 inputs
+    // Several matrices that read the same activations (q|k|v, gate|up) as one product over their concatenated rows:
+    // matrix s holds the 128-row tiles [seg_tile[s], seg_tile[s + 1]).  nseg == 1: the fields above apply.
+    int nseg;
+    int seg_tile[kMaxMulti];
+    const __half* seg_scales[kMaxMulti];
+    void* seg_y[kMaxMulti];
+    int64_t seg_ldy[kMaxMulti];
 };
+struct CodeMaps { CUtensorMap map[kMaxMulti]; };
 
 constexpr uint32_t kTcSmem = 232448;
 constexpr int kTcGroups = 4;                 // dequant warp groups (4 warps each, one per TMEM lane quadrant)
@@ -159,7 +167,7 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
 // template parameter so that the MMA warp's loop body is straight-line code.
 // FMT: 0 = byte format, 1 = six-bit planes, 2 = nibble pairs (p=2 n=16, p=1 n=4), 3 = 8-bit scalar codes (p=1 n=256).
 template <int FB, int FMT>
-__global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const TcParams prm, const __grid_constant__ CUtensorMap code_map) {
+__global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const __grid_constant__ TcParams prm, const __grid_constant__ CodeMaps code_maps) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
@@ -207,7 +215,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const TcParams
     const int ksteps = ksteps_all / ksplit;                  // 64-input steps of this block, a multiple of 4
     const int kstep0 = kz * ksteps;
     const int nsuper = ksteps >> 2;                          // A stages (256 inputs) of this block
-    const int64_t row0 = (int64_t)blockIdx.x * 128;
+    int seg = 0, seg_begin = 0;
+    if (prm.nseg > 1) {
+#pragma unroll
+        for (int i = 1; i < kMaxMulti; ++i)
+            if ((int)blockIdx.x >= prm.seg_tile[i]) { seg = i; seg_begin = prm.seg_tile[i]; }
+    }
+    const CUtensorMap* code_map = &code_maps.map[seg];
+    const int64_t row0 = (int64_t)((int)blockIdx.x - seg_begin) * 128;       // inside its matrix
+    const __half* const scales = prm.nseg > 1 ? prm.seg_scales[seg] : prm.scales;
+    void* const y = prm.nseg > 1 ? prm.seg_y[seg] : prm.y;
+    const int64_t ldy = prm.nseg > 1 ? prm.seg_ldy[seg] : prm.ldy;
     const int bt = blockIdx.y;
     const uint32_t b_step_bytes = (uint32_t)BN * 128u;
     const int tile0 = (int)(row0 / 16);                      // first 16-row tile of this block
@@ -257,7 +275,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const TcParams
             for (int j = 0; j < n0; ++j) {
                 if (elected) {
                     t_mbar_expect_tx(code_full(j), kTcCodeStage);
-                    t_tensor_load(code_stage(j), &code_map, (kstep0 / SPS + j) * (int)(kTcCodeStage / 64u), tile0, code_full(j));
+                    t_tensor_load(code_stage(j), code_map, (kstep0 / SPS + j) * (int)(kTcCodeStage / 64u), tile0, code_full(j));
                 }
                 __syncwarp();
             }
@@ -306,7 +324,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const TcParams
             bad |= t_wait(code_empty(s), (uint32_t)((it & 1) ^ 1), t_limit(bad)) ^ 1u;
             if (elected) {
                 t_mbar_expect_tx(code_full(s), kTcCodeStage);
-                t_tensor_load(code_stage(s), &code_map, (kstep0 / SPS + j) * (int)(kTcCodeStage / 64u), tile0, code_full(s));
+                t_tensor_load(code_stage(s), code_map, (kstep0 / SPS + j) * (int)(kTcCodeStage / 64u), tile0, code_full(s));
             }
             ++issued;
             const bool wrap = s + 1 == CS;
@@ -398,7 +416,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const TcParams
         const uint32_t sel0 = 0x7604u + ((uint32_t)h << 4), sel1 = 0x7624u + ((uint32_t)h << 4);   // bytes h and h+2 of a word
         const int rot = g >> 1;                    // chunk rotation that makes the 16-byte code loads conflict-free
         const int groups = (int)(prm.K / kGroup);
-        const __half* sc_row = prm.scales + ((row0 / 16 + rtl) * groups) * 16 + (i & 15);
+        const __half* sc_row = scales + ((row0 / 16 + rtl) * groups) * 16 + (i & 15);
         const uint32_t t_lane = tmem + ((uint32_t)(32 * q) << 16);
         // byte formats: this row's words are the 16-byte chunks of lanes (g, t) of its row tile; six-bit: word 2 (4g + t) +
         // (step & 1) of each of the tile's three 256-byte planes
@@ -572,17 +590,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const TcParams
                 uint32_t v0, v1, v2, v3;
                 asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v0), "=r"(v1), "=r"(v2), "=r"(v3)
                              : "r"(code0 + (uint32_t)((c * 128 + lane * 4) * 4)) : "memory");
-                const int64_t o = (int64_t)b * prm.ldy + row0 + lane * 4;
+                const int64_t o = (int64_t)b * ldy + row0 + lane * 4;
                 if (prm.y_mode == 0) {
                     const uint4 v = make_uint4(v0, v1, v2, v3);
-                    *reinterpret_cast<uint4*>(static_cast<float*>(prm.y) + o) = v;
+                    *reinterpret_cast<uint4*>(static_cast<float*>(y) + o) = v;
                     for (int pd = 0; pd < prm.n_more; ++pd)       // gathered output: the other devices' copies
                         *reinterpret_cast<uint4*>(static_cast<float*>(prm.y_more[pd]) + o) = v;
                 } else {
                     const __nv_bfloat162 lo = __floats2bfloat162_rn(__uint_as_float(v0), __uint_as_float(v1));
                     const __nv_bfloat162 hi = __floats2bfloat162_rn(__uint_as_float(v2), __uint_as_float(v3));
                     const uint2 v = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
-                    *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(prm.y) + o) = v;
+                    *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(y) + o) = v;
                     for (int pd = 0; pd < prm.n_more; ++pd)
                         *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(prm.y_more[pd]) + o) = v;
                 }
@@ -619,15 +637,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const TcParams
                 }
                 const int b = bt * BN + c;
                 if (b < prm.B) {
-                    const int64_t o = (int64_t)b * prm.ldy + row0 + lane * 4;
+                    const int64_t o = (int64_t)b * ldy + row0 + lane * 4;
                     if (prm.y_mode == 0) {
-                        *reinterpret_cast<float4*>(static_cast<float*>(prm.y) + o) = acc;
+                        *reinterpret_cast<float4*>(static_cast<float*>(y) + o) = acc;
                         for (int pd = 0; pd < prm.n_more; ++pd)
                             *reinterpret_cast<float4*>(static_cast<float*>(prm.y_more[pd]) + o) = acc;
                     } else {
                         const __nv_bfloat162 lo = __floats2bfloat162_rn(acc.x, acc.y), hi = __floats2bfloat162_rn(acc.z, acc.w);
                         const uint2 v = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
-                        *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(prm.y) + o) = v;
+                        *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(y) + o) = v;
                         for (int pd = 0; pd < prm.n_more; ++pd)
                             *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(prm.y_more[pd]) + o) = v;
                     }
@@ -644,71 +662,69 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const TcParams
 
 namespace {
 
-// Rotation of the activations (Appendix F) for the tensor-core path: four warps per (token, group) - the transform sits
-// on the latency path between dependent launches -, output written in the blocked order the MMA's shared-memory
+// Rotation of the activations (Appendix F) for the tensor-core path, output in the blocked order the MMA's shared-memory
 // descriptor expects, so that one stage (BN tokens x 64 inputs) is one contiguous run:
 //   [batch tile][K/64][BN/8 token blocks][8 input cores][8 tokens][8 inputs] fp16.
-// Warp q of the block owns inputs 256 q .. + 255 of the group, 8 consecutive ones per lane (one core-matrix row):
-// butterflies over those 8 in registers, over the 32 lanes by shuffles, over the 4 warps through shared memory.
-__global__ void __launch_bounds__(128) rht_activations_tc_kernel(const __nv_bfloat16* __restrict__ x, __half* __restrict__ xdag,
-                                                                 int64_t B, int64_t K, uint64_t xi, int BN) {
-    __shared__ __align__(16) float ex[4][256];
-    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
-    const int64_t groups = K / kGroup;
+// A block rotates one 1024-group of the eight tokens of a token block, one warp each; the rotated halves meet in shared
+// memory (over the exchange buffers, which are idle by then), from where the block writes sixteen runs of 1 KB.  Tokens
+// beyond the batch are written as zeros.  Bound: memory for long prompts (4 bytes per activation), else the latency of
+// one warp's transform.  1999 tokens x 4096: 22 -> 12.3 us, x 14336: 69 -> 33 us (before: four warps per group with five
+// shuffle stages, 16-byte stores 128 bytes apart).
+constexpr int kRotWarps = 8;
+__global__ void __launch_bounds__(kRotWarps * 32) rht_activations_tc_kernel(const __nv_bfloat16* __restrict__ x, __half* __restrict__ xdag,
+                                                                            int64_t B, int64_t K, uint64_t xi, int BN) {
+    __shared__ __align__(16) float ex[kRotWarps][kFwhtExchange];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int groups = (int)(K / kGroup), blocks_per_tile = BN / 8;
+    const int64_t tb = blockIdx.x / groups;                     // token block
+    const int gi = (int)(blockIdx.x % groups);
+    const int64_t bt = tb / blocks_per_tile, nb = tb % blocks_per_tile;
+    const int64_t b = bt * BN + nb * 8 + warp;                  // this warp's token
+    const uint32_t sign = lane_sign_bits(xi, (int64_t)gi * kGroup, lane);
     pdl_trigger();
     pdl_wait();
-    const int64_t b = blockIdx.x / groups, gi = blockIdx.x % groups;       // grid = B * groups blocks
-    const int64_t k0 = gi * kGroup + q * 256 + lane * 8;
-    float v[8];
-    {
-        const uint4 q4 = __ldg(reinterpret_cast<const uint4*>(x + b * K + k0));
-        const uint32_t w4[4] = {q4.x, q4.y, q4.z, q4.w};
-        const uint32_t bits = (uint32_t)(sign_word(xi, (uint64_t)k0 >> 6) >> ((uint64_t)k0 & 63ull)) & 0xffu;
+    float v[32];
+    if (b < B) {
+        const uint4* src = reinterpret_cast<const uint4*>(x + b * K + (int64_t)gi * kGroup) + lane;
+        uint4 raw[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            v[2 * e] = __uint_as_float((w4[e] << 16) ^ (((bits >> (2 * e)) & 1u) << 31));
-            v[2 * e + 1] = __uint_as_float((w4[e] & 0xffff0000u) ^ (((bits >> (2 * e + 1)) & 1u) << 31));
+        for (int c = 0; c < 4; ++c) raw[c] = __ldg(src + c * 32);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const uint32_t w[4] = {raw[c].x, raw[c].y, raw[c].z, raw[c].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                v[c * 8 + 2 * e] = with_sign(__uint_as_float(w[e] << 16), sign, c * 8 + 2 * e);
+                v[c * 8 + 2 * e + 1] = with_sign(__uint_as_float(w[e] & 0xffff0000u), sign, c * 8 + 2 * e + 1);
+            }
         }
+        fwht1024_to_columns(v, ex[warp], lane);
+    } else {
+#pragma unroll
+        for (int r = 0; r < 32; ++r) v[r] = 0.f;
     }
-#pragma unroll
-    for (int h = 1; h < 8; h <<= 1) {
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            if ((r & h) == 0) { const float a = v[r], c = v[r | h]; v[r] = a + c; v[r | h] = a - c; }
-        }
-    }
-#pragma unroll
-    for (int m = 1; m < 32; m <<= 1) {
-        const bool upper = (lane & m) != 0;
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            const float o = __shfl_xor_sync(0xffffffffu, v[r], m);
-            v[r] = upper ? (o - v[r]) : (v[r] + o);
-        }
-    }
-    *reinterpret_cast<float4*>(&ex[q][lane * 8]) = make_float4(v[0], v[1], v[2], v[3]);
-    *reinterpret_cast<float4*>(&ex[q][lane * 8 + 4]) = make_float4(v[4], v[5], v[6], v[7]);
     __syncthreads();
-    float o[8];
+    // Lane c*8 + e holds inputs c*256 + j*8 + e.  A lane and its neighbour exchange halves so that each holds the pairs
+    // (e & 6, + 1) for sixteen j (even lanes j < 16).  Piece p = 32 c + j of the staging area is the 128 bytes of one core:
+    // token t at 16-byte slot t ^ ((p >> 4) & 7), which spreads a store's lanes over all banks.
+    uint32_t* stage = reinterpret_cast<uint32_t*>(&ex[0][0]);
+    const uint32_t pick = (lane & 1) ? 0x3276u : 0x5410u;
+    const int p0 = (lane >> 3) * 32 + 16 * (lane & 1), slot = warp ^ ((p0 >> 4) & 7);
 #pragma unroll
-    for (int r = 0; r < 8; ++r) o[r] = 0.f;
-#pragma unroll
-    for (int qq = 0; qq < 4; ++qq) {
-        const float4 u0 = *reinterpret_cast<const float4*>(&ex[qq][lane * 8]);
-        const float4 u1 = *reinterpret_cast<const float4*>(&ex[qq][lane * 8 + 4]);
-        const float sgn = (__popc(q & qq) & 1) ? -1.f : 1.f;
-        o[0] = fmaf(sgn, u0.x, o[0]); o[1] = fmaf(sgn, u0.y, o[1]); o[2] = fmaf(sgn, u0.z, o[2]); o[3] = fmaf(sgn, u0.w, o[3]);
-        o[4] = fmaf(sgn, u1.x, o[4]); o[5] = fmaf(sgn, u1.y, o[5]); o[6] = fmaf(sgn, u1.z, o[6]); o[7] = fmaf(sgn, u1.w, o[7]);
+    for (int i = 0; i < 16; ++i) {
+        const __half2 h = __floats2half2_rn(v[i] * 0.03125f, v[i + 16] * 0.03125f);
+        const uint32_t own = *reinterpret_cast<const uint32_t*>(&h);
+        const uint32_t other = __shfl_xor_sync(0xffffffffu, own, 1);
+        stage[(p0 + i) * 32 + slot * 4 + ((lane & 7) >> 1)] = __byte_perm(own, other, pick);
     }
-    uint32_t w4[4];
+    __syncthreads();
+    uint4* out = reinterpret_cast<uint4*>(xdag + (bt * (K / 64) + gi * 16) * (int64_t)BN * 64 + nb * 512);
+    const int64_t step = (int64_t)BN * 64 / 8;                  // 16-byte units between consecutive 64-input steps
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const __half2 hh = __floats2half2_rn(o[2 * e] * 0.03125f, o[2 * e + 1] * 0.03125f);
-        w4[e] = *reinterpret_cast<const uint32_t*>(&hh);
+    for (int r = 0; r < 4; ++r) {
+        const int u = r * 256 + (int)threadIdx.x, p = u >> 3;   // unit u & 63 of the run of 64-input step u >> 6
+        out[(u >> 6) * step + (u & 63)] = reinterpret_cast<const uint4*>(stage)[p * 8 + ((u & 7) ^ ((p >> 4) & 7))];
     }
-    const int64_t bt = b / BN, nloc = b % BN;
-    const int64_t off = ((bt * (K / 64) + k0 / 64) * BN * 64) + (nloc / 8) * 512 + ((k0 % 64) / 8) * 64 + (nloc % 8) * 8;
-    *reinterpret_cast<uint4*>(xdag + off) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
 }
 
 }  // namespace
@@ -739,9 +755,10 @@ size_t tc_workspace_bytes(const higgs_desc& d, int64_t B) {
 // D1 for the tensor-core path: rotated activations in the blocked operand layout (tc_workspace_bytes() bytes).
 int launch_rht_tc(const higgs_desc& d, const void* x, int64_t B, __half* xdag_tc, cudaStream_t st) {
     const int BN = tc_batch_tile(B);
-    const int64_t blocks = B * (d.K / kGroup);              // four warps per (token, group)
+    const int64_t tiles = (B + BN - 1) / BN;
+    const int64_t blocks = tiles * (BN / 8) * (d.K / kGroup);          // one per (token block, group)
     if (blocks > 0x7fffffff) return HIGGS_ERR_UNSUPPORTED;
-    return cuda_status(launch_pdl(rht_activations_tc_kernel, dim3((unsigned)blocks), dim3(128), 0, st,
+    return cuda_status(launch_pdl(rht_activations_tc_kernel, dim3((unsigned)blocks), dim3(kRotWarps * 32), 0, st,
                                   static_cast<const __nv_bfloat16*>(x), xdag_tc, B, d.K, d.rht_seed, BN));
 }
 
@@ -796,8 +813,10 @@ bool make_code_map(const higgs_desc& d, const void* packed, CUtensorMap* map) {
 
 // D2-D5 on the tensor cores, from activations rotated by launch_rht_tc for the same B.
 int launch_linear_tc(const higgs_desc& d, const __half* xdag_tc, int64_t B, const void* packed, const void* scales,
-                     const float* grid, void* y, int y_mode, cudaStream_t st, int64_t ldy, const GatherTargets* more) {
+                     const float* grid, void* y, int y_mode, cudaStream_t st, int64_t ldy, const GatherTargets* more,
+                     const MultiSegments* segs) {
     if (more && more->count > kMaxGather - 1) return HIGGS_ERR_INVALID_ARG;
+    if (segs && (segs->count < 1 || segs->count > kMaxMulti || more)) return HIGGS_ERR_INVALID_ARG;
     const int BN = tc_batch_tile(B);
     const int64_t tiles = (B + BN - 1) / BN;
     static int configured[64] = {0};
@@ -812,9 +831,26 @@ int launch_linear_tc(const higgs_desc& d, const __half* xdag_tc, int64_t B, cons
         return 1;
     });
     if (conf < 0) return HIGGS_ERR_CUDA;
-    CUtensorMap code_map;
-    if (!make_code_map(d, packed, &code_map)) return HIGGS_ERR_CUDA;
-    TcParams prm;
+    CodeMaps maps;
+    TcParams prm = {};
+    prm.nseg = segs ? segs->count : 1;
+    if (!segs) {
+        if (!make_code_map(d, packed, &maps.map[0])) return HIGGS_ERR_CUDA;
+    } else {
+        int64_t tile = 0;
+        for (int i = 0; i < kMaxMulti; ++i) {
+            prm.seg_tile[i] = i < segs->count ? (int)tile : 0x7fffffff;      // (no tile lies beyond the last matrix)
+            if (i >= segs->count) continue;
+            higgs_desc one = d;
+            one.N = segs->rows[i];
+            if (one.N % 128 || !make_code_map(one, segs->packed[i], &maps.map[i])) return one.N % 128 ? HIGGS_ERR_INVALID_ARG : HIGGS_ERR_CUDA;
+            prm.seg_scales[i] = static_cast<const __half*>(segs->scales[i]);
+            prm.seg_y[i] = segs->y[i];
+            prm.seg_ldy[i] = segs->rows[i];
+            tile += segs->rows[i] / 128;
+        }
+        if (tile * 128 != d.N) return HIGGS_ERR_INVALID_ARG;
+    }
     prm.packed = static_cast<const uint8_t*>(packed);
     prm.scales = static_cast<const __half*>(scales);
     prm.grid = grid;
@@ -847,7 +883,7 @@ int launch_linear_tc(const higgs_desc& d, const __half* xdag_tc, int64_t B, cons
     // rest of shared memory) and 32 KB for wider tiles
     const Format fmt = format_of(d.p, d.n);
     const int fi = fmt == Format::kSixBit ? 1 : fmt == Format::kNibble ? 2 : fmt == Format::kByte8 ? 3 : 0;
-    typedef void (*TcKernel)(const TcParams, const CUtensorMap);
+    typedef void (*TcKernel)(const TcParams, const CodeMaps);
     static const TcKernel table[3][4] = {
         {linear_tc_kernel<4, 0>, linear_tc_kernel<4, 1>, linear_tc_kernel<4, 2>, linear_tc_kernel<4, 3>},
         {linear_tc_kernel<2, 0>, linear_tc_kernel<2, 1>, linear_tc_kernel<2, 2>, linear_tc_kernel<2, 3>},
@@ -868,7 +904,7 @@ int launch_linear_tc(const higgs_desc& d, const __half* xdag_tc, int64_t B, cons
             cfg.numAttrs = 1;
         }
     }
-    return cuda_status(cudaLaunchKernelEx(&cfg, kernel, prm, code_map));
+    return cuda_status(cudaLaunchKernelEx(&cfg, kernel, prm, maps));
 }
 
 // Failure-path check for the tensor-core kernel's wait helper: a barrier nothing arrives at, no copy or MMA in flight.
