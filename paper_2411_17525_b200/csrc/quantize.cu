@@ -221,7 +221,8 @@ __global__ void __launch_bounds__(128) encode_kernel(const T* __restrict__ W, co
 // ---- exact pruned search ---------------------------------------------------------------------------------------
 // The same nearest-point rule as above, evaluated only on the grid points that can win.  The plane (the line for
 // p = 1) is cut into square cells; cell i of an axis covers the values whose scaled coordinate x * cells / 2R + cells / 2
-// rounds to i (found with one fused multiply-add onto 2^23: the integer is then the low bits of the float).  A cell's
+// rounds to i.  The encoder finds it with two fused multiply-adds: onto [0, 1] with saturation, then onto 2^23, where the
+// integer is the low bits of the float; values beyond the table (and NaN) fall into the outermost cells, which are marked.  A cell's
 // candidate list is built in two steps.  (1) U = min over grid points of the distance to the cell's farthest corner
 // bounds the winner's distance from any point of the cell, so only points whose distance to the cell is at most U (+ a
 // slack far above fp32 rounding) can be nearest.  (2) Of those, c is dropped if another candidate c' is nearer at all
@@ -285,7 +286,8 @@ __global__ void __launch_bounds__(256) build_cells_kernel(const float* __restric
         }
         __syncwarp();
         uint32_t word = kCellScan;
-        if (k <= kPrefilter) {
+        const bool border = cx == 0 || cx == CELLS - 1 || (P == 2 && (cy == 0 || cy == CELLS - 1));
+        if (k <= kPrefilter && !border) {
             // step (2): lane i judges candidate i against every candidate j
             const bool have = lane < k;
             const int mine = have ? slist[wi][lane] : 0;
@@ -347,15 +349,15 @@ __device__ __forceinline__ void enc_mbar_wait(uint32_t bar, uint32_t parity) {
     atomicExch(&g_encode_status, (int)HIGGS_ERR_TIMEOUT);
 }
 
-// the exhaustive scan of one point by the whole warp (lowest index among equal distances); point c is the first
-// eight (four for p = 1) bytes of row c of the replicated grid
+// the exhaustive scan of one point by the whole warp (lowest index among equal distances); the first eight (four for
+// p = 1) bytes of row c of the replicated grid are point c, negated
 template <int P>
 __device__ __noinline__ int warp_scan(const uint8_t* rep, int n, float px, float py, int lane) {
     float bd = INFINITY;
     int bc = 0x7fffffff;
     for (int c = lane; c < n; c += 32) {           // ascending within the lane: '<' keeps its lowest index
         const float* g = reinterpret_cast<const float*>(rep + c * 128);
-        const float dx = px - g[0], dy = P == 2 ? py - g[1] : 0.f;
+        const float dx = px + g[0], dy = P == 2 ? py + g[1] : 0.f;
         const float d = P == 2 ? fmaf(dy, dy, dx * dx) : dx * dx;
         if (d < bd) { bd = d; bc = c; }
     }
@@ -368,78 +370,222 @@ __device__ __noinline__ int warp_scan(const uint8_t* rep, int n, float px, float
     return bc == 0x7fffffff ? 0 : bc;               // no distance compared below infinity (a NaN input): index 0, as the scan
 }
 
-// Persistent blocks of 16 warps; a block takes one row tile (16 rows) x one group per turn, warp w the tile's row w.
-// Shared memory: the cell table; the grid with every point repeated across a 128-byte row (16 copies of an 8-byte
-// point for p = 2, 32 copies of a float for p = 1: a lane reads "its" copy and the 32 lookups of a warp never meet in
-// a bank); two tiles of canonical codes, through which the block emits the packed stream itself (thread t assembles
-// the words of 64-input block t / 32, lane t % 32).  The warps of a block are not held in step: a warp puts its row
-// into the turn's tile and arrives on an mbarrier, and only a turn later - after its next search - waits for that
-// phase and packs the finished tile, so a warp may run up to one turn ahead of the slowest (a block-wide barrier per
-// turn made all sixteen warps wait for memory together and cost 20 %).  Writing tile t % 2 in turn t is safe: it was
-// last read when every warp packed tile t - 2, before its arrival of turn t - 1, which this warp has waited for.
+// two fp32 operations in one instruction
+__device__ __forceinline__ uint64_t pair_of(float a, float b) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
+    return v;
+}
+__device__ __forceinline__ void unpair(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) { uint64_t v; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b)); return v; }
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) { uint64_t v; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b)); return v; }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) { uint64_t v; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b)); return v; }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t v;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
+    return v;
+}
+__device__ __forceinline__ void pair_stages(uint64_t (&q)[16]) {
+#pragma unroll
+    for (int h = 1; h < 16; h <<= 1) {
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+            if ((t & h) == 0) {
+                const uint64_t a = q[t], b = q[t | h];
+                q[t] = add2(a, b);
+                q[t | h] = sub2(a, b);
+            }
+        }
+    }
+}
+
+// The encoder's transform: the butterflies of fwht1024_warp in the same order (bit-identical values), on pairs.  In: q[t] =
+// elements (c*256 + lane*8 + 2 (t & 3), + 1), c = t >> 2, after the stage of bit 0.  Bits 1, 2, 8, 9 are register stages, bit 3
+// a shuffle stage; then the pairs are exchanged through shared memory so that bits 4 to 7 are register stages too: out,
+// q[s] = elements (e0 + 16 s, + 1) with e0 = encoder_element(lane).  `ex` is 2 KB per warp: the sixteen lower lanes'
+// pairs go first, then the upper lanes'; row r = lane & 15 is 128 bytes, its 16-byte chunks permuted by r % 8 (no bank
+// conflicts either way).  256 instructions and 96 shared-memory wavefronts; 480 and 160 with five shuffle stages.
+__device__ __forceinline__ int encoder_element(int lane) { return ((lane >> 1) & 3) * 2 + (lane & 1) * 8 + (lane >> 3) * 256; }
+__device__ __forceinline__ void encoder_transform(uint64_t (&q)[16], uint8_t* ex, int lane) {
+    pair_stages(q);
+    const float sgn = (lane & 1) ? -1.0f : 1.0f;
+    const uint64_t sgn2 = pair_of(sgn, sgn);
+#pragma unroll
+    for (int t = 0; t < 16; ++t) {
+        float a, b;
+        unpair(q[t], a, b);
+        q[t] = fma2(q[t], sgn2, pair_of(__shfl_xor_sync(0xffffffffu, a, 1), __shfl_xor_sync(0xffffffffu, b, 1)));
+    }
+    uint64_t o[16];
+    const int r = lane & 15, l0 = lane & 1, k = lane >> 1;
+    __syncwarp();                     // (the buffer's previous readers)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        if ((lane >> 4) == h) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) *reinterpret_cast<ulonglong2*>(ex + r * 128 + ((j ^ (r & 7)) << 4)) = make_ulonglong2(q[2 * j], q[2 * j + 1]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+            const int row = l0 | (s << 1);
+            o[8 * h + s] = *reinterpret_cast<const uint64_t*>(ex + row * 128 + (((k >> 1) ^ (row & 7)) << 4) + (k & 1) * 8);
+        }
+        if (h == 0) __syncwarp();
+    }
+#pragma unroll
+    for (int s = 0; s < 16; ++s) q[s] = o[s];
+    pair_stages(q);
+}
+
+// A row's 1024 values in the lane order above (element c*256 + lane*8 + e), raw.
+template <typename T>
+struct RawGroup;
+template <>
+struct RawGroup<__nv_bfloat16> {
+    uint4 q[4];
+    __device__ __forceinline__ void load(const __nv_bfloat16* __restrict__ src, int lane) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) q[c] = __ldg(reinterpret_cast<const uint4*>(src + c * 256 + lane * 8));
+    }
+    __device__ __forceinline__ uint32_t word(int t) const { return (t & 3) == 0 ? q[t >> 2].x : (t & 3) == 1 ? q[t >> 2].y : (t & 3) == 2 ? q[t >> 2].z : q[t >> 2].w; }
+    // pair t with the signs of bits 2t, 2t + 1 of `bits` flipped: one multiply puts both bits on the two sign positions
+    __device__ __forceinline__ void get_signed(int t, uint32_t bits, float& a, float& b) const {
+        const uint32_t byte = (bits >> (8 * (t >> 2))) & 0xffu;
+        const uint32_t w = word(t) ^ ((byte * ((1u << (15 - 2 * (t & 3))) + (1u << (30 - 2 * (t & 3))))) & 0x80008000u);
+        a = __uint_as_float(w << 16);
+        b = __uint_as_float(w & 0xffff0000u);
+    }
+};
+template <>
+struct RawGroup<float> {
+    float4 q[8];
+    __device__ __forceinline__ void load(const float* __restrict__ src, int lane) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) q[c] = __ldg(reinterpret_cast<const float4*>(src + (c >> 1) * 256 + lane * 8 + (c & 1) * 4));
+    }
+    __device__ __forceinline__ void get_signed(int t, uint32_t bits, float& a, float& b) const {
+        a = with_sign((t & 1) ? q[t >> 1].z : q[t >> 1].x, bits, 2 * t);
+        b = with_sign((t & 1) ? q[t >> 1].w : q[t >> 1].y, bits, 2 * t + 1);
+    }
+};
+
+constexpr int kEncThreads = 1024, kEncTiles = 3, kEncExchange = 2048;
+// A row of the encoder's tile: the codes of every 256 values are followed by 8 (p = 2) or 16 bytes, which spreads the
+// lanes' byte stores (128 or 256 bytes apart) over the banks; rows are an odd multiple of 16 bytes apart in bank position.
+__host__ __device__ constexpr int enc_run(int P) { return P == 2 ? 136 : 272; }
+__host__ __device__ constexpr int enc_row_bytes(int P) { return 4 * enc_run(P) + 16; }
+__host__ __device__ constexpr size_t encode_smem(int P, int n) {
+    return (size_t)(P == 2 ? kCells2 * kCells2 : kCells1) * 4 + (size_t)n * 128 + 2 * kEncTiles * 16 * (size_t)enc_row_bytes(P) +
+           32 * (size_t)kEncExchange + 16;
+}
+static_assert(encode_smem(2, 256) <= 232448 && encode_smem(1, 256) <= 232448, "one block per SM");
+
+// One persistent block of 32 warps per SM, two independent halves; a half takes one row tile (16 rows) x one group per
+// turn, warp w of it row w.  Shared memory: the cell table; the grid, negated, with every point repeated across a 128-byte
+// row (16 copies of an 8-byte point for p = 2, 32 copies of a float for p = 1: a lane reads "its" copy and the 32 lookups
+// of a warp never meet in a bank); the warps' exchange buffers; and per half three tiles of canonical codes, through which
+// it emits the packed stream itself (thread t assembles the words of 64-input block t / 32, lane t % 32).  The warps of a
+// half are not held in step: a warp writes its codes into the turn's tile while it searches, then waits for the others'
+// arrivals of the turn BEFORE on an mbarrier, packs that turn's tile and arrives for its own - so a warp may run up to one
+// turn ahead of the slowest (a block-wide barrier per turn made all sixteen warps wait for memory together and cost 20 %).
+// Writing tile t % 3 in turn t is safe: it was last read when every warp packed turn t - 3, before its arrival of turn
+// t - 2, which this warp has waited for.
 // canonical and packed may each be null (not both).
+// Bound: instruction issue (69 % of the slots; ALU and FMA pipes 65 % each) next to the shared-memory path (71 %): 1547 warp
+// instructions and 452 wavefronts per row and group (1774 and about 600 with shuffle butterflies, scalar fp32 and the
+// codes gathered in registers).  14336 x 4096 bf16, n = 256: 135 -> 130 us; the 8B layers 535 -> 498 us.
 template <typename T, int P>
-__global__ void __launch_bounds__(512, 2) encode_pruned_kernel(const T* __restrict__ W, const float* __restrict__ grid, int n,
-                                                               const uint32_t* __restrict__ table,
-                                                               uint8_t* __restrict__ canonical, uint32_t* __restrict__ packed,
-                                                               int fmt, int bits, __half* __restrict__ scales,
-                                                               int64_t N, int64_t K, uint64_t xi) {
+__global__ void __launch_bounds__(kEncThreads, 1) encode_pruned_kernel(const T* __restrict__ W, const float* __restrict__ grid, int n,
+                                                                       const uint32_t* __restrict__ table,
+                                                                       uint8_t* __restrict__ canonical, uint32_t* __restrict__ packed,
+                                                                       int fmt, int bits, __half* __restrict__ scales,
+                                                                       int64_t N, int64_t K, uint64_t xi) {
     constexpr int NC = P == 2 ? kCells2 * kCells2 : kCells1;
     constexpr int CELLS = P == 2 ? kCells2 : kCells1;
-    constexpr int RS = kTileRowBytes(P);
+    constexpr int RS = enc_row_bytes(P);
     extern __shared__ __align__(128) uint8_t enc_smem[];
     uint32_t* cells = reinterpret_cast<uint32_t*>(enc_smem);
     uint8_t* rep = enc_smem + (size_t)NC * 4;
-    uint8_t* tiles_base = rep + (size_t)n * 128;
-    const uint32_t bar = enc_smem_u32(tiles_base + 2 * 16 * RS);      // mbarrier: one arrival per warp and turn
-    if (threadIdx.x == 0) enc_mbar_init(bar, 16);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, half = warp >> 4, wib = warp & 15;
+    uint8_t* ex = rep + (size_t)n * 128 + warp * kEncExchange;
+    uint8_t* tiles_base = rep + (size_t)n * 128 + 32 * kEncExchange + half * (kEncTiles * 16 * RS);
+    const uint32_t bar = enc_smem_u32(rep + (size_t)n * 128 + 32 * kEncExchange + 2 * kEncTiles * 16 * RS) + 8u * half;   // one arrival per warp and turn
+    if (wib == 0 && lane == 0) enc_mbar_init(bar, 16);
     for (int i = threadIdx.x; i < NC / 4; i += blockDim.x)
         reinterpret_cast<uint4*>(cells)[i] = reinterpret_cast<const uint4*>(table)[i];
     for (int i = threadIdx.x; i < n * 32; i += blockDim.x)
-        reinterpret_cast<float*>(rep)[i] = grid[P == 2 ? 2 * (i >> 5) + (i & 1) : (i >> 5)];
+        reinterpret_cast<float*>(rep)[i] = -grid[P == 2 ? 2 * (i >> 5) + (i & 1) : (i >> 5)];
     __syncthreads();
 
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const uint8_t* rep_lane = rep + (P == 2 ? (lane & 15) * 8 : lane * 4);
-    const int64_t groups = K / kGroup, kblocks = K / kBlockK;
-    const int64_t turns = (N / 16) * groups;
-    const float inv_w = CELLS / (2.0f * kCellR);
-    const float magic = 8388608.0f + 0.5f * CELLS;
-    // (row tile, group) of the block's turn, advanced by the grid's stride without a division per turn
-    int64_t rt = (int64_t)blockIdx.x / groups, gi = (int64_t)blockIdx.x % groups;
-    const int64_t step_tiles = (int64_t)gridDim.x / groups, step_groups = (int64_t)gridDim.x % groups;
-    int parity = 0;                  // tile of this turn
-    int64_t prev_rt = -1, prev_gi = 0;
-    for (int64_t turn = blockIdx.x; turn < turns; turn += gridDim.x, rt += step_tiles, gi += step_groups, parity ^= 1) {
+    const uint32_t cells_at = enc_smem_u32(cells), rep_lane = enc_smem_u32(rep) + (P == 2 ? (lane & 15) * 8 : lane * 4);
+    // (32-bit work items: 2^31 turns would be 2^45 weights)
+    const int groups = (int)(K / kGroup), turns = (int)(N / 16) * groups, stride = 2 * (int)gridDim.x;
+    const float cell_mul = (CELLS / (2.0f * kCellR)) / (CELLS - 1), cell_add = 0.5f * CELLS / (CELLS - 1);
+    // (row tile, group) of the half's turn, advanced by the grid's stride without a division per turn
+    const int first = 2 * (int)blockIdx.x + half;
+    int rt = first / groups, gi = first % groups;
+    const int step_tiles = stride / groups, step_groups = stride % groups;
+    const int pack_pad = (wib >> 2) * (enc_run(P) - 256 / P);       // this warp packs 64-input block wib of the tile
+    int tile = 0;                    // tile of this turn
+    int sign_gi = -1;            // group whose sign bits are in `sign`
+    uint32_t sign = 0u;
+    uint32_t phase = 0;              // parity of this turn's arrivals
+    int prev_rt = -1, prev_gi = 0;
+    for (int turn = first; turn < turns; turn += stride, rt += step_tiles, gi += step_groups) {
         if (gi >= groups) { gi -= groups; ++rt; }
-        const int64_t row = rt * 16 + wib;
-        float v[32];
-        load32<T>(W + row * K + gi * kGroup, lane, v);
-        float ss = 0.0f;
+        const int64_t row = (int64_t)rt * 16 + wib;
+        uint64_t q[16];
+        {
+            RawGroup<T> raw;
+            raw.load(W + row * K + (int64_t)gi * kGroup, lane);
+            if (turn + stride < turns) {                   // the next turn's row on its way into L2
+                int nr = rt + step_tiles, ng = gi + step_groups;
+                if (ng >= groups) { ng -= groups; ++nr; }
+                if (lane * 128 < kGroup * (int)sizeof(T))
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const uint8_t*>(W + ((int64_t)nr * 16 + wib) * K + (int64_t)ng * kGroup) + lane * 128));
+            }
+            if (gi != sign_gi) { sign = lane_sign_bits(xi, (int64_t)gi * kGroup, lane); sign_gi = gi; }
+            float ss = 0.0f;
 #pragma unroll
-        for (int r = 0; r < 32; ++r) ss = fmaf(v[r], v[r], ss);
+            for (int t = 0; t < 16; ++t) {
+                float a, b;
+                raw.get_signed(t, sign, a, b);
+                ss = fmaf(b, b, fmaf(a, a, ss));
+                q[t] = pair_of(a, b);
+            }
 #pragma unroll
-        for (int m = 16; m >= 1; m >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, m);
-        const float s = sqrtf(ss);
-        const float inv = s > 0.0f ? 1.0f / s : 0.0f;
+            for (int m = 16; m >= 1; m >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, m);
+            const float s = sqrtf(ss);
+            const float inv = s > 0.0f ? 1.0f / s : 0.0f;
+            if (lane == 0) scales[((int64_t)rt * groups + gi) * 16 + wib] = __float2half_rn(s * 0.03125f);
+            const uint64_t inv2 = pair_of(inv, inv);
 #pragma unroll
-        for (int r = 0; r < 32; ++r) v[r] *= inv;
-        apply_signs1024(v, xi, gi * kGroup, lane);
-        fwht1024_warp(v, lane);
-        if (lane == 0) scales[(rt * groups + gi) * 16 + wib] = __float2half_rn(s * 0.03125f);
+            for (int t = 0; t < 16; ++t) {
+                float a, b;
+                unpair(mul2(q[t], inv2), a, b);
+                q[t] = pair_of(a + b, a - b);              // the stage of bit 0
+            }
+        }
+        encoder_transform(q, ex, lane);
 
-        uint32_t out[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};      // the lane's codes, one byte each, in storage order
+        // this warp's row: code of tuple t of the lane
+        uint8_t* const mine = tiles_base + tile * (16 * RS) + wib * RS + (lane >> 3) * enc_run(P) + (encoder_element(lane) & 255) / P;
         uint32_t slow = 0u;                                       // bit t: tuple t needs the exhaustive scan
 #pragma unroll
         for (int t = 0; t < 32 / P; ++t) {
-            const float x = v[P * t], y = P == 2 ? v[2 * t + 1] : 0.f;
-            // the float 2^23 + i carries i in its low bits; anything else (outside the table, NaN) leaves other bits set
-            const uint32_t ix = __float_as_uint(fmaf(x, inv_w, magic)) ^ 0x4B000000u;
-            const uint32_t iy = P == 2 ? __float_as_uint(fmaf(y, inv_w, magic)) ^ 0x4B000000u : 0u;
-            const bool inside = (ix | iy) < (uint32_t)CELLS;
-            uint32_t list = kCellScan;
-            if (inside) list = cells[P == 2 ? iy * kCells2 + ix : ix];
-            if (list == kCellScan) { slow |= 1u << t; list = 0u; }
+            float x, y;
+            unpair(q[P == 2 ? t : t >> 1], x, y);
+            if (P == 1 && (t & 1)) x = y;
+            const uint32_t ix = __float_as_uint(fmaf(__saturatef(fmaf(x, cell_mul, cell_add)), (float)(CELLS - 1), 8388608.0f));
+            uint32_t at = cells_at + ix * 4u - 0x4B000000u * 4u;
+            if (P == 2) {
+                const uint32_t iy = __float_as_uint(fmaf(__saturatef(fmaf(y, cell_mul, cell_add)), (float)(CELLS - 1), 8388608.0f));
+                at += iy * (uint32_t)(4 * CELLS) - 0x4B000000u * (uint32_t)(4 * CELLS);
+            }
+            uint32_t list;
+            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(list) : "r"(at));
+            if (list == kCellScan) slow |= 1u << t;
             float best;
             uint32_t b;
 #pragma unroll
@@ -447,16 +593,20 @@ __global__ void __launch_bounds__(512, 2) encode_pruned_kernel(const T* __restri
                 const uint32_t c = __byte_perm(list, 0u, 0x4440u + i);
                 float d;
                 if (P == 2) {
-                    const float2 g = *reinterpret_cast<const float2*>(rep_lane + c * 128u);
-                    const float dx = x - g.x, dy = y - g.y;
+                    uint64_t g;
+                    asm volatile("ld.shared.b64 %0, [%1];" : "=l"(g) : "r"(rep_lane + c * 128u));
+                    float dx, dy;
+                    unpair(add2(q[t], g), dx, dy);
                     d = fmaf(dy, dy, dx * dx);
                 } else {
-                    const float dx = x - *reinterpret_cast<const float*>(rep_lane + c * 128u);
+                    float g;
+                    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(g) : "r"(rep_lane + c * 128u));
+                    const float dx = x + g;
                     d = dx * dx;
                 }
                 if (i == 0 || d < best) { best = d; b = c; }
             }
-            out[t >> 2] |= b << (8 * (t & 3));
+            mine[P == 2 ? 8 * t : 16 * (t >> 1) + (t & 1)] = (uint8_t)b;
         }
         if (__any_sync(0xffffffffu, slow != 0u)) {
 #pragma unroll
@@ -465,48 +615,45 @@ __global__ void __launch_bounds__(512, 2) encode_pruned_kernel(const T* __restri
                 while (m) {
                     const int src = __ffs(m) - 1;
                     m &= m - 1;
-                    const float px = __shfl_sync(0xffffffffu, v[P * t], src);
-                    const float py = P == 2 ? __shfl_sync(0xffffffffu, v[2 * t + 1], src) : 0.f;
+                    float x, y;
+                    unpair(q[P == 2 ? t : t >> 1], x, y);
+                    const float px = __shfl_sync(0xffffffffu, P == 1 && (t & 1) ? y : x, src);
+                    const float py = P == 2 ? __shfl_sync(0xffffffffu, y, src) : 0.f;
                     const int bc = warp_scan<P>(rep, n, px, py, lane);
-                    if (lane == src) out[t >> 2] = (out[t >> 2] & ~(0xffu << (8 * (t & 3)))) | ((uint32_t)bc << (8 * (t & 3)));
+                    if (lane == src) mine[P == 2 ? 8 * t : 16 * (t >> 1) + (t & 1)] = (uint8_t)bc;
                 }
             }
         }
-        // tuple t of chunk c sits at tuple index c*128 + lane*4 + (t&3) (p = 2: four consecutive bytes per chunk);
-        // value t of chunk c at c*256 + lane*8 + t (p = 1: eight)
+        __syncwarp();
         if (canonical) {
-            if (P == 2) {
-                uint8_t* dst = canonical + row * (K / 2) + gi * (kGroup / 2);
+            const uint8_t* codes = tiles_base + tile * (16 * RS) + wib * RS;
+            uint8_t* dst = canonical + row * (K / P) + (int64_t)gi * (kGroup / P);
 #pragma unroll
-                for (int c = 0; c < 4; ++c) *reinterpret_cast<uint32_t*>(dst + c * 128 + lane * 4) = out[c];
-            } else {
-                uint8_t* dst = canonical + row * K + gi * kGroup;
-#pragma unroll
-                for (int c = 0; c < 4; ++c) *reinterpret_cast<uint2*>(dst + c * 256 + lane * 8) = make_uint2(out[2 * c], out[2 * c + 1]);
+            for (int c = 0; c < 2 / P; ++c) {
+                const int at = (c * 32 + lane) * 16;
+                const uint8_t* from = codes + at + at / (256 / P) * (enc_run(P) - 256 / P);
+                const uint2 lo = *reinterpret_cast<const uint2*>(from), hi = *reinterpret_cast<const uint2*>(from + 8);
+                *reinterpret_cast<uint4*>(dst + at) = make_uint4(lo.x, lo.y, hi.x, hi.y);
             }
         }
         if (packed) {
             if (prev_rt >= 0) {      // the tile of the turn before: complete once all sixteen warps have arrived
-                enc_mbar_wait(bar, (uint32_t)(parity ^ 1));
-                pack_item<P>(tiles_base + (parity ^ 1) * (16 * RS), RS, fmt, bits, wib, lane, prev_rt, prev_gi * 16 + wib, kblocks, packed);
+                enc_mbar_wait(bar, phase ^ 1u);
+                pack_item<P>(tiles_base + (tile == 0 ? kEncTiles - 1 : tile - 1) * (16 * RS) + pack_pad, RS, fmt, bits, wib, lane, prev_rt,
+                             prev_gi * 16 + wib, groups * (kGroup / kBlockK), packed);
+                __syncwarp();
             }
-            uint8_t* mine = tiles_base + parity * (16 * RS) + wib * RS;
-            if (P == 2) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) *reinterpret_cast<uint32_t*>(mine + c * 128 + lane * 4) = out[c];
-            } else {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) *reinterpret_cast<uint2*>(mine + c * 256 + lane * 8) = make_uint2(out[2 * c], out[2 * c + 1]);
-            }
-            __syncwarp();
             if (lane == 0) enc_mbar_arrive(bar);
             prev_rt = rt;
             prev_gi = gi;
+            phase ^= 1u;
         }
+        tile = tile == kEncTiles - 1 ? 0 : tile + 1;
     }
     if (packed && prev_rt >= 0) {
-        enc_mbar_wait(bar, (uint32_t)(parity ^ 1));
-        pack_item<P>(tiles_base + (parity ^ 1) * (16 * RS), RS, fmt, bits, wib, lane, prev_rt, prev_gi * 16 + wib, kblocks, packed);
+        enc_mbar_wait(bar, phase ^ 1u);
+        pack_item<P>(tiles_base + (tile == 0 ? kEncTiles - 1 : tile - 1) * (16 * RS) + pack_pad, RS, fmt, bits, wib, lane, prev_rt, prev_gi * 16 + wib,
+                     groups * (kGroup / kBlockK), packed);
     }
 }
 
@@ -634,7 +781,7 @@ int launch_encode(const higgs_desc& d, const void* W, int w_dtype, const float* 
     }
     static int configured[64];
     const int ok = device_once(configured, [] {
-        constexpr int kMax = kCells2 * kCells2 * 4 + 256 * 128 + 2 * 16 * kTileRowBytes(1) + 16;
+        constexpr int kMax = (int)(encode_smem(1, 256) > encode_smem(2, 256) ? encode_smem(1, 256) : encode_smem(2, 256));
         bool good = true;
         good = good && cudaFuncSetAttribute(encode_pruned_kernel<float, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax) == cudaSuccess;
         good = good && cudaFuncSetAttribute(encode_pruned_kernel<float, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax) == cudaSuccess;
@@ -650,18 +797,14 @@ int launch_encode(const higgs_desc& d, const void* W, int w_dtype, const float* 
     }
     const uint32_t* tab = static_cast<const uint32_t*>(table);
     uint32_t* pk = static_cast<uint32_t*>(packed);
-    const size_t smem = encoder_table_bytes(d.p) + (size_t)d.n * 128 + 2 * 16 * (size_t)kTileRowBytes(d.p) + 16;
+    const size_t smem = encode_smem(d.p, d.n);
     const int64_t turns = (d.N / 16) * (d.K / kGroup);
     const int fmt = (int)format_of(d.p, d.n) - 1, bits = code_bits(d.n);
-    // persistent grid: as many blocks as are resident at once (two of 16 warps per SM); any count is correct
+    // persistent grid: one block per SM, two turns at a time; any count is correct
+    const int64_t resident = sm_count();
+    const unsigned blocks = (unsigned)((turns + 1) / 2 < resident ? (turns + 1) / 2 : resident);
 #define HIGGS_ENC(T, P) \
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, encode_pruned_kernel<T, P>, 512, smem) != cudaSuccess || per_sm < 1) per_sm = 1; \
-    resident = (int64_t)per_sm * sm_count(); \
-    blocks = (unsigned)(turns < resident ? turns : resident); \
-    encode_pruned_kernel<T, P><<<blocks, 512, smem, st>>>(static_cast<const T*>(W), grid, d.n, tab, canonical, pk, fmt, bits, sc, d.N, d.K, d.rht_seed)
-    int per_sm = 0;
-    int64_t resident = 0;
-    unsigned blocks = 0;
+    encode_pruned_kernel<T, P><<<blocks, kEncThreads, smem, st>>>(static_cast<const T*>(W), grid, d.n, tab, canonical, pk, fmt, bits, sc, d.N, d.K, d.rht_seed)
     if (w_dtype == HIGGS_F32 && d.p == 2) { HIGGS_ENC(float, 2); }
     else if (w_dtype == HIGGS_F32 && d.p == 1) { HIGGS_ENC(float, 1); }
     else if (w_dtype == HIGGS_BF16 && d.p == 2) { HIGGS_ENC(__nv_bfloat16, 2); }
