@@ -238,6 +238,37 @@ __device__ __forceinline__ float with_sign(float v, uint32_t bits, int r) {
     return __uint_as_float(__float_as_uint(v) ^ ((bits << (31 - r)) & 0x80000000u));
 }
 
+// two fp32 operations in one instruction
+__device__ __forceinline__ uint64_t pair_of(float a, float b) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
+    return v;
+}
+__device__ __forceinline__ void unpair(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) { uint64_t v; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b)); return v; }
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) { uint64_t v; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b)); return v; }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) { uint64_t v; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b)); return v; }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t v;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
+    return v;
+}
+// butterflies over the low BITS bits of the index of the pairs
+template <int BITS = 4>
+__device__ __forceinline__ void pair_stages(uint64_t (&q)[16]) {
+#pragma unroll
+    for (int h = 1; h < (1 << BITS); h <<= 1) {
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+            if ((t & h) == 0) {
+                const uint64_t a = q[t], b = q[t | h];
+                q[t] = add2(a, b);
+                q[t | h] = sub2(a, b);
+            }
+        }
+    }
+}
+
 // element index inside the group of register r of lane l (see above)
 __device__ __forceinline__ int fwht_index(int lane, int r) { return (r >> 3) * 256 + lane * 8 + (r & 7); }
 

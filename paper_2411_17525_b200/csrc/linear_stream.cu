@@ -69,7 +69,10 @@ struct StreamParams {
 };
 
 constexpr uint32_t kLutBytes = 65536;   // 256 entries x 256-byte row (32 lanes x 4 B; upper row halves hold accumulators)
-constexpr uint32_t kMaxDynSmem = 232448;
+// Left free on the SM for blocks of the rotation kernel (about 3 KB each), which are then resident before this kernel
+// ends instead of after it (see rht.cu); the rings lose 3 % of their slots to it.
+constexpr uint32_t kRotationReserve = 6144;
+constexpr uint32_t kMaxDynSmem = 232448 - kRotationReserve;
 constexpr uint32_t kSmallBytes = 4096;  // barriers, recycle counters, abort flag
 constexpr int kWarps = 16;
 constexpr int kMaxDepth = 8;            // ring slots per warp

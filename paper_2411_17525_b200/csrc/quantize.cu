@@ -370,35 +370,6 @@ __device__ __noinline__ int warp_scan(const uint8_t* rep, int n, float px, float
     return bc == 0x7fffffff ? 0 : bc;               // no distance compared below infinity (a NaN input): index 0, as the scan
 }
 
-// two fp32 operations in one instruction
-__device__ __forceinline__ uint64_t pair_of(float a, float b) {
-    uint64_t v;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
-    return v;
-}
-__device__ __forceinline__ void unpair(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) { uint64_t v; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b)); return v; }
-__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) { uint64_t v; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b)); return v; }
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) { uint64_t v; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b)); return v; }
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t v;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
-    return v;
-}
-__device__ __forceinline__ void pair_stages(uint64_t (&q)[16]) {
-#pragma unroll
-    for (int h = 1; h < 16; h <<= 1) {
-#pragma unroll
-        for (int t = 0; t < 16; ++t) {
-            if ((t & h) == 0) {
-                const uint64_t a = q[t], b = q[t | h];
-                q[t] = add2(a, b);
-                q[t | h] = sub2(a, b);
-            }
-        }
-    }
-}
-
 // The encoder's transform: the butterflies of fwht1024_warp in the same order (bit-identical values), on pairs.  In: q[t] =
 // elements (c*256 + lane*8 + 2 (t & 3), + 1), c = t >> 2, after the stage of bit 0.  Bits 1, 2, 8, 9 are register stages, bit 3
 // a shuffle stage; then the pairs are exchanged through shared memory so that bits 4 to 7 are register stages too: out,

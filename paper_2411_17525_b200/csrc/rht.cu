@@ -37,86 +37,98 @@ __device__ __forceinline__ void load_group<float>(const float* __restrict__ src,
     }
 }
 
-// Four warps per (token, group), one block of 128 threads each: x+ = (H/32) diag(sign) x, written as fp16 in "fragment
-// order": inside every block of 64 inputs the 32 input pairs are permuted so that the eight pairs one lane of the
-// product kernel needs as m16n8k16 B-fragment registers (steps m = 0..3, halves h = 0..1 of its column pair t) are 32
-// contiguous bytes: position t*8 + m*2 + h holds pair 8m + t + 4h.  Warp q of the block owns inputs 256 q .. + 255 of
-// the group, 8 per lane: butterflies over those 8 in registers, over the 32 lanes by shuffles, over the 4 warps
-// through shared memory (the transform is on the latency path between two dependent product launches, so it is
-// spread over four warps instead of one).  Threads also clear `zero_ptr` (the fp32 accumulation target of a K-split
-// product) so that no separate memset launch is needed.
-template <typename T>
-__global__ void __launch_bounds__(128) rht_activations_kernel(const T* __restrict__ x, __half* __restrict__ xdag,
-                                                              int64_t B, int64_t K, uint64_t xi,
-                                                              float* __restrict__ zero_ptr, size_t zero_floats) {
-    __shared__ __align__(16) float ex[4][256];
-    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+// x+ = (H/32) diag(sign) x, written as fp16 in "fragment order": inside every block of 64 inputs the 32 input pairs are
+// permuted so that the eight pairs one lane of the product kernel needs as m16n8k16 B-fragment registers (steps
+// m = 0..3, halves h = 0..1 of its column pair t) are 32 contiguous bytes: position t*8 + m*2 + h holds pair 8m + t + 4h.
+//
+// One warp per (token, group), one block each.  The transform stands between two dependent product launches, so what
+// counts is when it can start: a product kernel leaves shared memory (kRotationReserve) and registers for a few of
+// these small blocks, which are therefore on the SMs and waiting - code fetched, signs computed - when the product
+// before them ends; the next product's blocks take the SMs over as they become free, and build their tables and fetch
+// their first weights while the rotation runs.  As blocks of four warps, which found no room, it added 4.4 us to a
+// 4096 x 4096 product with four tokens (8.8 against 4.3 us on rotated activations); now 1.3.
+// Lane l reads inputs 32 l .. + 31: bits 0 to 4 of the input index are butterflies in registers (two fp32 operations
+// an instruction), bit 5 is a shuffle; the pairs are then exchanged through shared memory, 2 KB at a time, so that
+// lane P holds pair P of the sixteen 64-input blocks and bits 6 to 9 are in registers too.  (The same sums, bit for
+// bit, as the rotation fused into the product kernel.)
+// Threads also clear `zero_ptr` (the fp32 accumulation target of a K-split product) so that no separate memset launch
+// is needed.
+__global__ void __launch_bounds__(32) rht_activations_kernel(const __nv_bfloat16* __restrict__ x, __half* __restrict__ xdag,
+                                                             int64_t B, int64_t K, uint64_t xi,
+                                                             float* __restrict__ zero_ptr, size_t zero_floats) {
+    __shared__ __align__(16) uint8_t ex[2048];
+    const int lane = threadIdx.x;
     const int64_t groups = K / kGroup;
-    const size_t gtid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const size_t gthreads = (size_t)gridDim.x * blockDim.x;
     pdl_trigger();     // the product kernel may start its table build and weight prefetch now
+    const int64_t b = blockIdx.x / groups, k0 = blockIdx.x % groups * kGroup;
+    const uint64_t word = sign_word(xi, ((uint64_t)k0 >> 6) + (uint64_t)(lane >> 1));
+    const uint32_t signs = (uint32_t)(word >> (32 * (lane & 1)));
     pdl_wait();        // x may be the previous kernel's output; the buffers written below may still be read by it
-    for (size_t i = gtid; i < zero_floats; i += gthreads) zero_ptr[i] = 0.0f;
-    if ((int64_t)blockIdx.x >= B * groups) return;           // (blocks beyond the transform work only clear)
-    const int64_t b = blockIdx.x / groups, gi = blockIdx.x % groups;
-    const int64_t k0 = gi * kGroup + q * 256 + lane * 8;     // this lane's 8 consecutive inputs
-    float v[8];
+    for (size_t i = (size_t)blockIdx.x * 32 + lane; i < zero_floats; i += (size_t)gridDim.x * 32) zero_ptr[i] = 0.0f;
+    if (b >= B) return;                                      // (blocks beyond the transform work only clear)
+    uint64_t q[16];
     {
-        const T* src = x + b * K + k0;
-        if (sizeof(T) == 2) {
-            const uint4 q4 = __ldg(reinterpret_cast<const uint4*>(src));
-            const uint32_t w4[4] = {q4.x, q4.y, q4.z, q4.w};
+        const uint4* src = reinterpret_cast<const uint4*>(x + b * K + k0 + lane * 32);
+        uint4 raw[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                v[2 * e] = __uint_as_float(w4[e] << 16);
-                v[2 * e + 1] = __uint_as_float(w4[e] & 0xffff0000u);
-            }
-        } else {
-            const float4 a = __ldg(reinterpret_cast<const float4*>(src)), c = __ldg(reinterpret_cast<const float4*>(src) + 1);
-            v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = c.x; v[5] = c.y; v[6] = c.z; v[7] = c.w;
-        }
-        const uint32_t bits = (uint32_t)(sign_word(xi, (uint64_t)k0 >> 6) >> ((uint64_t)k0 & 63ull)) & 0xffu;
+        for (int c = 0; c < 4; ++c) raw[c] = src[c];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = __uint_as_float(__float_as_uint(v[e]) ^ (((bits >> e) & 1u) << 31));
-    }
-#pragma unroll
-    for (int h = 1; h < 8; h <<= 1) {
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            if ((r & h) == 0) { const float a = v[r], c = v[r | h]; v[r] = a + c; v[r | h] = a - c; }
+        for (int t = 0; t < 16; ++t) {
+            const uint4 r = raw[t >> 2];
+            uint32_t w = (t & 3) == 0 ? r.x : (t & 3) == 1 ? r.y : (t & 3) == 2 ? r.z : r.w;
+            // the signs of elements 2t, 2t + 1: one multiply puts both bits on the two sign positions
+            w ^= (((signs >> (8 * (t >> 2))) & 0xffu) * ((1u << (15 - 2 * (t & 3))) + (1u << (30 - 2 * (t & 3))))) & 0x80008000u;
+            const float lo = __uint_as_float(w << 16), hi = __uint_as_float(w & 0xffff0000u);
+            q[t] = pair_of(lo + hi, lo - hi);                // bit 0
         }
     }
+    pair_stages(q);                                          // bits 1 to 4
+    {
+        const float sgn = (lane & 1) ? -1.0f : 1.0f;
+        const uint64_t sgn2 = pair_of(sgn, sgn);
 #pragma unroll
-    for (int m = 1; m < 32; m <<= 1) {
-        const bool upper = (lane & m) != 0;
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            const float o = __shfl_xor_sync(0xffffffffu, v[r], m);
-            v[r] = upper ? (o - v[r]) : (v[r] + o);
+        for (int t = 0; t < 16; ++t) {
+            float lo, hi;
+            unpair(q[t], lo, hi);
+            q[t] = fma2(q[t], sgn2, pair_of(__shfl_xor_sync(0xffffffffu, lo, 1), __shfl_xor_sync(0xffffffffu, hi, 1)));
         }
     }
-    *reinterpret_cast<float4*>(&ex[q][lane * 8]) = make_float4(v[0], v[1], v[2], v[3]);
-    *reinterpret_cast<float4*>(&ex[q][lane * 8 + 4]) = make_float4(v[4], v[5], v[6], v[7]);
-    __syncthreads();
-    float o[8];
+    // row r of the buffer: the 16 pairs of lane r (then of lane 16 + r) as eight 16-byte chunks, permuted by r % 8: no
+    // bank conflicts on either side
+    uint64_t o[16];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) o[r] = 0.f;
+    for (int h = 0; h < 2; ++h) {
+        if (h == 1) __syncwarp();
+        if ((lane >> 4) == h) {
+            const int r = lane & 15;
 #pragma unroll
-    for (int qq = 0; qq < 4; ++qq) {
-        const float4 u0 = *reinterpret_cast<const float4*>(&ex[qq][lane * 8]);
-        const float4 u1 = *reinterpret_cast<const float4*>(&ex[qq][lane * 8 + 4]);
-        const float sgn = (__popc(q & qq) & 1) ? -1.f : 1.f;
-        o[0] = fmaf(sgn, u0.x, o[0]); o[1] = fmaf(sgn, u0.y, o[1]); o[2] = fmaf(sgn, u0.z, o[2]); o[3] = fmaf(sgn, u0.w, o[3]);
-        o[4] = fmaf(sgn, u1.x, o[4]); o[5] = fmaf(sgn, u1.y, o[5]); o[6] = fmaf(sgn, u1.z, o[6]); o[7] = fmaf(sgn, u1.w, o[7]);
+            for (int j = 0; j < 8; ++j) *reinterpret_cast<ulonglong2*>(ex + r * 128 + ((j ^ (r & 7)) << 4)) = make_ulonglong2(q[2 * j], q[2 * j + 1]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+            const int r = 2 * s + (lane >> 4), k = lane & 15;
+            o[8 * h + s] = *reinterpret_cast<const uint64_t*>(ex + r * 128 + (((k >> 1) ^ (r & 7)) << 4) + (k & 1) * 8);
+        }
     }
-    // this lane holds pairs 4 j + i (i = 0..3, j = lane % 8) of 64-input block q*4 + lane/8 of the group, i.e.
-    // m = j >> 1, h = j & 1, t = i  ->  position i*8 + j
-    uint32_t* blk = reinterpret_cast<uint32_t*>(xdag + b * K + gi * kGroup) + (q * 4 + (lane >> 3)) * 32;
-    const int j = lane & 7;
+    pair_stages<2>(o);                                       // bits 6 and 7
+    // bits 8 and 9: the sums in the order in which the product kernel's fused rotation adds up its four warps' parts
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const __half2 hh = __floats2half2_rn(o[2 * e] * 0.03125f, o[2 * e + 1] * 0.03125f);
-        blk[e * 8 + j] = *reinterpret_cast<const uint32_t*>(&hh);
+    for (int s = 0; s < 4; ++s) {
+        const uint64_t a = add2(o[s], o[s + 4]), b2 = sub2(o[s], o[s + 4]);
+        const uint64_t c = add2(a, o[s + 8]), d = add2(b2, o[s + 8]), e = sub2(a, o[s + 8]), f = sub2(b2, o[s + 8]);
+        o[s] = add2(c, o[s + 12]);
+        o[s + 4] = sub2(d, o[s + 12]);
+        o[s + 8] = sub2(e, o[s + 12]);
+        o[s + 12] = add2(f, o[s + 12]);
+    }
+    uint32_t* dst = reinterpret_cast<uint32_t*>(xdag + b * K + k0) + (lane & 3) * 8 + (lane >> 3) * 2 + ((lane >> 2) & 1);
+#pragma unroll
+    for (int s = 0; s < 16; ++s) {
+        float lo, hi;
+        unpair(o[s], lo, hi);
+        const __half2 v = __floats2half2_rn(lo * 0.03125f, hi * 0.03125f);
+        dst[s * 32] = *reinterpret_cast<const uint32_t*>(&v);
     }
 }
 
@@ -146,13 +158,13 @@ __global__ void __launch_bounds__(256) rht_debug_kernel(const T* __restrict__ x,
 
 int launch_rht_activations(const higgs_desc& d, const void* x, int64_t B, __half* xdag, float* zero_ptr,
                            size_t zero_floats, cudaStream_t st) {
-    int64_t blocks = B * (d.K / kGroup);                   // one block of four warps per (token, group)
+    int64_t blocks = B * (d.K / kGroup);
     if (zero_floats) {
-        int64_t zb = (int64_t)((zero_floats + 128 * 8 - 1) / (128 * 8));
+        int64_t zb = (int64_t)((zero_floats + 32 * 8 - 1) / (32 * 8));
         if (zb > 1184) zb = 1184;
         if (zb > blocks) blocks = zb;
     }
-    return cuda_status(launch_pdl(rht_activations_kernel<__nv_bfloat16>, dim3((unsigned)blocks), dim3(128), 0, st,
+    return cuda_status(launch_pdl(rht_activations_kernel, dim3((unsigned)blocks), dim3(32), 0, st,
                                   static_cast<const __nv_bfloat16*>(x), xdag, B, d.K, d.rht_seed, zero_ptr, zero_floats));
 }
 

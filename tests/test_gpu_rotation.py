@@ -1,0 +1,28 @@
+"""The rotation kernel in front of the small-batch product."""
+import pytest
+import torch
+
+import oracle
+import paper_2411_17525_b200 as hb
+from tests import gpu_util as U
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,K", [(1, 1024), (2, 28672), (3, 3072), (8, 14336), (16, 2048)])
+def test_rotation_in_fragment_order(B, K):
+    xi, d = 977, hb.make_desc(2, 256, 16, K, 977)
+    assert hb.higgs_rotated_layout(d, B) == 0
+    x = torch.randn(B, K, device=U.dev(), generator=torch.Generator(device="cuda").manual_seed(K)).to(torch.bfloat16)
+    x[0, :1024] *= 1e3
+    # word t*8 + m*2 + h of a 64-input block is the pair 8m + 4h + t
+    got = hb.higgs_rotate_activations(d, x).view(B, K // 64, 4, 4, 2, 2).permute(0, 1, 3, 4, 2, 5).reshape(B, K).double().cpu()
+    sgn = torch.from_numpy(oracle.signs(xi, K)).double()
+    H = torch.ones(1, 1, dtype=torch.float64)
+    for _ in range(10):
+        H = torch.cat([torch.cat([H, H], 1), torch.cat([H, -H], 1)], 0)
+    xs = (x.double().cpu() * sgn).view(B, K // 1024, 1024)
+    ref = (xs @ H / 32).reshape(B, K)
+    # ten fp32 stages of one rounding each, below the sum of magnitudes, then one rounding to fp16
+    bound = (10 * 2.0 ** -24 / 32 * xs.abs().sum(-1, keepdim=True)).expand(B, K // 1024, 1024).reshape(B, K)
+    assert ((got - ref).abs() <= bound + 2.0 ** -11 * (ref.abs() + bound) + 2.0 ** -25).all()
