@@ -221,6 +221,8 @@ int higgs_quantize_prepared(const higgs_desc* desc, const void* W, int w_dtype, 
  *   scales   device, tile-major fp16 scales as written by higgs_quantize
  *   grid     device, [n][p] fp32
  *   y        device, [B][N] row-major, y_dtype in {HIGGS_F32, HIGGS_BF16}
+ *   workspace  device, 256-byte aligned, higgs_workspace_bytes(desc, HIGGS_OP_LINEAR, B) bytes; may be NULL where
+ *            higgs_linear_launch_count(desc, B, y_dtype) is 1 (the one kernel needs none)
  * Kernels behind the call: for one or two tokens (K up to 8192) a single kernel
  * that rotates the activations in its prologue; up to 16 tokens a rotation
  * kernel and the small-batch product kernel; above that (and from 9 tokens

@@ -18,6 +18,9 @@ def __getattr__(name):
     if _BINDING is None:
         _BINDING = importlib.import_module(".binding", __name__)
     try:
-        return getattr(_BINDING, name)
+        value = getattr(_BINDING, name)
     except AttributeError:
         raise AttributeError(f"module {__name__!r} has no attribute {name!r}") from None
+    if callable(value):
+        globals()[name] = value          # found directly from now on (this hook takes 0.3 us)
+    return value

@@ -319,9 +319,10 @@ static int linear_args(const higgs_desc* d, int64_t B, const void* x, const void
     if (B < 0) return HIGGS_ERR_INVALID_ARG;
     if (B == 0 || d->N == 0) return -1;   // nothing to do
     if (d->K == 0) return HIGGS_ERR_UNSUPPORTED;
-    if (!x || !packed || !scales || !grid || !y || !workspace) return HIGGS_ERR_INVALID_ARG;
+    if (!x || !packed || !scales || !grid || !y) return HIGGS_ERR_INVALID_ARG;
     if (!aligned(x, 16) || !aligned(packed, 16) || !aligned(scales, 16) || !aligned(workspace, 256) || !aligned(y, 16))
         return HIGGS_ERR_INVALID_ARG;
+    if (!workspace) return !tc_eligible(*d, B) && linear_fused_eligible(*d, B) ? HIGGS_OK : HIGGS_ERR_INVALID_ARG;
     if (workspace_bytes < higgs_workspace_bytes(d, HIGGS_OP_LINEAR, B)) return HIGGS_ERR_WORKSPACE;
     return HIGGS_OK;
 }

@@ -67,14 +67,16 @@ inline int cuda_status(cudaError_t e) { return e == cudaSuccess ? HIGGS_OK : HIG
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // One-time set-up per device (function attributes, occupancy queries) that several host threads may reach at once:
-// `state[dev]` is read and written under one process-wide mutex.  Returns the stored value (0 = not yet set).
+// `state[dev]` is written under one process-wide mutex.  Returns the stored value (0 = not yet set).
 inline std::mutex& device_setup_mutex() { static std::mutex m; return m; }
 template <typename F>
 inline int device_once(int (&state)[64], F&& setup) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return setup();
+    const int known = __atomic_load_n(&state[dev], __ATOMIC_ACQUIRE);
+    if (known != 0) return known;
     std::lock_guard<std::mutex> lock(device_setup_mutex());
-    if (state[dev] == 0) state[dev] = setup();
+    if (state[dev] == 0) __atomic_store_n(&state[dev], setup(), __ATOMIC_RELEASE);
     return state[dev];
 }
 
