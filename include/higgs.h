@@ -223,8 +223,9 @@ int higgs_quantize_prepared(const higgs_desc* desc, const void* W, int w_dtype, 
  *   y        device, [B][N] row-major, y_dtype in {HIGGS_F32, HIGGS_BF16}
  *   workspace  device, 256-byte aligned, higgs_workspace_bytes(desc, HIGGS_OP_LINEAR, B) bytes; may be NULL where
  *            higgs_linear_launch_count(desc, B, y_dtype) is 1 (the one kernel needs none)
- * Kernels behind the call: for one or two tokens (K up to 8192) a single kernel
- * that rotates the activations in its prologue; up to 16 tokens a rotation
+ * Kernels behind the call: for one or two tokens and a small layer (K = 1024, or
+ * fewer than 2 M weights times tokens) a single kernel that rotates the
+ * activations in its prologue; else up to 16 tokens a rotation
  * kernel and the small-batch product kernel; above that (and from 9 tokens
  * for layers with at least 4096 rows, 4096 inputs and 16 M weights) a rotation kernel and the tcgen05 kernel.
  * When the small-batch kernel splits K over more than two thread blocks the
@@ -266,9 +267,9 @@ int higgs_linear_prerotated(const higgs_desc* desc, const void* xdag, int64_t B,
  * x (q before k and v; gate before up) - Section 4.3 notes that the transform of the activations can be isolated from
  * the product of Appendix F, so layers with a common input need it once: y as higgs_linear, and xdag_out (device, higgs_rotated_bytes(desc, B) bytes,
  * 16-byte aligned) receives what higgs_rotate_activations(desc, x, B) writes, to be passed to
- * higgs_linear_prerotated for the other layers (same K, seed and higgs_rotated_layout).  For one or two tokens on a
- * layer whose K is not split this is ONE launch - the product kernel rotates x itself and one of its blocks stores
- * the result - instead of a rotation launch followed by a product launch; otherwise it is those two launches.
+ * higgs_linear_prerotated for the other layers (same K, seed and higgs_rotated_layout).  Where higgs_linear is
+ * one launch this is too - the product kernel rotates x itself and one of its blocks stores the result - otherwise it
+ * is a rotation launch and a product launch.
  * xdag_out is complete when the call's last kernel has completed (stream order).
  */
 int higgs_linear_share(const higgs_desc* desc, const void* x, int64_t B, const void* packed, const void* scales,

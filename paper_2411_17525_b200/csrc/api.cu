@@ -340,7 +340,7 @@ int higgs_linear(const higgs_desc* d, const void* x, int64_t B, const void* pack
                                 y_dtype == HIGGS_F32 ? 0 : 1, st);
     }
     if (linear_fused_eligible(*d, B)) {
-        // one or two tokens, K not split: the product kernel rotates the activations itself (D1 fused into D2-D5)
+        // one or two tokens, a small layer: the product kernel rotates the activations itself (D1 fused into D2-D5)
         void* yo = y;
         return launch_linear_mma(*d, nullptr, B, packed, scales, grid, yo, d->N, y_dtype == HIGGS_F32 ? 0 : 1, st, x);
     }
@@ -369,6 +369,12 @@ int higgs_linear_share(const higgs_desc* d, const void* x, int64_t B, const void
     rc = higgs_rotate_activations(d, x, B, xdag_out, stream);
     if (rc != HIGGS_OK) return rc;
     return higgs_linear_prerotated(d, xdag_out, B, packed, scales, grid, y, y_dtype, workspace, workspace_bytes, stream);
+}
+
+// One launch for the concatenation `all` of one or two tokens: sets of up to 2048 rows keep it even where a rotation launch
+// of its own would be faster, because callers count on it.
+static bool multi_fused(const higgs_desc& all, int64_t B) {
+    return linear_fused_eligible(all, B) || (all.N <= 2048 && linear_fused_possible(all, B));
 }
 
 // Several matrices take the tensor-core path together when their concatenation does and every one fills whole 128-row
@@ -431,7 +437,7 @@ int higgs_linear_multi(int32_t count, const higgs_desc* const* descs, const void
     const int mode = y_dtype == HIGGS_F32 ? 0 : 1;
     if (segs.count > 1 && B <= 16 && !tc_eligible(v, B) && !linear_uses_atomics(v, B)) {
         // ONE launch of the small-batch kernel over the concatenated rows (per 16 tokens), the rotation done once
-        if (linear_fused_eligible(v, B))
+        if (multi_fused(v, B))
             return launch_linear_mma(v, nullptr, B, segs.packed[0], segs.scales[0], grid, segs.y[0], segs.rows[0], mode, st, x,
                                      nullptr, nullptr, &segs);
         __half* xdag = static_cast<__half*>(workspace);
@@ -477,7 +483,7 @@ int higgs_linear_multi_launch_count(int32_t count, const higgs_desc* const* desc
         separate += higgs_linear_launch_count(descs[i], B, y_dtype);
     }
     if (live > 1 && B <= 16 && !tc_eligible(v, B) && !linear_uses_atomics(v, B))
-        return linear_fused_eligible(v, B) ? 1 : 1 + (int)((B + 15) / 16);
+        return multi_fused(v, B) ? 1 : 1 + (int)((B + 15) / 16);
     if (multi_on_tc(live, rows, v, B)) return 2;
     return separate;
 }

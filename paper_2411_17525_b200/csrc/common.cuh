@@ -312,6 +312,7 @@ int launch_linear_mma(const higgs_desc& d, const __half* xdag, int64_t B, const 
                       const GatherTargets* more = nullptr, __half* xdag_emit = nullptr, const MultiSegments* segs = nullptr);
 int launch_scatter_out(const float* y32, int64_t B, int64_t N, void* const* dsts, int n_dst, int64_t ldy, int y_dtype,
                        cudaStream_t st);
+bool linear_fused_possible(const higgs_desc& d, int64_t B);
 bool linear_fused_eligible(const higgs_desc& d, int64_t B);
 int launch_convert_out(const float* y32, void* y, int y_dtype, size_t count, cudaStream_t st);
 size_t make_grid_workspace(int p, int n, int64_t m);

@@ -63,15 +63,19 @@ __global__ void __launch_bounds__(32) rht_activations_kernel(const __nv_bfloat16
     const int64_t b = blockIdx.x / groups, k0 = blockIdx.x % groups * kGroup;
     const uint64_t word = sign_word(xi, ((uint64_t)k0 >> 6) + (uint64_t)(lane >> 1));
     const uint32_t signs = (uint32_t)(word >> (32 * (lane & 1)));
+    const __nv_bfloat16* src = x + b * K + k0 + lane * 32;
+    if (b < B) {       // into L2 already now: a line the previous kernel is still going to write is written there
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(src));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(src + 16));
+    }
     pdl_wait();        // x may be the previous kernel's output; the buffers written below may still be read by it
     for (size_t i = (size_t)blockIdx.x * 32 + lane; i < zero_floats; i += (size_t)gridDim.x * 32) zero_ptr[i] = 0.0f;
     if (b >= B) return;                                      // (blocks beyond the transform work only clear)
     uint64_t q[16];
     {
-        const uint4* src = reinterpret_cast<const uint4*>(x + b * K + k0 + lane * 32);
         uint4 raw[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) raw[c] = src[c];
+        for (int c = 0; c < 4; ++c) raw[c] = reinterpret_cast<const uint4*>(src)[c];
 #pragma unroll
         for (int t = 0; t < 16; ++t) {
             const uint4 r = raw[t >> 2];
