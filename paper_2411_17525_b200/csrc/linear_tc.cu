@@ -3,9 +3,10 @@
 // Here the path is a dense contraction, so it runs as tcgen05.mma with the accumulator in tensor memory (TMEM).
 //
 // One block computes a 128-row x BN-token tile of y over a slice of K ("swap-AB": the weights are the M = 128 side).
-//   producer warps   stream, per 64 inputs, the codes of the 128 rows (8 bulk copies of 512 B, a deep ring: they
-//                    are the HBM stream) and, per 64/128/256 inputs, the tile of rotated activations (one bulk copy,
-//                    from L2) into shared memory (TMA, cp.async.bulk + mbarrier);
+//   producer warps   stream the codes of the 128 rows (one tiled TMA copy per 64 to 256 inputs: about 1 KB of each row
+//                    tile, because smaller ones leave the copy engine behind HBM) and, per 64/128/256 inputs, the tile of
+//                    rotated activations (one bulk copy, from L2) into shared memory; both rings are as deep as shared
+//                    memory allows: a copy takes about 1 us from HBM and hardly less from a busy L2;
 //   16 dequant warps each thread owns one row of the tile: it turns the row's 32 code bytes of a 64-input step into
 //                    table lookups (fp16 pairs), multiplies by the row's group scale and writes them with tcgen05.st
 //                    straight into the TMEM columns the MMA reads as its A operand - dequantisation is fused into
@@ -28,6 +29,8 @@
 
 #include <cuda.h>
 
+#include <algorithm>
+
 namespace higgs {
 
 __device__ int g_tc_status = 0;
@@ -46,6 +49,7 @@ struct TcParams {
     int64_t N, K, ldy;
     int B, BN, n, p, y_mode; // y_mode 0: fp32, 1: bf16
     int bits;                // log2(n)
+    int b_stages;            // activation-tile stages
     int ksplit;              // K slices (= cluster size along z); each a multiple of 256 inputs
     // Several matrices that read the same activations (q|k|v, gate|up) as one product over their concatenated rows:
     // matrix s holds the 128-row tiles [seg_tile[s], seg_tile[s + 1]).  nseg == 1: the fields above apply.
@@ -59,12 +63,13 @@ struct CodeMaps { CUtensorMap map[kMaxMulti]; };
 
 constexpr uint32_t kTcSmem = 232448;
 constexpr int kTcGroups = 4;                 // dequant warp groups (4 warps each, one per TMEM lane quadrant)
-constexpr int kTcBStages = 3;                // activation-tile stages in shared memory (at most 32 KB each)
+constexpr uint32_t kTcBBytes = 98304;        // activation-tile stages in shared memory (8 to 32 KB each) ...
+constexpr int kTcMaxBStages = 12;            // ... and at most so many
 constexpr int kTcMaxCodeStages = 32;         // code stages in shared memory (4 KB each), below and above the table
 constexpr int kTcDequantWarps = 4 * kTcGroups;
 constexpr int kTcThreads = (3 + kTcDequantWarps) * 32;
-// a code stage: byte formats 128 rows x 64 inputs (4 KB, one step); six-bit format 128 rows x 128 inputs (6 KB, two steps:
-// its three bit planes cover two neighbouring 64-input blocks)
+// What a deeper activation ring and larger code stages gave (16 tokens, byte format, chains): 28672x4096 34.4 -> 27.1 us,
+// 4096x14336 18.5 -> 15.1, 8192x28672 51.4 -> 44.2; with 3 activation stages neither the lookups nor the MMAs mattered.
 constexpr uint32_t kTcWait = 1u << 22;
 // TMEM columns: [0, BN) accumulator; A stages of 128 columns (256 inputs) from column 128 (BN <= 128: three stages)
 // or 256 (two stages).
@@ -117,12 +122,18 @@ __device__ __forceinline__ void t_bulk_load(uint32_t dst, const void* src, uint3
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                  "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
-// One tiled TMA copy: the box (64 x 8-byte elements = one 512-byte block, 8 row tiles) at element column x, row tile y
-// of the packed stream viewed as a 2-D tensor [N/16 row tiles][K x 8 bytes]; lands as [8][512 B] in shared memory.
-__device__ __forceinline__ void t_tensor_load(uint32_t dst, const CUtensorMap* map, int32_t x, int32_t y, uint32_t bar) {
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar) : "memory");
+// One tiled TMA copy: the box (one code stage: 256 to 1024 bytes of 8 row tiles) at 128-byte line `line` of row tile `tile`
+// of the packed stream viewed as a 3-D tensor [N/16 row tiles][lines][128 bytes]; lands as [8][lines][128 B] in shared
+// memory with the 16-byte chunks of a line permuted (128-byte swizzle: see code_swizzle).
+__device__ __forceinline__ void t_tensor_load(uint32_t dst, const CUtensorMap* map, int32_t line, int32_t tile, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(line), "r"(tile), "r"(bar) : "memory");
 }
+// Where byte o of a code stage (1 KB aligned) lies: chunk index xor line index.  A dequant warp's 16-byte loads, one row
+// per lane, are 64 (32) bytes apart and would meet in the banks four ways; swizzled they do not, and every lane gets its
+// chunks in order.  (Rotating the order of the loads per lane instead cost 100 of the 264 instructions a warp spent on 64
+// inputs, in moves.)
+__device__ __forceinline__ uint32_t code_swizzle(uint32_t o) { return o ^ (((o >> 7) & 7u) << 4); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
@@ -173,10 +184,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const __grid_c
 
     // ---- shared memory map ----
     //   [base, base+2 KB)    mbarriers, TMEM base address, abort flag
-    //   [base+2 KB, lut)     code stages, region A (4 KB each): deep, because the codes are the HBM stream
+    //   [base+2 KB, lut)     code stages, region A (8 or 12 KB each): deep, because the codes are the HBM stream
     //   [lut, lut+64 KB)     lookup table, 256-byte rows (bytes 0..127 = the entry replicated per lane)
-    //   [lut+64 KB, ...)     three activation-tile stages (FB x BN x 128 bytes each; they come from L2)
-    //   [..., end)           code stages, region B (whatever the activation stages leave: 52 KB for BN <= 128)
+    //   [lut+64 KB, ...)     activation-tile stages (FB x BN x 128 bytes each; they come from L2)
+    //   [..., end)           code stages, region B (whatever the activation stages leave)
     //   after the main loop: [base+2 KB, +BN x 512 B) the block's (partial) output tile, [token][row] fp32
     // Three rings: codes (freed when the four dequant warps of a step have read them), activation tiles and the
     // A operand in TMEM (both freed by tcgen05.commit when the MMAs that read them are done).
@@ -186,20 +197,23 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const __grid_c
     auto code_full = [&](int s) { return bars + 8u * (uint32_t)s; };
     auto code_empty = [&](int s) { return bars + 8u * (uint32_t)(32 + s); };
     auto b_full = [&](int s) { return bars + 8u * (uint32_t)(64 + s); };
-    auto b_free = [&](int s) { return bars + 8u * (uint32_t)(68 + s); };
-    auto a_full = [&](int s) { return bars + 8u * (uint32_t)(72 + s); };
-    auto a_free = [&](int s) { return bars + 8u * (uint32_t)(76 + s); };
-    const uint32_t d_full = bars + 8u * 80u;
+    auto b_free = [&](int s) { return bars + 8u * (uint32_t)(64 + kTcMaxBStages + s); };
+    auto a_full = [&](int s) { return bars + 8u * (uint32_t)(64 + 2 * kTcMaxBStages + s); };
+    auto a_free = [&](int s) { return bars + 8u * (uint32_t)(68 + 2 * kTcMaxBStages + s); };
+    const uint32_t d_full = bars + 8u * (uint32_t)(72 + 2 * kTcMaxBStages);
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_raw + 1024);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_raw + 1032);
     constexpr bool SIX = FMT == 1, NIB = FMT == 2, B8 = FMT == 3;
-    // bytes of the block's 128 rows in one code stage: 512 B per row tile and 64 inputs (byte format), 768 B per 128
-    // inputs (six-bit), 256 B (nibble), 1 KB (8-bit)
-    constexpr uint32_t kTcCodeStage = SIX ? 6144u : NIB ? 2048u : B8 ? 8192u : 4096u;
-    constexpr int SPS = SIX ? 2 : 1;                         // 64-input steps per code stage
+    // a row tile's bytes: 512 per 64 inputs (byte format), 768 per 128 inputs (six-bit: three bit planes of two
+    // neighbouring 64-input blocks), 256 per 64 (nibble), 1 KB per 64 (8-bit)
+    constexpr int SPS = SIX ? 4 : NIB ? 4 : B8 ? 1 : 2;    // 64-input steps per code stage
+    constexpr uint32_t kTcCodeStage = SPS * (SIX ? 3072u : NIB ? 2048u : B8 ? 8192u : 4096u);
+    constexpr uint32_t kTileStage = kTcCodeStage / 8u;       // bytes of a row tile in one stage
+    constexpr int kStageLines = (int)(kTcCodeStage / 1024u); // 128-byte lines of a row tile in one stage
     const uint32_t code0 = base + 2048u;
     const uint32_t b_stage_bytes = (uint32_t)FB * (uint32_t)prm.BN * 128u;
-    const uint32_t code1 = lut + 65536u + (uint32_t)kTcBStages * b_stage_bytes;      // region B
+    const int BS = prm.b_stages;
+    const uint32_t code1 = lut + 65536u + (uint32_t)BS * b_stage_bytes;              // region B
     int nA = (int)((lut - code0) / kTcCodeStage);
     if (nA > 16) nA = 16;
     int nB = (int)((base + kTcSmem - code1) / kTcCodeStage);
@@ -254,10 +268,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const __grid_c
             }
         }
     }
-    // The code ring needs one stage per warp group; the block's shared-memory window always leaves room for more, but
+    // The code ring needs one 64-input step per warp group; the block's shared-memory window always leaves room for more, but
     // a window that did not would be reported, not run.
     int role = warp;
-    if (CS < kTcGroups) role = -1;
+    if (CS * SPS < kTcGroups) role = -1;
     // (2) barriers, each ring by the warp that produces into it; the code producer starts the weight stream (which
     //     depends on nothing) before the block-wide barrier: the first CS stages need no wait.
     int code_issued = 0;
@@ -275,7 +289,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const __grid_c
             for (int j = 0; j < n0; ++j) {
                 if (elected) {
                     t_mbar_expect_tx(code_full(j), kTcCodeStage);
-                    t_tensor_load(code_stage(j), code_map, (kstep0 / SPS + j) * (int)(kTcCodeStage / 64u), tile0, code_full(j));
+                    t_tensor_load(code_stage(j), code_map, (kstep0 / SPS + j) * kStageLines, tile0, code_full(j));
                 }
                 __syncwarp();
             }
@@ -291,8 +305,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const __grid_c
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(base + 1024u), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     } else if (warp == 2) {
-        if (lane < 4) { t_mbar_init(b_full(lane), 1); t_mbar_init(b_free(lane), 1); }
-        if (lane == 4) {
+        if (lane < kTcMaxBStages) { t_mbar_init(b_full(lane), 1); t_mbar_init(b_free(lane), 1); }
+        if (lane == 31) {
             *abort_flag = 0;
             if (role < 0) { *abort_flag = 1; atomicExch(&g_tc_status, (int)HIGGS_ERR_TIMEOUT); }
         }
@@ -324,7 +338,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const __grid_c
             bad |= t_wait(code_empty(s), (uint32_t)((it & 1) ^ 1), t_limit(bad)) ^ 1u;
             if (elected) {
                 t_mbar_expect_tx(code_full(s), kTcCodeStage);
-                t_tensor_load(code_stage(s), code_map, (kstep0 / SPS + j) * (int)(kTcCodeStage / 64u), tile0, code_full(s));
+                t_tensor_load(code_stage(s), code_map, (kstep0 / SPS + j) * kStageLines, tile0, code_full(s));
             }
             ++issued;
             const bool wrap = s + 1 == CS;
@@ -352,13 +366,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const __grid_c
                 t_bulk_load(b_stage(s), xsrc + (int64_t)t * FB * BN * 64, bytes, b_full(s));
             }
             ++issued;
-            const bool wrap = s + 1 == kTcBStages;
+            const bool wrap = s + 1 == BS;
             s = wrap ? 0 : s + 1;
             it += wrap ? 1 : 0;
             __syncwarp();
         }
-        for (int t = issued > kTcBStages ? issued - kTcBStages : 0; t < issued; ++t)
-            bad |= t_wait(b_full(t % kTcBStages), (uint32_t)((t / kTcBStages) & 1), t_limit(bad)) ^ 1u;
+        for (int t = issued > BS ? issued - BS : 0; t < issued; ++t)
+            bad |= t_wait(b_full(t % BS), (uint32_t)((t / BS) & 1), t_limit(bad)) ^ 1u;
         t_report(bad, abort_flag);
     } else if (role == 1) {
         // =============================== MMA issuer ===============================
@@ -392,7 +406,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const __grid_c
                     if (h % FB == FB - 1) tc_commit(b_free(sb));      // arrives when the MMAs issued so far are done
                 }
                 if (h % FB == FB - 1) {
-                    const bool wrap = sb + 1 == kTcBStages;
+                    const bool wrap = sb + 1 == BS;
                     sb = wrap ? 0 : sb + 1;
                     ub += wrap ? 1 : 0;
                 }
@@ -414,37 +428,34 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const __grid_c
         const int rtl = i >> 4, g = i & 7, h = (i >> 3) & 1;
         const uint32_t lut_lane = lut + lane * 4;
         const uint32_t sel0 = 0x7604u + ((uint32_t)h << 4), sel1 = 0x7624u + ((uint32_t)h << 4);   // bytes h and h+2 of a word
-        const int rot = g >> 1;                    // chunk rotation that makes the 16-byte code loads conflict-free
         const int groups = (int)(prm.K / kGroup);
         const __half* sc_row = scales + ((row0 / 16 + rtl) * groups) * 16 + (i & 15);
+        __half sc_next = sc_row[(kstep0 >> 4) * 16];
         const uint32_t t_lane = tmem + ((uint32_t)(32 * q) << 16);
-        // byte formats: this row's words are the 16-byte chunks of lanes (g, t) of its row tile; six-bit: word 2 (4g + t) +
-        // (step & 1) of each of the tile's three 256-byte planes
-        // nibble format: the 8-byte chunks of lanes (g, t = 0..3) are 32 contiguous bytes; 8-bit format: the 16-byte chunks
-        // of lanes (g, t) in each 512-byte half of the row tile's 1 KB block
-        const uint32_t code_off = SIX ? (uint32_t)(rtl * 768 + g * 32 + (sg & 1) * 4) : NIB ? (uint32_t)(rtl * 256 + g * 32)
-                                : B8 ? (uint32_t)(rtl * 1024 + g * 64) : (uint32_t)(rtl * 512 + g * 64);
+        // byte formats: this row's words are the 16-byte chunks of lanes (g, t = 0..3) of its row tile (8-bit: of each of two
+        // 512-byte halves); nibble format: two such chunks; six-bit: word 2 (4g + t) + (step & 1) of each of the tile's three
+        // 256-byte planes.  (t and the nibble format's second chunk only flip bits that are zero here.)
+        const uint32_t code_at = (uint32_t)rtl * kTileStage + (SIX ? (uint32_t)(sg % SPS >> 1) * 768u + (uint32_t)(g * 32 + (sg & 1) * 4)
+                                                                   : (uint32_t)(sg % SPS) * (kTileStage / SPS) + (uint32_t)(g * (NIB ? 32 : 64)));
+        const uint32_t code_off = code_swizzle(code_at);
+        const uint32_t code_off1 = code_swizzle(code_at + (SIX ? 256u : 512u)), code_off2 = code_swizzle(code_at + 512u);
         const int tx = rtl & 1;                    // six-bit: odd row tiles visit the lanes t in the order t ^ 1 (bank conflicts)
-        int cur_group = -1;
+        int cur_group = kstep0 >> 4;
         uint32_t sc2 = 0;
         uint32_t bad = 0;
         int sa = 0, ua = 0;
-        int cs = (sg / SPS) % CS, ucs = 0;         // code stage of step 4 S + sg and its use count (CS >= 4)
+        int cs = (sg / SPS) % CS, ucs = 0;         // code stage of step 4 S + sg and its use count (CS * SPS >= 4)
         for (int S = 0; S < nsuper; ++S) {
             const int jg = kstep0 + 4 * S + sg;    // 64-input step of the layer
             bad |= t_wait(code_full(cs), (uint32_t)(ucs & 1), t_limit(bad)) ^ 1u;
-            if ((jg >> 4) != cur_group) {          // new group of 1024 inputs: this row's scale
+            if (S == 0 || (jg >> 4) != cur_group) {      // new group of 1024 inputs: this row's scale, and the next one's load
                 cur_group = jg >> 4;
-                const __half sc = sc_row[cur_group * 16];
-                const __half2 s2 = __half2half2(sc);
+                const __half2 s2 = __half2half2(sc_next);
                 sc2 = *reinterpret_cast<const uint32_t*>(&s2);
+                if (cur_group + 1 < groups) sc_next = sc_row[(cur_group + 1) * 16];
             }
             uint4 c4[4] = {};                      // c4[t] = the four index words (steps m = 0..3) of lane (g, t)
             uint32_t a[32];
-            auto unrotate = [&]() {                // chunk t was loaded by instruction (t - rot) & 3
-                if (rot & 1) { const uint4 t0 = c4[0]; c4[0] = c4[3]; c4[3] = c4[2]; c4[2] = c4[1]; c4[1] = t0; }
-                if (rot & 2) { uint4 t0 = c4[0]; c4[0] = c4[2]; c4[2] = t0; t0 = c4[1]; c4[1] = c4[3]; c4[3] = t0; }
-            };
             if (B8) {
                 // 8-bit scalar codes: a register (two consecutive inputs of the row) is halfword h of word 2m + kh of lane
                 // (g, t) - two code bytes, two lookups (a table entry carries its value in both halves).  Words 0..3 of
@@ -454,8 +465,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const __grid_c
                 for (int hh = 0; hh < 2; ++hh) {
 #pragma unroll
                     for (int jj = 0; jj < 4; ++jj)
-                        c4[jj] = t_lds128(code_stage(cs) + code_off + (uint32_t)(hh * 512) + (uint32_t)(((jj + rot) & 3) * 16));
-                    unrotate();
+                        c4[jj] = t_lds128(code_stage(cs) + ((hh ? code_off1 : code_off) ^ (uint32_t)(jj * 16)));
 #pragma unroll
                     for (int t = 0; t < 4; ++t) {
 #pragma unroll
@@ -476,31 +486,31 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const __grid_c
             } else {
             if (NIB) {
                 // nibble pairs: byte 2m + kh of lane (g, t) holds the codes of row halves 0 (low nibble) and 1 (high nibble);
-                // the row's eight nibbles per lane become the bytes of two index words.  The two 16-byte loads are issued in
-                // the order that keeps the eight g of a warp on different banks.
-                const bool swp = (g & 4) != 0;
-                const uint4 f0 = t_lds128(code_stage(cs) + code_off + (swp ? 16u : 0u));
-                const uint4 f1 = t_lds128(code_stage(cs) + code_off + (swp ? 0u : 16u));
-                const uint4 lo = swp ? f1 : f0, hi = swp ? f0 : f1;        // lanes t = 0, 1 and t = 2, 3
+                // the row's eight nibbles per lane become the bytes of two index words.
+                const uint4 lo = t_lds128(code_stage(cs) + code_off), hi = t_lds128(code_stage(cs) + (code_off ^ 16u));   // lanes t = 0, 1 and 2, 3
                 const uint32_t sh = (uint32_t)(4 * h);
                 c4[0] = make_uint4((lo.x >> sh) & 0x0f0f0f0fu, (lo.y >> sh) & 0x0f0f0f0fu, 0u, 0u);
                 c4[1] = make_uint4((lo.z >> sh) & 0x0f0f0f0fu, (lo.w >> sh) & 0x0f0f0f0fu, 0u, 0u);
                 c4[2] = make_uint4((hi.x >> sh) & 0x0f0f0f0fu, (hi.y >> sh) & 0x0f0f0f0fu, 0u, 0u);
                 c4[3] = make_uint4((hi.z >> sh) & 0x0f0f0f0fu, (hi.w >> sh) & 0x0f0f0f0fu, 0u, 0u);
             } else if (!SIX) {
-                // the 16-byte chunks of lanes (g, t = 0..3) of row tile rtl; instruction jj reads chunk (jj + rot) & 3
-                // so that the eight g of a warp hit eight different bank groups
 #pragma unroll
-                for (int jj = 0; jj < 4; ++jj)
-                    c4[jj] = t_lds128(code_stage(cs) + code_off + (uint32_t)(((jj + rot) & 3) * 16));
+                for (int jj = 0; jj < 4; ++jj) c4[jj] = t_lds128(code_stage(cs) + (code_off ^ (uint32_t)(jj * 16)));
             } else {
                 uint32_t w0[4], w1[4], w2[4];
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
-                    const uint32_t addr = code_stage(cs) + code_off + (uint32_t)((t ^ tx) * 8);
-                    w0[t] = t_lds32(addr);
-                    w1[t] = t_lds32(addr + 256u);
-                    w2[t] = t_lds32(addr + 512u);
+                    const uint32_t flip = (uint32_t)((t ^ tx) * 8);
+                    w0[t] = t_lds32(code_stage(cs) + (code_off ^ flip));
+                    w1[t] = t_lds32(code_stage(cs) + (code_off1 ^ flip));
+                    w2[t] = t_lds32(code_stage(cs) + (code_off2 ^ flip));
+                }
+#pragma unroll
+                for (int t = 0; t < 4; t += 2) {
+                    auto put_in_order = [&](uint32_t& a0, uint32_t& a1) { const uint32_t u = a0; a0 = tx ? a1 : a0; a1 = tx ? u : a1; };
+                    put_in_order(w0[t], w0[t + 1]);
+                    put_in_order(w1[t], w1[t + 1]);
+                    put_in_order(w2[t], w2[t + 1]);
                 }
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
@@ -513,13 +523,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const __grid_c
                     asm("lop3.b32 %0, %1, %2, 0x0f0f0f0f, 0xe4;" : "=r"(r3) : "r"(w1[t] >> 4), "r"(w2[t] >> 2));
                     c4[t] = make_uint4(r0, r1, r2, r3);
                 }
-                if (tx) { uint4 t0 = c4[0]; c4[0] = c4[1]; c4[1] = t0; t0 = c4[2]; c4[2] = c4[3]; c4[3] = t0; }
             }
             __syncwarp();
             if (lane == 0) t_mbar_arrive(code_empty(cs));     // the code words are in registers: hand the stage back
             cs += 4 / SPS;
             if (cs >= CS) { cs -= CS; ++ucs; }
-            if (!SIX && !NIB) unrotate();
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
 #pragma unroll
@@ -790,8 +798,8 @@ EncodeTiledFn encode_tiled_fn() {
     return fn;
 }
 
-// The packed byte stream of a layer as a 2-D tensor of 8-byte elements: row = 16-row tile (K x 8 bytes: K/64 blocks
-// of 512 bytes), box = one block column of eight consecutive row tiles (the 128 rows of a thread block).
+// The packed byte stream of a layer as a 3-D tensor of 8-byte elements: 16-row tiles of 128-byte lines (byte format: four
+// lines per 64 inputs), box = the lines of one code stage in eight consecutive row tiles (the 128 rows of a thread block).
 bool make_code_map(const higgs_desc& d, const void* packed, CUtensorMap* map) {
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return false;
@@ -800,12 +808,12 @@ bool make_code_map(const higgs_desc& d, const void* packed, CUtensorMap* map) {
     // two neighbouring blocks)
     const Format f = format_of(d.p, d.n);
     const cuuint64_t bpi = f == Format::kSixBit ? 6 : f == Format::kNibble ? 4 : f == Format::kByte8 ? 16 : 8;
-    const cuuint64_t dims[2] = {(cuuint64_t)d.K * bpi / 8, (cuuint64_t)(d.N / 16)};
-    const cuuint64_t strides[1] = {(cuuint64_t)d.K * bpi};
-    const cuuint32_t box[2] = {f == Format::kSixBit ? 96u : f == Format::kNibble ? 32u : f == Format::kByte8 ? 128u : 64u, 8};
-    const cuuint32_t estr[2] = {1, 1};
-    return enc(map, CU_TENSOR_MAP_DATA_TYPE_INT64, 2, const_cast<void*>(packed), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+    const cuuint64_t dims[3] = {16, (cuuint64_t)d.K * bpi / 128, (cuuint64_t)(d.N / 16)};
+    const cuuint64_t strides[2] = {128, (cuuint64_t)d.K * bpi};
+    const cuuint32_t box[3] = {16, f == Format::kSixBit ? 12u : f == Format::kNibble ? 8u : f == Format::kByte8 ? 8u : 8u, 8};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_INT64, 3, const_cast<void*>(packed), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -879,6 +887,7 @@ int launch_linear_tc(const higgs_desc& d, const __half* xdag_tc, int64_t B, cons
         cfg.numAttrs = 2;
     }
     cfg.attrs = attr;
+    prm.b_stages = std::min(kTcMaxBStages, (int)(kTcBBytes / (uint32_t)((BN <= 32 ? 4 : BN <= 64 ? 2 : 1) * BN * 128)));
     // activation-tile stage = FB steps of BN x 128 bytes, at most 16 KB for BN <= 128 (so that the code ring gets the
     // rest of shared memory) and 32 KB for wider tiles
     const Format fmt = format_of(d.p, d.n);

@@ -1,0 +1,30 @@
+"""The tensor-core product at every code format and at token tiles that change the depth of its rings."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2411_17525_b200 as hb
+from tests import gpu_util as U
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("p,n", [(2, 256), (2, 64), (1, 16), (2, 16), (1, 256)])
+@pytest.mark.parametrize("N,K,B", [(128, 1024, 17), (256, 3072, 33), (128, 5120, 65), (128, 2048, 144), (384, 1024, 256), (19072, 1024, 257)])
+def test_tensor_core_rings(p, n, N, K, B):
+    """Rings shorter and longer than the layer, K split over a cluster or not, one or two token tiles."""
+    rng = np.random.default_rng(n + B)
+    g64, gt = U.grid32(p, n)
+    c = rng.integers(0, n, size=(N, K // p))
+    s = (0.5 + rng.random((N, K // 1024))).astype(np.float16)
+    x = torch.from_numpy(rng.standard_normal((B, K)).astype(np.float32)).to(U.dev()).to(torch.bfloat16)
+    d = hb.make_desc(p, n, N, K, 29)
+    assert hb.higgs_rotated_layout(d, B) > 0
+    packed = hb.higgs_pack_codes(d, torch.from_numpy(c.astype(np.uint8)).to(U.dev()))
+    y = hb.higgs_linear(d, x, packed, hb.scales_to_tile_major(torch.from_numpy(s).to(U.dev())), gt)
+    assert hb.higgs_device_status() == hb.HIGGS_OK
+    rows = np.unique(np.r_[0:16, 127, N - 128, N - 1, rng.integers(0, N, 24)])
+    ref = oracle.linear_dense(x.float().cpu().numpy().astype(np.float64), c[rows].astype(np.int32), s[rows].astype(np.float64), 1024, g64, 29)
+    # fp16 roundings of table entry, scaled weight and rotated activation: 3 x 2^-11 of the norm each at worst
+    assert U.linear_error(y[:, torch.from_numpy(rows).to(U.dev())].float().cpu().numpy(), ref) <= 3 * 2.0 ** -11
