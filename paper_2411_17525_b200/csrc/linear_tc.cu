@@ -218,7 +218,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const __grid_c
     if (nA > 16) nA = 16;
     int nB = (int)((base + kTcSmem - code1) / kTcCodeStage);
     if (nB > kTcMaxCodeStages - nA) nB = kTcMaxCodeStages - nA;
-    const int CS = nA + nB;
+    // A stage's uses must all belong to the same warp groups: a group that runs ahead waits for phases in its own order only, and
+    // would take the phase before the one it waits for if the copy another group still waits for landed late.
+    const int CS = (nA + nB) / (4 / SPS) * (4 / SPS);
     auto code_stage = [&](int s) { return s < nA ? code0 + (uint32_t)s * kTcCodeStage : code1 + (uint32_t)(s - nA) * kTcCodeStage; };
     auto b_stage = [&](int s) { return lut + 65536u + (uint32_t)s * b_stage_bytes; };
 
@@ -887,7 +889,9 @@ int launch_linear_tc(const higgs_desc& d, const __half* xdag_tc, int64_t B, cons
         cfg.numAttrs = 2;
     }
     cfg.attrs = attr;
-    prm.b_stages = std::min(kTcMaxBStages, (int)(kTcBBytes / (uint32_t)((BN <= 32 ? 4 : BN <= 64 ? 2 : 1) * BN * 128)));
+    // (up to 64 tokens, and in the 8-bit format, the ring leaves room for an eighth code stage)
+    const uint32_t b_room = BN <= 64 || (BN <= 128 && format_of(d.p, d.n) == Format::kByte8) ? kTcBBytes - 4096u : kTcBBytes;
+    prm.b_stages = std::min(kTcMaxBStages, (int)(b_room / (uint32_t)((BN <= 32 ? 4 : BN <= 64 ? 2 : 1) * BN * 128)));
     // activation-tile stage = FB steps of BN x 128 bytes, at most 16 KB for BN <= 128 (so that the code ring gets the
     // rest of shared memory) and 32 KB for wider tiles
     const Format fmt = format_of(d.p, d.n);
