@@ -48,6 +48,7 @@ struct TcParams {
     int n_more;
     int64_t N, K, ldy;
     int B, BN, n, p, y_mode; // y_mode 0: fp32, 1: bf16
+    int BL;                  // token tile of the rotated activations' layout (BN is this kernel's, at most BL)
     int bits;                // log2(n)
     int b_stages;            // activation-tile stages
     int ksplit;              // K slices (= cluster size along z); each a multiple of 256 inputs
@@ -357,16 +358,32 @@ __global__ void __launch_bounds__(kTcThreads, 1) linear_tc_kernel(const __grid_c
         pdl_wait();            // the rotated activations are the previous kernel's output
         int issued = 0;
         const int nb = ksteps / FB;
-        const uint32_t bytes = b_step_bytes * (uint32_t)FB;
-        const __half* xsrc = prm.xdag + ((int64_t)bt * ksteps_all + kstep0) * BN * 64;
+        // The tile's token blocks (eight tokens, 1 KB per 64 inputs) lie in one tile of the layout, or at the end of one and the
+        // start of the next.
+        const int BL = prm.BL, lt = bt * BN / BL, off = bt * BN - lt * BL, whole = BL == BN;
+        const int n1 = min(BN, BL - off), n2 = (lt + 1) * BL < prm.B ? BN - n1 : 0;
+        const uint32_t bytes = (uint32_t)(n1 + n2) * 128u * (uint32_t)FB;
+        const __half* src1 = prm.xdag + (((int64_t)lt * ksteps_all + kstep0) * BL + off) * 64;
+        const __half* src2 = prm.xdag + ((int64_t)(lt + 1) * ksteps_all + kstep0) * BL * 64;
         int s = 0, it = 0;
         uint32_t bad = 0;
         for (int t = 0; t < nb; ++t) {
             bad |= t_wait(b_free(s), (uint32_t)((it & 1) ^ 1), t_limit(bad)) ^ 1u;
             if (elected) {
                 t_mbar_expect_tx(b_full(s), bytes);
-                t_bulk_load(b_stage(s), xsrc + (int64_t)t * FB * BN * 64, bytes, b_full(s));
+                if (whole) {
+                    t_bulk_load(b_stage(s), src1, bytes, b_full(s));
+                } else {
+#pragma unroll
+                    for (int h = 0; h < FB; ++h) {
+                        const uint32_t dst = b_stage(s) + (uint32_t)h * b_step_bytes;
+                        t_bulk_load(dst, src1 + h * BL * 64, (uint32_t)n1 * 128u, b_full(s));
+                        if (n2) t_bulk_load(dst + (uint32_t)n1 * 128u, src2 + h * BL * 64, (uint32_t)n2 * 128u, b_full(s));
+                    }
+                }
             }
+            src1 += FB * BL * 64;
+            src2 += FB * BL * 64;
             ++issued;
             const bool wrap = s + 1 == BS;
             s = wrap ? 0 : s + 1;
@@ -782,6 +799,35 @@ int tc_k_split(const higgs_desc& d, int64_t B) {
     return ks;
 }
 
+static int tc_sms() {
+    static int cached[64] = {0};
+    return device_once(cached, [] {
+        int dev = 0, n = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
+        return n;
+    });
+}
+
+// The product's own token tile when K is not split: narrower tiles than the layout's may fill the last wave of blocks better.
+// A wave takes about 0.45 + 1.15 BN / 256 us per 256 inputs (measured 0.71 us at 64 tokens, 1.0 at 160, 1.6 at 256) and 3 us to
+// start and to end.  4096x4096 with 1500 tokens: nine tiles of 176 fill two waves, six of 256 fill 1.3: 70 -> 51 us;
+// 6144x4096 with 1000: 59 -> 50; 4096x14336 with 600: 95 -> 84.  Below a tenth of predicted gain the layout's tile stays: its
+// copies are whole (28672x4096 with 300 tokens, 112 instead of 160 a tile: 77 -> 97 us).
+static int tc_token_tile(const higgs_desc& d, int64_t B) {
+    const int64_t row_tiles = d.N / 128, t0 = (B + 255) / 256;
+    const int sms = tc_sms();
+    int best_bn = tc_batch_tile(B);
+    double best = 0.0, first = 0.0;
+    for (int64_t t = t0; t <= 2 * t0; ++t) {
+        const int bn = (int)(((B + t - 1) / t + 15) / 16 * 16);
+        const int64_t waves = (row_tiles * ((B + bn - 1) / bn) + sms - 1) / sms;
+        const double cost = (double)waves * ((double)(d.K / 256) * (0.45 + 1.15 / 256 * bn) + 3.0);
+        if (t == t0) first = cost;
+        if (t == t0 || (cost < best && cost < 0.9 * first)) { best = cost; best_bn = bn; }
+    }
+    return best_bn;
+}
+
 namespace {
 
 // cuTensorMapEncodeTiled through the runtime's driver-entry-point query (the library does not link libcuda).
@@ -827,7 +873,7 @@ int launch_linear_tc(const higgs_desc& d, const __half* xdag_tc, int64_t B, cons
                      const MultiSegments* segs) {
     if (more && more->count > kMaxGather - 1) return HIGGS_ERR_INVALID_ARG;
     if (segs && (segs->count < 1 || segs->count > kMaxMulti || more)) return HIGGS_ERR_INVALID_ARG;
-    const int BN = tc_batch_tile(B);
+    const int ksplit = tc_k_split(d, B), BN = ksplit == 1 ? tc_token_tile(d, B) : tc_batch_tile(B);
     const int64_t tiles = (B + BN - 1) / BN;
     static int configured[64] = {0};
     const int conf = device_once(configured, [] {
@@ -869,9 +915,9 @@ int launch_linear_tc(const higgs_desc& d, const __half* xdag_tc, int64_t B, cons
     prm.n_more = more ? more->count : 0;
     for (int i = 0; i < kMaxGather - 1; ++i) prm.y_more[i] = (more && i < more->count) ? more->y[i] : nullptr;
     prm.N = d.N; prm.K = d.K; prm.ldy = ldy > 0 ? ldy : d.N;
-    prm.B = (int)B; prm.BN = BN; prm.n = d.n; prm.p = d.p; prm.y_mode = y_mode;
+    prm.B = (int)B; prm.BN = BN; prm.BL = tc_batch_tile(B); prm.n = d.n; prm.p = d.p; prm.y_mode = y_mode;
     prm.bits = code_bits(d.n);
-    prm.ksplit = tc_k_split(d, B);
+    prm.ksplit = ksplit;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(d.N / 128), (unsigned)tiles, (unsigned)prm.ksplit);
     cfg.blockDim = dim3(kTcThreads);

@@ -28,3 +28,20 @@ def test_tensor_core_rings(p, n, N, K, B):
     ref = oracle.linear_dense(x.float().cpu().numpy().astype(np.float64), c[rows].astype(np.int32), s[rows].astype(np.float64), 1024, g64, 29)
     # fp16 roundings of table entry, scaled weight and rotated activation: 3 x 2^-11 of the norm each at worst
     assert U.linear_error(y[:, torch.from_numpy(rows).to(U.dev())].float().cpu().numpy(), ref) <= 3 * 2.0 ** -11
+
+
+@pytest.mark.parametrize("p,n", [(2, 256), (2, 64)])
+@pytest.mark.parametrize("N,K,B", [(4096, 1024, 1500), (6144, 2048, 1000), (2304, 3072, 1111)])
+def test_token_tiles_that_cross_the_layouts(p, n, N, K, B):
+    """The product's token tiles begin and end inside the layout's: every token against the same layer in batches of one tile."""
+    rng = np.random.default_rng(B)
+    _, gt = U.grid32(p, n)
+    d = hb.make_desc(p, n, N, K, 31)
+    packed = hb.higgs_pack_codes(d, torch.from_numpy(rng.integers(0, n, size=(N, K // p)).astype(np.uint8)).to(U.dev()))
+    sc = hb.scales_to_tile_major(torch.from_numpy((0.5 + rng.random((N, K // 1024))).astype(np.float16)).to(U.dev()))
+    x = torch.from_numpy(rng.standard_normal((B, K)).astype(np.float32)).to(U.dev()).to(torch.bfloat16)
+    y = hb.higgs_linear(d, x, packed, sc, gt)
+    ref = torch.cat([hb.higgs_linear(d, x[b:b + 256].contiguous(), packed, sc, gt) for b in range(0, B, 256)])
+    assert hb.higgs_device_status() == hb.HIGGS_OK
+    # the same fp16 operands; fp32 sums of K products in another order when a part is cut into K slices
+    assert (y - ref).abs().max() <= 2.0 ** -24 * K * ref.abs().max()
