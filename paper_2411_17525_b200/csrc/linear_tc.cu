@@ -810,8 +810,8 @@ static int tc_sms() {
 
 // The product's own token tile when K is not split: narrower tiles than the layout's may fill the last wave of blocks better.
 // A wave takes about 0.45 + 1.15 BN / 256 us per 256 inputs (measured 0.71 us at 64 tokens, 1.0 at 160, 1.6 at 256) and 3 us to
-// start and to end.  4096x4096 with 1500 tokens: nine tiles of 176 fill two waves, six of 256 fill 1.3: 70 -> 51 us;
-// 6144x4096 with 1000: 59 -> 50; 4096x14336 with 600: 95 -> 84.  Below a tenth of predicted gain the layout's tile stays: its
+// start and to end.  4096x4096 with 1500 tokens: nine tiles of 176 fill two waves, six of 256 fill 1.3: 61 -> 51 us;
+// 6144x4096 with 1000: 61 -> 50; 4096x14336 with 600: 92 -> 74.  Below a tenth of predicted gain the layout's tile stays: its
 // copies are whole (28672x4096 with 300 tokens, 112 instead of 160 a tile: 77 -> 97 us).
 static int tc_token_tile(const higgs_desc& d, int64_t B) {
     const int64_t row_tiles = d.N / 128, t0 = (B + 255) / 256;
