@@ -174,27 +174,53 @@ __device__ __forceinline__ void apply_signs1024(float (&v)[32], uint64_t xi, int
     }
 }
 
+// two fp32 operations in one instruction
+__device__ __forceinline__ uint64_t pair_of(float a, float b) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
+    return v;
+}
+__device__ __forceinline__ void unpair(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) { uint64_t v; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b)); return v; }
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) { uint64_t v; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b)); return v; }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) { uint64_t v; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b)); return v; }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t v;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
+    return v;
+}
+// butterflies over the low BITS bits of the index of the pairs
+template <int BITS = 4>
+__device__ __forceinline__ void pair_stages(uint64_t (&q)[16]) {
+#pragma unroll
+    for (int h = 1; h < (1 << BITS); h <<= 1) {
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+            if ((t & h) == 0) {
+                const uint64_t a = q[t], b = q[t | h];
+                q[t] = add2(a, b);
+                q[t | h] = sub2(a, b);
+            }
+        }
+    }
+}
+
 // The 1024-point transform with one exchange through shared memory instead of five shuffle stages.  A warp owns one
 // group; before, lane l holds v[c*8 + e] = element c*256 + l*8 + e (the mapping above: index bits 0-2, 8, 9 in
 // registers, bits 3-7 across lanes); after, lane c*8 + e holds v[j] = element c*256 + j*8 + e (bits 3-7 in registers).
 // Same butterflies in the same order of stages as fwht1024_warp, so the values are bit-identical to it.  160 shuffles and
 // 160 fused multiply-adds become 8 vector stores, 32 loads and 160 additions: 64 shared-memory wavefronts instead of
-// 160.  `ex`: this warp's exchange buffer, 32 rows of 32 floats, 16-byte aligned; row l holds lane l's values, its
+// 160; the butterflies of index bits above the lowest work on fp32 pairs, 192 instructions instead of 320.  `ex`: this warp's exchange buffer, 32 rows of 32 floats, 16-byte aligned; row l holds lane l's values, its
 // four-float chunks permuted by l % 8, which keeps the vector stores (lane l writes row l) and the loads (lane l reads
 // column l) free of bank conflicts.
 constexpr int kFwhtExchange = 1024;
 __device__ __forceinline__ void butterflies32(float (&v)[32]) {
+    uint64_t q[16];
 #pragma unroll
-    for (int h = 1; h < 32; h <<= 1) {
+    for (int t = 0; t < 16; ++t) q[t] = pair_of(v[2 * t] + v[2 * t + 1], v[2 * t] - v[2 * t + 1]);
+    pair_stages(q);
 #pragma unroll
-        for (int r = 0; r < 32; ++r) {
-            if ((r & h) == 0) {
-                const float a = v[r], b = v[r | h];
-                v[r] = a + b;
-                v[r | h] = a - b;
-            }
-        }
-    }
+    for (int t = 0; t < 16; ++t) unpair(q[t], v[2 * t], v[2 * t + 1]);
 }
 __device__ __forceinline__ void fwht1024_to_columns(float (&v)[32], float* ex, int lane) {
     butterflies32(v);
@@ -240,36 +266,37 @@ __device__ __forceinline__ float with_sign(float v, uint32_t bits, int r) {
     return __uint_as_float(__float_as_uint(v) ^ ((bits << (31 - r)) & 0x80000000u));
 }
 
-// two fp32 operations in one instruction
-__device__ __forceinline__ uint64_t pair_of(float a, float b) {
-    uint64_t v;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
-    return v;
-}
-__device__ __forceinline__ void unpair(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) { uint64_t v; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b)); return v; }
-__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) { uint64_t v; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b)); return v; }
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) { uint64_t v; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b)); return v; }
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t v;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
-    return v;
-}
-// butterflies over the low BITS bits of the index of the pairs
-template <int BITS = 4>
-__device__ __forceinline__ void pair_stages(uint64_t (&q)[16]) {
+// A row's 1024 values in the order of a group's load (lane l, c = 0..3, e = 0..7: element c*256 + lane*8 + e), raw.
+template <typename T>
+struct RawGroup;
+template <>
+struct RawGroup<__nv_bfloat16> {
+    uint4 q[4];
+    __device__ __forceinline__ void load(const __nv_bfloat16* __restrict__ src, int lane) {
 #pragma unroll
-    for (int h = 1; h < (1 << BITS); h <<= 1) {
-#pragma unroll
-        for (int t = 0; t < 16; ++t) {
-            if ((t & h) == 0) {
-                const uint64_t a = q[t], b = q[t | h];
-                q[t] = add2(a, b);
-                q[t | h] = sub2(a, b);
-            }
-        }
+        for (int c = 0; c < 4; ++c) q[c] = __ldg(reinterpret_cast<const uint4*>(src + c * 256 + lane * 8));
     }
-}
+    __device__ __forceinline__ uint32_t word(int t) const { return (t & 3) == 0 ? q[t >> 2].x : (t & 3) == 1 ? q[t >> 2].y : (t & 3) == 2 ? q[t >> 2].z : q[t >> 2].w; }
+    // pair t with the signs of bits 2t, 2t + 1 of `bits` flipped: one multiply puts both bits on the two sign positions
+    __device__ __forceinline__ void get_signed(int t, uint32_t bits, float& a, float& b) const {
+        const uint32_t byte = (bits >> (8 * (t >> 2))) & 0xffu;
+        const uint32_t w = word(t) ^ ((byte * ((1u << (15 - 2 * (t & 3))) + (1u << (30 - 2 * (t & 3))))) & 0x80008000u);
+        a = __uint_as_float(w << 16);
+        b = __uint_as_float(w & 0xffff0000u);
+    }
+};
+template <>
+struct RawGroup<float> {
+    float4 q[8];
+    __device__ __forceinline__ void load(const float* __restrict__ src, int lane) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) q[c] = __ldg(reinterpret_cast<const float4*>(src + (c >> 1) * 256 + lane * 8 + (c & 1) * 4));
+    }
+    __device__ __forceinline__ void get_signed(int t, uint32_t bits, float& a, float& b) const {
+        a = with_sign((t & 1) ? q[t >> 1].z : q[t >> 1].x, bits, 2 * t);
+        b = with_sign((t & 1) ? q[t >> 1].w : q[t >> 1].y, bits, 2 * t + 1);
+    }
+};
 
 // element index inside the group of register r of lane l (see above)
 __device__ __forceinline__ int fwht_index(int lane, int r) { return (r >> 3) * 256 + lane * 8 + (r & 7); }

@@ -68,40 +68,6 @@ __device__ __forceinline__ void fill_pair_table(float* table, const float* __res
     }
 }
 
-template <typename T>
-struct RawRow;
-template <>
-struct RawRow<__nv_bfloat16> {
-    uint4 q[4];
-    __device__ __forceinline__ void load(const __nv_bfloat16* __restrict__ src, int lane) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) q[c] = __ldg(reinterpret_cast<const uint4*>(src + c * 256 + lane * 8));
-    }
-    __device__ __forceinline__ void get(float (&v)[32]) const {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const uint32_t w[4] = {q[c].x, q[c].y, q[c].z, q[c].w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                v[c * 8 + 2 * e] = __uint_as_float(w[e] << 16);
-                v[c * 8 + 2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
-            }
-        }
-    }
-};
-template <>
-struct RawRow<float> {
-    float4 q[8];
-    __device__ __forceinline__ void load(const float* __restrict__ src, int lane) {
-#pragma unroll
-        for (int c = 0; c < 8; ++c) q[c] = __ldg(reinterpret_cast<const float4*>(src + (c >> 1) * 256 + lane * 8 + (c & 1) * 4));
-    }
-    __device__ __forceinline__ void get(float (&v)[32]) const {
-#pragma unroll
-        for (int c = 0; c < 8; ++c) { v[4 * c] = q[c].x; v[4 * c + 1] = q[c].y; v[4 * c + 2] = q[c].z; v[4 * c + 3] = q[c].w; }
-    }
-};
-
 template <typename OutT>
 __device__ __forceinline__ void store_row(OutT* __restrict__ dst, int lane, const float (&v)[32]);
 template <>
@@ -127,9 +93,10 @@ __device__ __forceinline__ void store_row<__nv_bfloat16>(__nv_bfloat16* __restri
 // ERROR = false: W_out[row][k] = the dequantised matrix.  ERROR = true: the two sums of t^2 = ||W^ - W||^2 / ||W||^2,
 // taken in the rotated space (the transform is orthonormal): W is rotated as the encoder rotates it and compared with
 // scale * G[code].  A block writes its pair of partial sums; launch_layer_error's second kernel adds them in block order.
-// Bound: instruction issue (75-79 % of the slots; 810 instructions per row and group, 360 of them the transform), next to 2 or 4 + b/8
-// bytes per weight from HBM.  14336 x 4096 bf16 at 4 bits: error 185 + 47 us (canonical codes unpacked to memory byte by
-// byte, then one warp per row and group adding to two global doubles) -> 59 us; the 147 MB it reads take 22 us.
+// Bound: instruction issue (75-79 % of the slots with scalar arithmetic, 810 instructions per row and group of which 360 the
+// transform; most of it works on fp32 pairs now), next to 2 or 4 + b/8 bytes per weight from HBM.  14336 x 4096 bf16 at 4 bits: error
+// 185 + 47 us (canonical codes unpacked to memory byte by byte, then one warp per row and group adding to two global
+// doubles) -> 63 -> 57 us with pairs (3 bits 68 -> 60), dequantised 56 -> 52; the 147 MB it reads take 22 us.
 template <int FMT, typename T, bool ERROR>
 __global__ void __launch_bounds__(kDqWarps * 32, 2) packed_rows_kernel(const uint8_t* __restrict__ packed, const __half* __restrict__ scales,
                                                                        const float* __restrict__ grid, int p, int n, int bits,
@@ -153,7 +120,7 @@ __global__ void __launch_bounds__(kDqWarps * 32, 2) packed_rows_kernel(const uin
         const __half* sc = scales + (rt * groups + gi) * kRowTile + warp;
         const float scale[2] = {__half2float(sc[0]), __half2float(sc[8])};
         const uint32_t sign = lane_sign_bits(xi, gi * kGroup, lane);
-        RawRow<T> raw[2];
+        RawGroup<T> raw[2];
         if (ERROR) {
 #pragma unroll
             for (int rh = 0; rh < 2; ++rh) raw[rh].load(W + (rt * 16 + warp + 8 * rh) * K + gi * kGroup, lane);
@@ -162,19 +129,26 @@ __global__ void __launch_bounds__(kDqWarps * 32, 2) packed_rows_kernel(const uin
         for (int rh = 0; rh < 2; ++rh) {
             float v[32];
             if (ERROR) {
-                raw[rh].get(v);
-                float dsum = 0.f, nsum = 0.f;
+                uint64_t dsum2 = pair_of(0.f, 0.f), nsum2 = dsum2;
 #pragma unroll
-                for (int r = 0; r < 32; ++r) {
-                    dsum = fmaf(v[r], v[r], dsum);
-                    v[r] = with_sign(v[r], sign, r);
+                for (int t = 0; t < 16; ++t) {
+                    raw[rh].get_signed(t, sign, v[2 * t], v[2 * t + 1]);
+                    const uint64_t x = pair_of(v[2 * t], v[2 * t + 1]);
+                    dsum2 = fma2(x, x, dsum2);
                 }
                 fwht1024_to_columns(v, ex, lane);
+                const uint64_t scale2 = pair_of(scale[rh], scale[rh]), to_unit = pair_of(-0.03125f, -0.03125f);
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const float d = fmaf(scale[rh], table_lane[codes.index(j, rh, lane) * 32], -0.03125f * v[j]);
-                    nsum = fmaf(d, d, nsum);
+                for (int j = 0; j < 32; j += 2) {
+                    const uint64_t g = pair_of(table_lane[codes.index(j, rh, lane) * 32], table_lane[codes.index(j + 1, rh, lane) * 32]);
+                    const uint64_t d = fma2(scale2, g, mul2(pair_of(v[j], v[j + 1]), to_unit));
+                    nsum2 = fma2(d, d, nsum2);
                 }
+                float dsum, nsum, odd;
+                unpair(dsum2, dsum, odd);
+                dsum += odd;
+                unpair(nsum2, nsum, odd);
+                nsum += odd;
 #pragma unroll
                 for (int m = 16; m > 0; m >>= 1) {
                     nsum += __shfl_xor_sync(0xffffffffu, nsum, m);

@@ -695,7 +695,7 @@ namespace {
 // A block rotates one 1024-group of the eight tokens of a token block, one warp each; the rotated halves meet in shared
 // memory (over the exchange buffers, which are idle by then), from where the block writes sixteen runs of 1 KB.  Tokens
 // beyond the batch are written as zeros.  Bound: memory for long prompts (4 bytes per activation), else the latency of
-// one warp's transform.  1999 tokens x 4096: 22 -> 12.3 us, x 14336: 69 -> 33 us (before: four warps per group with five
+// one warp's transform.  1999 tokens x 4096: 22 -> 10.0 us, x 14336: 69 -> 29.7 us (before: four warps per group with five
 // shuffle stages, 16-byte stores 128 bytes apart).
 constexpr int kRotWarps = 8;
 __global__ void __launch_bounds__(kRotWarps * 32) rht_activations_tc_kernel(const __nv_bfloat16* __restrict__ x, __half* __restrict__ xdag,

@@ -409,38 +409,6 @@ __device__ __forceinline__ void encoder_transform(uint64_t (&q)[16], uint8_t* ex
     pair_stages(q);
 }
 
-// A row's 1024 values in the lane order above (element c*256 + lane*8 + e), raw.
-template <typename T>
-struct RawGroup;
-template <>
-struct RawGroup<__nv_bfloat16> {
-    uint4 q[4];
-    __device__ __forceinline__ void load(const __nv_bfloat16* __restrict__ src, int lane) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) q[c] = __ldg(reinterpret_cast<const uint4*>(src + c * 256 + lane * 8));
-    }
-    __device__ __forceinline__ uint32_t word(int t) const { return (t & 3) == 0 ? q[t >> 2].x : (t & 3) == 1 ? q[t >> 2].y : (t & 3) == 2 ? q[t >> 2].z : q[t >> 2].w; }
-    // pair t with the signs of bits 2t, 2t + 1 of `bits` flipped: one multiply puts both bits on the two sign positions
-    __device__ __forceinline__ void get_signed(int t, uint32_t bits, float& a, float& b) const {
-        const uint32_t byte = (bits >> (8 * (t >> 2))) & 0xffu;
-        const uint32_t w = word(t) ^ ((byte * ((1u << (15 - 2 * (t & 3))) + (1u << (30 - 2 * (t & 3))))) & 0x80008000u);
-        a = __uint_as_float(w << 16);
-        b = __uint_as_float(w & 0xffff0000u);
-    }
-};
-template <>
-struct RawGroup<float> {
-    float4 q[8];
-    __device__ __forceinline__ void load(const float* __restrict__ src, int lane) {
-#pragma unroll
-        for (int c = 0; c < 8; ++c) q[c] = __ldg(reinterpret_cast<const float4*>(src + (c >> 1) * 256 + lane * 8 + (c & 1) * 4));
-    }
-    __device__ __forceinline__ void get_signed(int t, uint32_t bits, float& a, float& b) const {
-        a = with_sign((t & 1) ? q[t >> 1].z : q[t >> 1].x, bits, 2 * t);
-        b = with_sign((t & 1) ? q[t >> 1].w : q[t >> 1].y, bits, 2 * t + 1);
-    }
-};
-
 constexpr int kEncThreads = 1024, kEncTiles = 3, kEncExchange = 2048;
 // A row of the encoder's tile: the codes of every 256 values are followed by 8 (p = 2) or 16 bytes, which spreads the
 // lanes' byte stores (128 or 256 bytes apart) over the banks; rows are an odd multiple of 16 bytes apart in bank position.
