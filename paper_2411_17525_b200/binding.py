@@ -290,21 +290,21 @@ def higgs_quantize(desc: higgs_desc, W: torch.Tensor, grid: torch.Tensor, want_c
         assert packed.is_cuda and packed.dtype == torch.uint8 and packed.numel() >= higgs_packed_bytes(desc)
         assert scales.is_cuda and scales.dtype == torch.float16 and scales.numel() * 2 >= higgs_scales_bytes(desc)
     else:
-        packed = torch.empty(max(higgs_packed_bytes(desc), 16), dtype=torch.uint8, device=dev)
-        scales = torch.empty((desc.N // 16, max(desc.K // desc.g, 0), 16), dtype=torch.float16, device=dev)
+        packed = W.new_empty(max(lib.higgs_packed_bytes(desc), 16), dtype=torch.uint8)
+        scales = W.new_empty((desc.N // 16, max(desc.K // desc.g, 0), 16), dtype=torch.float16)
     canonical = torch.empty((desc.N, desc.K // desc.p), dtype=torch.uint8, device=dev) if want_canonical else None
     if workspace is None:
-        workspace = _workspace(higgs_workspace_bytes(desc, HIGGS_OP_QUANTIZE), dev)
+        workspace = _workspace(lib.higgs_workspace_bytes(desc, HIGGS_OP_QUANTIZE, 0), dev)
     elif workspace is False:          # lend none (allowed with want_canonical): the library then packs in a second kernel
         assert want_canonical
         workspace = torch.empty(0, dtype=torch.uint8, device=dev)
     if table is not None:
         assert table.is_cuda and table.dtype == torch.uint8 and table.numel() >= lib.higgs_encoder_table_bytes(desc.p, desc.n)
-        _check(lib.higgs_quantize_prepared(ctypes.byref(desc), _ptr(W), _dtype_code(W), _ptr(grid), _ptr(table), _ptr(packed),
+        _check(lib.higgs_quantize_prepared(desc, _ptr(W), _dtype_code(W), _ptr(grid), _ptr(table), _ptr(packed),
                                            _ptr(scales), _ptr(canonical), _ptr(workspace), workspace.numel(), _stream()),
                "higgs_quantize_prepared")
     else:
-        _check(lib.higgs_quantize(ctypes.byref(desc), _ptr(W), _dtype_code(W), _ptr(grid), _ptr(packed), _ptr(scales),
+        _check(lib.higgs_quantize(desc, _ptr(W), _dtype_code(W), _ptr(grid), _ptr(packed), _ptr(scales),
                                   _ptr(canonical), _ptr(workspace), workspace.numel(), _stream()), "higgs_quantize")
     return packed, scales, canonical
 
@@ -662,11 +662,12 @@ def higgs_make_uniform_grid(n: int, device=None):
 def higgs_layer_error(desc: higgs_desc, W: torch.Tensor, packed: torch.Tensor, scales: torch.Tensor, grid: torch.Tensor) -> float:
     """Relative quantisation error t^2 = ||W^ - W||^2 / ||W||^2 of the layer (Section 5, 'Measuring Grid Parameters')."""
     assert W.is_cuda and W.is_contiguous() and W.dtype in (torch.float32, torch.bfloat16)
-    sums = torch.zeros(3, dtype=torch.float64, device=W.device)
-    ws = _workspace(higgs_workspace_bytes(desc, HIGGS_OP_QUANTIZE, 0), W.device)
-    _check(lib.higgs_layer_error(ctypes.byref(desc), _ptr(W), _dtype_code(W), _ptr(packed), _ptr(scales), _ptr(grid), _ptr(sums),
+    sums = W.new_empty(3, dtype=torch.float64)           # (all three are written)
+    ws = _workspace(lib.higgs_workspace_bytes(desc, HIGGS_OP_QUANTIZE, 0), W.device)
+    ratio = sums[2]
+    _check(lib.higgs_layer_error(desc, _ptr(W), _dtype_code(W), _ptr(packed), _ptr(scales), _ptr(grid), _ptr(sums),
                                  _ptr(ws), ws.numel(), _stream()), "higgs_layer_error")
-    return float(sums[2].item())
+    return ratio.item()
 
 
 def higgs_quantize_general(p: int, n: int, W: torch.Tensor, grid: torch.Tensor, rht_seed: int, want_error: bool = True):

@@ -106,6 +106,7 @@ __global__ void __launch_bounds__(kDqWarps * 32, 2) packed_rows_kernel(const uin
     constexpr int ROWS = FMT == 1 ? 64 : FMT == 2 ? 16 : 256;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float* ex = dq_smem + ROWS * 32 + warp * kFwhtExchange;
+    if (ERROR) pdl_trigger();          // (the kernel that adds the partial sums waits for this one's end on the SM)
     fill_pair_table<FMT>(dq_smem, grid, p, n, bits);
     __syncthreads();
     const float* table_lane = dq_smem + lane;
@@ -184,6 +185,7 @@ __global__ void __launch_bounds__(64) error_total_kernel(const double* __restric
     __shared__ double total[2];
     const int which = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double s = 0.0;
+    pdl_wait();
     for (int i = lane; i < blocks; i += 32) s += partials[2 * i + which];
 #pragma unroll
     for (int m = 16; m > 0; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
@@ -247,8 +249,7 @@ int launch_layer_error(const higgs_desc& d, const void* packed, const void* scal
     const int rc = w_dtype == HIGGS_F32 ? launch_format<float, true>(d, packed, scales, grid, W, nullptr, partials, &blocks, st)
                                         : launch_format<__nv_bfloat16, true>(d, packed, scales, grid, W, nullptr, partials, &blocks, st);
     if (rc != HIGGS_OK) return rc;
-    error_total_kernel<<<1, 64, 0, st>>>(partials, blocks, sums);
-    return cuda_status(cudaGetLastError());
+    return cuda_status(launch_pdl(error_total_kernel, dim3(1), dim3(64), 0, st, static_cast<const double*>(partials), blocks, sums));
 }
 
 int launch_dequantize(const higgs_desc& d, const void* packed, const void* scales, const float* grid, void* W_out,
