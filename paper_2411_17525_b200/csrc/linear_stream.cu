@@ -76,7 +76,10 @@ constexpr uint32_t kMaxDynSmem = 232448 - kRotationReserve;
 constexpr uint32_t kSmallBytes = 4096;  // barriers, recycle counters, abort flag
 constexpr int kWarps = 16;
 constexpr int kMaxDepth = 8;            // ring slots per warp
-constexpr int kArmFirst = 1;            // tasks a warp requests before its loop starts; the ring then fills two requests per consumed task
+// Tasks a warp requests before its loop starts; the ring then fills two requests per consumed task.  Two in a cluster pair, whose
+// prologue is longer by a cluster barrier (28672x8192 at one token 31.1 -> 30.1 us, 8192x8192 12.0 -> 11.7, 8 bits 4096x8192
+// 12.8 -> 12.1), one elsewhere (28672x4096 16.9 us against 17.0 with two, 8192x28672 31.3 against 31.8).
+__host__ __device__ constexpr int arm_first(bool pair) { return pair ? 2 : 1; }
 constexpr int kMaxAccSlots = 32;        // items whose partial tiles may be parked at once
 constexpr uint32_t kWaitLimit = 1u << 22;
 constexpr uint32_t kNibbleTileBytes = 32768; // nibble format: the table rows are full, the partial tiles live at the end of shared memory
@@ -443,7 +446,7 @@ __global__ void __launch_bounds__((kWarps + 1) * 32, 1) linear_stream_kernel(con
     // The first task's copy starts now: the weights are inputs that no kernel of the stream writes (a producer of
     // weights ends with a fence kernel, so this kernel cannot have started while one was running).
     int issued = 0;
-    for (; issued < n_tasks && issued < D && issued < kArmFirst; ++issued) issue(issued);
+    for (; issued < n_tasks && issued < D && issued < arm_first(PAIR); ++issued) issue(issued);
     int d_issue = issued == D ? 0 : issued;      // slot of the next task to be requested
     // Everything above depends only on the weights.  The activations (and y, which the previous kernel in the
     // stream may still be reading or clearing) are touched only after the previous kernel has completed.
@@ -753,7 +756,7 @@ __global__ void __launch_bounds__((kWarps + 1) * 32, 1) linear_stream_kernel(con
         __syncwarp();
         ++done;
         // the slot's words are in registers: request further tasks - task i + D into this slot in the steady state, two
-        // per consumed task while the ring is still filling (the first kArmFirst were requested before the loop)
+        // per consumed task while the ring is still filling (the first arm_first were requested before the loop)
         if (issued < n_tasks) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
