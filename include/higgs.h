@@ -223,8 +223,8 @@ int higgs_quantize_prepared(const higgs_desc* desc, const void* W, int w_dtype, 
  *   y        device, [B][N] row-major, y_dtype in {HIGGS_F32, HIGGS_BF16}
  *   workspace  device, 256-byte aligned, higgs_workspace_bytes(desc, HIGGS_OP_LINEAR, B) bytes; may be NULL where
  *            higgs_linear_launch_count(desc, B, y_dtype) is 1 (the one kernel needs none)
- * Kernels behind the call: for one or two tokens and a small layer (K = 1024, or
- * fewer than 2 M weights times tokens) a single kernel that rotates the
+ * Kernels behind the call: for one or two tokens and a small layer (K times tokens
+ * below 4096, or fewer than 2 M weights times tokens) a single kernel that rotates the
  * activations in its prologue; else up to 16 tokens a rotation
  * kernel and the small-batch product kernel; above that (and from 9 tokens
  * for layers with at least 4096 rows, 4096 inputs and 16 M weights) a rotation kernel and the tcgen05 kernel.

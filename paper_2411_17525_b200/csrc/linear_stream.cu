@@ -1005,9 +1005,11 @@ bool linear_fused_possible(const higgs_desc& d, int64_t B) {
 // ends (rht.cu) runs while the next product starts up; the fused rotation starts only after that.  Chains of 40 products,
 // fused / separate in us: one token 512x1024 2.8 / 3.1, 28672x1024 9.0 / 9.7, 512x2048 3.2 / 3.3, 16384x2048 7.7 / 7.6,
 // 2048x2048 3.6 / 3.4, 4096x4096 6.0 / 5.1, 2048x8192 7.6 / 6.4, 10240x8192 15.3 / 13.9; two tokens 512x1024 3.2 / 3.3,
-// 14336x1024 6.6 / 6.8, 512x2048 3.9 / 3.3, 4096x4096 7.3 / 5.2, 10240x8192 16.8 / 14.3.
+// 14336x1024 6.6 / 6.8, 512x2048 3.9 / 3.3, 4096x4096 7.3 / 5.2, 10240x8192 16.8 / 14.3.  One token and K = 2048 stay
+// fused: between products of other shapes the gain is gone (eight 1b blocks 190 us, 192 with every rotation separate) and
+// the step has half as many launches.
 bool linear_fused_eligible(const higgs_desc& d, int64_t B) {
-    return !(d.K >= 2048 && d.N * d.K * B >= ((int64_t)1 << 21)) && linear_fused_possible(d, B);
+    return !(d.K * B >= 4096 && d.N * d.K * B >= ((int64_t)1 << 21)) && linear_fused_possible(d, B);
 }
 
 // y_mode: 0 store fp32, 1 store bf16, 2 atomicAdd fp32 (target must be zero).  B <= 16.
