@@ -312,7 +312,7 @@ static int linear_tail(const higgs_desc* d, const __half* xdag, int64_t B, const
 }
 
 static int linear_args(const higgs_desc* d, int64_t B, const void* x, const void* packed, const void* scales,
-                       const float* grid, void* y, int y_dtype, void* workspace, size_t workspace_bytes) {
+                       const float* grid, void* y, int y_dtype, void* workspace, size_t workspace_bytes, bool may_lack_workspace = false) {
     int rc = check_desc(d);
     if (rc != HIGGS_OK) return rc;
     if (y_dtype != HIGGS_F32 && y_dtype != HIGGS_BF16) return HIGGS_ERR_UNSUPPORTED;
@@ -322,14 +322,14 @@ static int linear_args(const higgs_desc* d, int64_t B, const void* x, const void
     if (!x || !packed || !scales || !grid || !y) return HIGGS_ERR_INVALID_ARG;
     if (!aligned(x, 16) || !aligned(packed, 16) || !aligned(scales, 16) || !aligned(workspace, 256) || !aligned(y, 16))
         return HIGGS_ERR_INVALID_ARG;
-    if (!workspace) return !tc_eligible(*d, B) && linear_fused_eligible(*d, B) ? HIGGS_OK : HIGGS_ERR_INVALID_ARG;
+    if (!workspace) return may_lack_workspace && !tc_eligible(*d, B) && linear_fused_eligible(*d, B) ? HIGGS_OK : HIGGS_ERR_INVALID_ARG;
     if (workspace_bytes < higgs_workspace_bytes(d, HIGGS_OP_LINEAR, B)) return HIGGS_ERR_WORKSPACE;
     return HIGGS_OK;
 }
 
 int higgs_linear(const higgs_desc* d, const void* x, int64_t B, const void* packed, const void* scales,
                  const float* grid, void* y, int y_dtype, void* workspace, size_t workspace_bytes, void* stream) {
-    int rc = linear_args(d, B, x, packed, scales, grid, y, y_dtype, workspace, workspace_bytes);
+    int rc = linear_args(d, B, x, packed, scales, grid, y, y_dtype, workspace, workspace_bytes, true);
     if (rc != HIGGS_OK) return rc < 0 ? HIGGS_OK : rc;
     cudaStream_t st = as_stream(stream);
     if (tc_eligible(*d, B)) {

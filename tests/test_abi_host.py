@@ -171,3 +171,18 @@ def test_encoder_table_queries_and_arguments():
     assert L.higgs_quantize_prepared(P, a, hb.HIGGS_BF16, a, a, a, a, None, a, 16, None) == hb.HIGGS_ERR_WORKSPACE
     empty = hb.make_desc(2, 256, 0, 4096, 1)
     assert L.higgs_quantize_prepared(ctypes.byref(empty), None, hb.HIGGS_BF16, None, None, None, None, None, None, 0, None) == hb.HIGGS_OK
+
+
+def test_only_the_plain_product_runs_without_a_workspace():
+    """higgs_linear needs no workspace where it is one launch; the other entry points always want theirs."""
+    L = binding.lib
+    a = ctypes.c_void_p(0x1000)
+    dst = (ctypes.c_void_p * 1)(0x1000)
+    d = hb.make_desc(2, 256, 512, 1024, 1)
+    P = ctypes.byref(d)
+    assert hb.higgs_linear_launch_count(d, 1) == 1
+    assert L.higgs_linear_share(P, a, 1, a, a, a, a, 0, a, None, 0, None) == hb.HIGGS_ERR_INVALID_ARG
+    assert L.higgs_linear_prerotated(P, a, 1, a, a, a, a, 0, None, 0, None) == hb.HIGGS_ERR_INVALID_ARG
+    assert L.higgs_linear_gather(P, a, 1, a, a, a, dst, 1, 512, 0, 0, None, 0, None) == hb.HIGGS_ERR_INVALID_ARG
+    assert L.higgs_linear_kshard(P, a, 1, a, a, a, dst, 1, 0, None, 0, None) == hb.HIGGS_ERR_INVALID_ARG
+    assert L.higgs_linear(P, a, 3, a, a, a, a, 0, None, 0, None) == hb.HIGGS_ERR_INVALID_ARG          # two launches
