@@ -186,3 +186,34 @@ def test_only_the_plain_product_runs_without_a_workspace():
     assert L.higgs_linear_gather(P, a, 1, a, a, a, dst, 1, 512, 0, 0, None, 0, None) == hb.HIGGS_ERR_INVALID_ARG
     assert L.higgs_linear_kshard(P, a, 1, a, a, a, dst, 1, 0, None, 0, None) == hb.HIGGS_ERR_INVALID_ARG
     assert L.higgs_linear(P, a, 3, a, a, a, a, 0, None, 0, None) == hb.HIGGS_ERR_INVALID_ARG          # two launches
+
+
+def test_replaced_functions_show_through_the_package(monkeypatch):
+    """A name of the binding that is replaced, removed or defined anew is what the package gives from then on."""
+    original = hb.higgs_sign                                 # (the package has taken it over now)
+    for fake in (lambda *a: 7, lambda *a: 8):
+        with monkeypatch.context() as m:
+            m.setattr(binding, "higgs_sign", fake)
+            assert hb.higgs_sign(1, 2) == binding.higgs_sign(1, 2) == fake()
+        assert hb.higgs_sign is original
+    with monkeypatch.context() as m:
+        m.delattr(binding, "higgs_sign")
+        assert not hasattr(hb, "higgs_sign")
+    assert hb.higgs_sign is original
+    with monkeypatch.context() as m:
+        m.setattr(hb, "higgs_sign", min)                     # set on the package itself: stays
+        binding.a_new_name = 1
+        del binding.a_new_name
+        assert hb.higgs_sign is min
+    assert hb.higgs_sign is original
+
+
+def test_a_reloaded_binding_shows_through_the_package():
+    import subprocess
+    import sys
+    code = ("import importlib, paper_2411_17525_b200 as hb\n"
+            "from paper_2411_17525_b200 import binding\n"
+            "old = hb.higgs_sign\n"
+            "importlib.reload(binding)\n"
+            "assert hb.higgs_sign is binding.higgs_sign is not old\n")
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT)
