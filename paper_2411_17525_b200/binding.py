@@ -176,13 +176,17 @@ def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else t.data_ptr()
 
 
-_raw_stream, _current_device, _cuda_ready = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice, False
+# (what torch.cuda.current_stream() itself asks; a torch that lacks them, one built without CUDA for instance, is asked for the object)
+_raw_stream, _current_device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+_cuda_ready = False
 
 
 def _stream() -> int:
     """The current stream of the current device (0.2 us; a torch.cuda.Stream object takes 3.4)."""
     global _cuda_ready
     if not _cuda_ready:
+        if _raw_stream is None or _current_device is None:
+            return torch.cuda.current_stream().cuda_stream
         torch.cuda.init()
         _cuda_ready = True
     return _raw_stream(_current_device())

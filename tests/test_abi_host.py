@@ -3,6 +3,8 @@
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -209,11 +211,21 @@ def test_replaced_functions_show_through_the_package(monkeypatch):
 
 
 def test_a_reloaded_binding_shows_through_the_package():
-    import subprocess
-    import sys
     code = ("import importlib, paper_2411_17525_b200 as hb\n"
             "from paper_2411_17525_b200 import binding\n"
             "old = hb.higgs_sign\n"
             "importlib.reload(binding)\n"
             "assert hb.higgs_sign is binding.higgs_sign is not old\n")
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT)
+
+
+def test_a_torch_without_the_raw_stream_functions():
+    """Two functions of torch that are no public ones save time; without them the binding loads and asks for the stream object."""
+    code = ("import torch, types\n"
+            "del torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice\n"
+            "import paper_2411_17525_b200 as hb\n"
+            "from paper_2411_17525_b200 import binding\n"
+            "assert hb.higgs_sign(1, 2) in (-1, 1)\n"
+            "torch.cuda.current_stream = lambda: types.SimpleNamespace(cuda_stream=77)\n"
+            "assert binding._stream() == 77\n")
     subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT)
