@@ -248,6 +248,61 @@ __device__ __forceinline__ void fwht1024_from_columns(float (&v)[32], float* ex,
     butterflies32(v);
 }
 
+// One 1024-group rotated by the four warps of a block, for calls too small to fill the GPU: there the length of one warp's chain
+// is what counts, and a lane holds 8 values here instead of 32.  Warp q owns inputs 256 q .. + 255; `src` is this lane's
+// eight of them, k0 the first one's index; v = the lane's outputs times 32.  Index bits 0 to 2 are butterflies in registers, 3 to 7
+// shuffles, 8 and 9 meet in shared memory: LANES_FIRST adds up in the order of the small-batch kernel's own rotation,
+// otherwise in that of fwht1024_warp, bit for bit.  All four warps call it.
+template <bool LANES_FIRST>
+__device__ __forceinline__ void rotate_by_four_warps(const __nv_bfloat16* src, uint64_t xi, int64_t k0, float (*ex)[256], int q, int lane, float (&v)[8]) {
+    const uint4 q4 = __ldcg(reinterpret_cast<const uint4*>(src));
+    const uint32_t w4[4] = {q4.x, q4.y, q4.z, q4.w};
+    const uint32_t bits = (uint32_t)(sign_word(xi, (uint64_t)k0 >> 6) >> ((uint64_t)k0 & 63ull)) & 0xffu;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        v[2 * e] = __uint_as_float((w4[e] << 16) ^ (((bits >> (2 * e)) & 1u) << 31));
+        v[2 * e + 1] = __uint_as_float((w4[e] & 0xffff0000u) ^ (((bits >> (2 * e + 1)) & 1u) << 31));
+    }
+    auto over_lanes = [&]() {
+#pragma unroll
+        for (int m = 1; m < 32; m <<= 1) {
+            const bool upper = (lane & m) != 0;
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                const float u = __shfl_xor_sync(0xffffffffu, v[r], m);
+                v[r] = upper ? (u - v[r]) : (v[r] + u);
+            }
+        }
+    };
+#pragma unroll
+    for (int h = 1; h < 8; h <<= 1) {
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            if ((r & h) == 0) { const float a = v[r], c = v[r | h]; v[r] = a + c; v[r | h] = a - c; }
+        }
+    }
+    if (LANES_FIRST) over_lanes();
+    *reinterpret_cast<float4*>(&ex[q][lane * 8]) = make_float4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<float4*>(&ex[q][lane * 8 + 4]) = make_float4(v[4], v[5], v[6], v[7]);
+    __syncthreads();
+    const float s8 = (q & 1) ? -1.f : 1.f, s9 = (q & 2) ? -1.f : 1.f;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        float u[4][4];
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            const float4 f = *reinterpret_cast<const float4*>(&ex[w][lane * 8 + 4 * c]);
+            u[w][0] = f.x; u[w][1] = f.y; u[w][2] = f.z; u[w][3] = f.w;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {       // (products with +-1 are exact)
+            const float a = fmaf(s8, u[1][e], u[0][e]);
+            v[4 * c + e] = LANES_FIRST ? fmaf(s8 * s9, u[3][e], fmaf(s9, u[2][e], a)) : fmaf(s9, fmaf(s8, u[3][e], u[2][e]), a);
+        }
+    }
+    if (!LANES_FIRST) over_lanes();
+}
+
 // Sign bits of this lane's 32 elements c*256 + l*8 + e of the group at input k0, bit c*8 + e of the result; and a value
 // with its sign flipped where bit r is set.
 __device__ __forceinline__ uint32_t lane_sign_bits(uint64_t xi, int64_t k0, int lane) {
@@ -339,6 +394,7 @@ int launch_linear_mma(const higgs_desc& d, const __half* xdag, int64_t B, const 
                       const GatherTargets* more = nullptr, __half* xdag_emit = nullptr, const MultiSegments* segs = nullptr);
 int launch_scatter_out(const float* y32, int64_t B, int64_t N, void* const* dsts, int n_dst, int64_t ldy, int y_dtype,
                        cudaStream_t st);
+bool linear_leaves_sms(const higgs_desc& d, int64_t B, int64_t blocks);
 bool linear_fused_possible(const higgs_desc& d, int64_t B);
 bool linear_fused_eligible(const higgs_desc& d, int64_t B);
 int launch_convert_out(const float* y32, void* y, int y_dtype, size_t count, cudaStream_t st);

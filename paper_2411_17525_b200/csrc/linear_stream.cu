@@ -993,6 +993,11 @@ bool linear_uses_atomics(const higgs_desc& d, int64_t B) {
     return pl.chunks > 1 && !pl.pair;
 }
 
+// Whether `blocks` further blocks find SMs that the small-batch product leaves free.
+bool linear_leaves_sms(const higgs_desc& d, int64_t B, int64_t blocks) {
+    return d.N > 0 && blocks < sm_count() && make_plan(d, B > 16 ? 16 : B).blocks + blocks <= sm_count();
+}
+
 // The rotation can be fused into the product kernel for one or two tokens when every block owns whole 1024-groups and
 // the K ranges do not meet in atomics (one chunk, or the two chunks of a cluster pair).
 bool linear_fused_possible(const higgs_desc& d, int64_t B) {

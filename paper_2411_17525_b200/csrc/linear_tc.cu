@@ -754,6 +754,31 @@ __global__ void __launch_bounds__(kRotWarps * 32) rht_activations_tc_kernel(cons
     }
 }
 
+// The same with four warps per (token, group), a block each.  A padding token of the layout gets its zeros from the block of a
+// token of the batch (blocks of their own would crowd out those that have work).
+__global__ void __launch_bounds__(128) rht_activations_tc_wide_kernel(const __nv_bfloat16* x, __half* __restrict__ xdag, int B, int K,
+                                                                      uint64_t xi, int BN, int padded) {
+    __shared__ __align__(16) float ex[4][256];
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    const int groups = K / kGroup, b = (int)blockIdx.x / groups, k0 = (int)blockIdx.x % groups * kGroup + q * 256 + lane * 8;
+    auto place = [&](int token) {
+        const int tile = token / BN, t = token % BN;
+        return reinterpret_cast<uint4*>(xdag + ((int64_t)tile * (K / 64) + k0 / 64) * BN * 64 + (t / 8) * 512 + ((k0 % 64) / 8) * 64 + (t % 8) * 8);
+    };
+    pdl_trigger();
+    pdl_wait();
+    float v[8];
+    rotate_by_four_warps<false>(x + (int64_t)b * K + k0, xi, k0, ex, q, lane, v);
+    uint32_t w[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const __half2 h = __floats2half2_rn(v[2 * e] * 0.03125f, v[2 * e + 1] * 0.03125f);
+        w[e] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    *place(b) = make_uint4(w[0], w[1], w[2], w[3]);
+    for (int token = b + B; token < padded; token += B) *place(token) = make_uint4(0u, 0u, 0u, 0u);
+}
+
 }  // namespace
 
 // Token-tile width of the tensor-core path for batch B: a multiple of 16, at most 256, balanced over the tiles.
@@ -779,12 +804,36 @@ size_t tc_workspace_bytes(const higgs_desc& d, int64_t B) {
     return (size_t)tiles * BN * d.K * 2;
 }
 
+static int tc_sms() {
+    static int cached[64] = {0};
+    return device_once(cached, [] {
+        int dev = 0, n = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
+        return n;
+    });
+}
+
+// Calls whose rotation takes four warps per group: the product leaves SMs free and its own time does not hide the rotation's start
+// (few blocks, short K), and the rotation's blocks fit the free SMs once or twice.  Chains of one layer, eight warps per
+// block / four warps per group in us: 512x1024 with 17 tokens 6.4 / 5.7, with 200 11.3 / 10.7, 2048x2048 with 64 7.7 / 7.2, 256x4096
+// with 24 6.7 / 6.1, 2048x3072 with 48 9.1 / 7.9; beyond the line 2048x2048 with 100 9.1 / 9.4, 256x4096 with 128 9.9 / 11.6,
+// 2560x4096 with 17 7.2 / 7.5, 4096x1024 with 256 12.4 / 13.1.
+static bool tc_rotation_is_small(const higgs_desc& d, int64_t B) {
+    const int64_t sms = tc_sms(), groups = d.K / kGroup;
+    if (groups > 4 || B * groups > 2 * sms) return false;
+    const int64_t product = d.N / 128 * tc_k_split(d, B) * ((B + tc_batch_tile(B) - 1) / tc_batch_tile(B));
+    return product <= sms * 2 / 3 && product * groups <= sms * 4 / 3 && product + B * groups <= sms * 7 / 4;
+}
+
 // D1 for the tensor-core path: rotated activations in the blocked operand layout (tc_workspace_bytes() bytes).
 int launch_rht_tc(const higgs_desc& d, const void* x, int64_t B, __half* xdag_tc, cudaStream_t st) {
     const int BN = tc_batch_tile(B);
     const int64_t tiles = (B + BN - 1) / BN;
     const int64_t blocks = tiles * (BN / 8) * (d.K / kGroup);          // one per (token block, group)
     if (blocks > 0x7fffffff) return HIGGS_ERR_UNSUPPORTED;
+    if (tc_rotation_is_small(d, B))
+        return cuda_status(launch_pdl(rht_activations_tc_wide_kernel, dim3((unsigned)(B * (d.K / kGroup))), dim3(128), 0, st,
+                                      static_cast<const __nv_bfloat16*>(x), xdag_tc, (int)B, (int)d.K, d.rht_seed, BN, (int)(tiles * BN)));
     return cuda_status(launch_pdl(rht_activations_tc_kernel, dim3((unsigned)blocks), dim3(kRotWarps * 32), 0, st,
                                   static_cast<const __nv_bfloat16*>(x), xdag_tc, B, d.K, d.rht_seed, BN));
 }
@@ -797,15 +846,6 @@ int tc_k_split(const higgs_desc& d, int64_t B) {
     int ks = 1;
     while (ks < kTcMaxSplit && tiles * (ks * 2) <= 128 && d.K % (256 * ks * 2) == 0 && d.K / (ks * 2) >= 512) ks *= 2;
     return ks;
-}
-
-static int tc_sms() {
-    static int cached[64] = {0};
-    return device_once(cached, [] {
-        int dev = 0, n = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
-        return n;
-    });
 }
 
 // The product's own token tile when K is not split: narrower tiles than the layout's may fill the last wave of blocks better.

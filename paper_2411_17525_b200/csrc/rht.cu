@@ -136,6 +136,33 @@ __global__ void __launch_bounds__(32) rht_activations_kernel(const __nv_bfloat16
     }
 }
 
+// The same with four warps per (token, group), for layers that leave SMs free: there a block needs no room beside a product block,
+// and what counts is how long one group takes.  Chains of one layer, one warp / four warps in us: 2048x1024 with 12 tokens
+// 4.1 / 3.6, 256x8192 with one 3.2 / 3.05, 512x3072 with two 3.4 / 3.15; where a block finds no free SM: 2560x1024 with three 3.8 /
+// 4.1, 4096x4096 with four 5.7 / 8.8.
+__global__ void __launch_bounds__(128) rht_activations_wide_kernel(const __nv_bfloat16* x, __half* __restrict__ xdag, int64_t B, int64_t K,
+                                                                   uint64_t xi, float* __restrict__ zero_ptr, size_t zero_floats) {
+    __shared__ __align__(16) float ex[4][256];
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    const unsigned groups = (unsigned)(K / kGroup), gi = blockIdx.x % groups;
+    pdl_trigger();
+    const int64_t b = blockIdx.x / groups, k0 = (int64_t)gi * kGroup + q * 256 + lane * 8;       // this lane's 8 consecutive inputs
+    pdl_wait();
+    for (size_t i = (size_t)blockIdx.x * 128 + threadIdx.x; i < zero_floats; i += (size_t)gridDim.x * 128) zero_ptr[i] = 0.0f;
+    if (b >= B) return;
+    float o[8];
+    rotate_by_four_warps<true>(x + b * K + k0, xi, k0, ex, q, lane, o);
+    // this lane holds pairs 4 j + i (i = 0..3, j = lane % 8) of 64-input block q*4 + lane/8 of the group, i.e.
+    // m = j >> 1, h = j & 1, t = i  ->  position i*8 + j
+    uint32_t* blk = reinterpret_cast<uint32_t*>(xdag + b * K + (int64_t)gi * kGroup) + (q * 4 + (lane >> 3)) * 32;
+    const int j = lane & 7;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const __half2 hh = __floats2half2_rn(o[2 * e] * 0.03125f, o[2 * e + 1] * 0.03125f);
+        blk[e * 8 + j] = *reinterpret_cast<const uint32_t*>(&hh);
+    }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256) rht_debug_kernel(const T* __restrict__ x, float* __restrict__ out,
                                                         int64_t rows, int64_t K, uint64_t xi, float mul) {
@@ -163,11 +190,18 @@ __global__ void __launch_bounds__(256) rht_debug_kernel(const T* __restrict__ x,
 int launch_rht_activations(const higgs_desc& d, const void* x, int64_t B, __half* xdag, float* zero_ptr,
                            size_t zero_floats, cudaStream_t st) {
     int64_t blocks = B * (d.K / kGroup);
+    // (a block of four warps finds an SM of its own beside the product's blocks; above 16 tokens several products follow: 1040x2048 with
+    // 32 8.4 / 9.3)
+    const bool wide = B <= 16 && linear_leaves_sms(d, B, blocks);
+    const int threads = wide ? 128 : 32;
     if (zero_floats) {
-        int64_t zb = (int64_t)((zero_floats + 32 * 8 - 1) / (32 * 8));
+        int64_t zb = (int64_t)((zero_floats + threads * 8 - 1) / (threads * 8));
         if (zb > 1184) zb = 1184;
         if (zb > blocks) blocks = zb;
     }
+    if (wide)
+        return cuda_status(launch_pdl(rht_activations_wide_kernel, dim3((unsigned)blocks), dim3(128), 0, st,
+                                      static_cast<const __nv_bfloat16*>(x), xdag, B, d.K, d.rht_seed, zero_ptr, zero_floats));
     return cuda_status(launch_pdl(rht_activations_kernel, dim3((unsigned)blocks), dim3(32), 0, st,
                                   static_cast<const __nv_bfloat16*>(x), xdag, B, d.K, d.rht_seed, zero_ptr, zero_floats));
 }
