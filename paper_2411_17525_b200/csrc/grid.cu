@@ -384,7 +384,8 @@ __global__ void __launch_bounds__(kFitThreads, 1) grid_fit_kernel(GridWs w, cons
                     }
                 }
                 const unsigned wb = __reduce_min_sync(0xffffffffu, __float_as_uint(b));        // (not negative: ordered as integers)
-                const int to = (int)__reduce_min_sync(0xffffffffu, __float_as_uint(b) == wb ? (unsigned)bi : 0x7fffffffu);
+                int to = (int)__reduce_min_sync(0xffffffffu, __float_as_uint(b) == wb ? (unsigned)bi : 0x7fffffffu);
+                if (to >= n) to = 0;               // no distance compared below infinity (NaN, or squares that overflow): index 0, as a plain scan
                 const unsigned ws = __reduce_min_sync(0xffffffffu, __float_as_uint(bi == to ? s2 : b));
                 if (lane == 0) {
                     settle(i, y, a, to, fminf(__fsqrt_rd(__fmul_rd(__uint_as_float(ws), 0.999996f)), beyond));

@@ -52,3 +52,14 @@ def test_fit_follows_the_plain_iteration(p, n, m, max_iters):
     assert np.max(np.abs(grid.cpu().numpy() - want)) <= 2.0 ** -22              # an fp32 rounding of a mean of size <= 4
     assert abs(float(mse) - err / (m * p)) <= 1e-6 * err / (m * p) + 1e-30
     assert torch.equal(grid, again)
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), -float("inf"), 1e30])
+@pytest.mark.parametrize("p,n,m", [(1, 16, 300), (2, 256, 4133), (2, 600, 5000), (4, 40, 333)])
+def test_samples_without_a_nearest_centre(p, n, m, bad):
+    """A sample whose distances are all NaN or infinite belongs to cell 0, whichever way it is scanned."""
+    x = np.random.default_rng(n).standard_normal((m, p)).astype(np.float32)
+    x[n + 3, p - 1] = x[m - 1, 0] = bad
+    _, _, it = hb.higgs_make_grid(p, n, torch.from_numpy(x).to(U.dev()), max_iters=12)
+    assert hb.higgs_device_status() == hb.HIGGS_OK
+    assert 1 <= abs(int(it)) <= 12
