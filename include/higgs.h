@@ -150,11 +150,14 @@ int higgs_make_uniform_grid(int n, float* grid_out, float* step_out, float* mse_
  *                the samples
  *   iters_out    device, optional: iterations run (int32), negative if
  *                max_iters was reached without convergence
- * Distances are fp32, sums 64-bit fixed point with a resolution of 2^-62
- * times num_samples times the largest |coordinate| (exact for N(0, 1) samples
- * but the tiniest), independent of the order of summation; the result is a fixed
- * point of the same iteration the fp64 definition runs but need not be
- * bit-identical to it.
+ * Distances are fp32, sums 64-bit fixed point in steps of 2^-62 times
+ * num_samples times the largest |coordinate|, both rounded up to powers of two
+ * (exact for N(0, 1) samples but the tiniest), independent of the order of
+ * summation.  Sample sets whose range that does not suit (more than one sample in
+ * 32 would be rounded, magnitudes of 2^61 and more, none above 2^-40, infinities, NaN) are summed in
+ * fp64; a sample whose distances all are NaN or infinite belongs to centre 0.  The
+ * result is a fixed point of the same iteration the fp64 definition runs but need
+ * not be bit-identical to it.
  * 1 <= p <= 4 and 1 <= n <= 4096 (n need not be a power of two), else
  * HIGGS_ERR_UNSUPPORTED.
  */

@@ -21,9 +21,9 @@ struct GridWs {
     float* centres;               // [n][p]
     long long* delta;             // [3][n][p] changes of the cells' sums, fixed point
     int32_t* delta_cnt;           // [3][n]    changes of the cells' sizes
-    double* err;                  // [kMaxFitBlocks] squared error of a block's samples
+    double* err;                  // [kMaxFitBlocks] squared error of a block's samples; before the fit the range of the samples, as uint2
     unsigned long long* bar;      // [2] grid barrier: arrivals (low half), blocks with a changed assignment (high half)
-    int32_t* flags;               // [0] done, [1] iterations, [2] bits of the largest |sample|
+    int32_t* flags;               // [0] done, [1] iterations, [2] the samples are left to plain_fit_kernel
     uint16_t* near_idx;           // [kMaxNearCentres][kNear] neighbour lists
     float* excl;                  // [kMaxNearCentres]
     int32_t* assign;              // [m]
@@ -48,13 +48,80 @@ GridWs carve(void* ws, int p, int n, int64_t m) {
     return w;
 }
 
-__global__ void grid_init_kernel(GridWs w, int p, int n, int64_t m) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < m) w.assign[i] = -1;
-    if (i < (int64_t)3 * n * p) w.delta[i] = 0;
-    if (i < 3 * n) w.delta_cnt[i] = 0;
-    if (i < 2) w.bar[i] = 0;
-    if (i < 4) w.flags[i] = 0;
+// Also the bits of the largest |coordinate| among a block's samples.
+constexpr int kRangeThreads = 256;
+__global__ void __launch_bounds__(kRangeThreads) grid_init_kernel(GridWs w, const float* __restrict__ samples, int p, int n, int64_t m) {
+    __shared__ unsigned s_top[kRangeThreads / 32];
+    const int64_t first = (int64_t)blockIdx.x * kRangeThreads + threadIdx.x, step = (int64_t)gridDim.x * kRangeThreads;
+    for (int64_t i = first; i < (int64_t)3 * n * p; i += step) w.delta[i] = 0;
+    for (int64_t i = first; i < 3 * n; i += step) w.delta_cnt[i] = 0;
+    if (first < 2) w.bar[first] = 0;
+    if (first < 8) w.flags[first] = 0;
+    unsigned top = 0u;
+    for (int64_t i = first; i < m; i += step) {
+        w.assign[i] = -1;
+        for (int k = 0; k < p; ++k) top = max(top, __float_as_uint(fabsf(samples[i * p + k])));
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((threadIdx.x & 31) == 0) s_top[threadIdx.x >> 5] = top;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < kRangeThreads / 32; ++i) top = max(top, s_top[i]);
+        reinterpret_cast<uint2*>(w.err)[blockIdx.x] = make_uint2(top, 0u);
+    }
+}
+
+// The scale of the fixed-point sums, 2^shift: m times the largest |coordinate|, below 2^(exponent - 126), stays below 2^62.
+__device__ __forceinline__ int sum_shift(unsigned top, int64_t m) { return 62 - (m > 1 ? 64 - __clzll(m - 1) : 0) - (max((int)(top >> 23), 1) - 126); }
+__device__ __forceinline__ double power_of_two(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+// The largest |coordinate| over all blocks (slots at most kFitThreads, one per thread of a block of 32 warps at most).
+__device__ __forceinline__ uint2 range_of(const GridWs& w, int slots) {
+    __shared__ unsigned s_top, s_rounded;
+    if (threadIdx.x == 0) s_top = s_rounded = 0u;
+    __syncthreads();
+    unsigned top = 0u, rounded = 0u;
+    for (int i = threadIdx.x; i < slots; i += blockDim.x) {
+        const uint2 r = reinterpret_cast<const uint2*>(w.err)[i];
+        top = max(top, r.x);
+        rounded += r.y;
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    rounded = __reduce_add_sync(0xffffffffu, rounded);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&s_top, top);
+        atomicAdd(&s_rounded, rounded);
+    }
+    __syncthreads();
+    return make_uint2(s_top, s_rounded);
+}
+
+// The number of a block's samples with a coordinate that the fixed-point sums round.  (Same grid as grid_init_kernel; a block
+// writes only the second half of its slot.)
+__global__ void __launch_bounds__(kRangeThreads) grid_range_kernel(GridWs w, const float* __restrict__ samples, int p, int64_t m, int slots) {
+    const double scale = power_of_two(sum_shift(range_of(w, slots).x, m));
+    unsigned rounded = 0u;
+    for (int64_t i = (int64_t)blockIdx.x * kRangeThreads + threadIdx.x; i < m; i += (int64_t)gridDim.x * kRangeThreads) {
+        bool exact = true;
+        for (int k = 0; k < p; ++k) {
+            const double v = (double)samples[i * p + k] * scale;
+            exact = exact && rint(v) == v;
+        }
+        rounded += exact ? 0u : 1u;
+    }
+    __shared__ unsigned s_count;
+    if (threadIdx.x == 0) s_count = 0u;
+    __syncthreads();
+    rounded = __reduce_add_sync(0xffffffffu, rounded);
+    if ((threadIdx.x & 31) == 0 && rounded) atomicAdd(&s_count, rounded);
+    __syncthreads();
+    if (threadIdx.x == 0) reinterpret_cast<uint2*>(w.err)[blockIdx.x].y = s_count;
+}
+
+// Whether a sample set is left to plain_fit_kernel: more than one sample in 32 would be rounded (an outlier of 2^16 among 2^18
+// samples of N(0, I) rounds those below 2^-5, one in 40; a coordinate of 2^(23 - shift) or more is exact, so a mean beyond that is
+// off by half an ulp at most), or squares and their sums may leave the normal fp32 range, on which the bounds rely.
+__device__ __forceinline__ bool range_unsuited(uint2 range, int64_t m) {
+    return (range.x >> 23) >= 127 + 61 || (range.x >> 23) < 127 - 40 || range.y > (unsigned)(m >> 5);
 }
 
 // Every block is resident (a cooperative launch, or one block), so the blocks can meet at a barrier: a counter in the
@@ -104,6 +171,95 @@ __device__ __forceinline__ float centre_distance(const float (&x)[P], const floa
     return d;
 }
 
+// The nearest of all centres; centre 0 when no distance compares below infinity.
+template <int P>
+__device__ __forceinline__ int nearest_centre(const float (&x)[P], const float* sc, int n, float& best) {
+    int bi = 0;
+    best = INFINITY;
+#pragma unroll 4
+    for (int q = 0; q < n; ++q) {
+        const float d = centre_distance<P>(x, sc + q * P);
+        if (d < best) { best = d; bi = q; }
+    }
+    return bi;
+}
+
+// What grid_finalize_kernel reads: this block's share of the squared error, and from block 0 the rest.
+__device__ __forceinline__ void write_result(const GridWs& w, const float* sc, int coords, double err, bool done, int it, double* s_err) {
+    const int tid = threadIdx.x;
+#pragma unroll
+    for (int k = 16; k > 0; k >>= 1) err += __shfl_xor_sync(0xffffffffu, err, k);
+    if ((tid & 31) == 0) s_err[tid >> 5] = err;
+    __syncthreads();
+    if (tid == 0) {
+        double total = 0.0;
+        for (int i = 0; i < kFitThreads / 32; ++i) total += s_err[i];
+        w.err[blockIdx.x] = total;
+        if (blockIdx.x == 0) { w.flags[0] = done ? 1 : 0; w.flags[1] = it; }
+    }
+    if (blockIdx.x == 0)
+        for (int i = tid; i < coords; i += kFitThreads) w.centres[i] = sc[i];
+}
+
+// The iteration as it stands, without bounds and with fp64 sums over all samples, for the sample sets that grid_fit_kernel leaves
+// untouched (it is launched after that kernel every time; a kernel of its own because a call in there takes registers from the
+// other path: 2 % of its time).  The sums of an iteration are in w.delta (as doubles), three buffers in turn as there.
+template <int P>
+__global__ void __launch_bounds__(kFitThreads, 1) plain_fit_kernel(GridWs w, const float* __restrict__ samples, int n, int64_t m, int max_iters) {
+    if (!w.flags[2]) return;
+    extern __shared__ __align__(16) unsigned char grid_smem[];
+    double* block_sums = reinterpret_cast<double*>(grid_smem);         // [n][P]
+    float* sc = reinterpret_cast<float*>(block_sums + (size_t)n * P);  // [n][P]
+    int* block_cnt = reinterpret_cast<int*>(sc + (size_t)n * P);       // [n]
+    __shared__ double s_err[kFitThreads / 32];
+    const int tid = threadIdx.x, blocks = (int)gridDim.x;
+    const int64_t first = ((int64_t)(tid >> 5) * blocks + blockIdx.x) * 32 + (tid & 31), step = (int64_t)blocks * kFitThreads;
+    unsigned seen[2] = {0u, 0u};
+    double err = 0.0;
+    int it = 0;
+    bool done = false, ok;
+    for (int i = tid; i < n * P; i += kFitThreads) sc[i] = samples[i];
+    for (; it < max_iters; ++it) {
+        for (int i = tid; i < n * P; i += kFitThreads) block_sums[i] = 0.0;
+        for (int i = tid; i < n; i += kFitThreads) block_cnt[i] = 0;
+        __syncthreads();
+        err = 0.0;
+        int changed = 0;
+        for (int64_t i = first; i < m; i += step) {
+            float x[P], best;
+#pragma unroll
+            for (int k = 0; k < P; ++k) x[k] = samples[i * P + k];
+            const int to = nearest_centre<P>(x, sc, n, best);
+            if (w.assign[i] != to) { w.assign[i] = to; changed = 1; }
+            err += (double)best;
+#pragma unroll
+            for (int k = 0; k < P; ++k) atomicAdd(&block_sums[to * P + k], (double)x[k]);
+            atomicAdd(&block_cnt[to], 1);
+        }
+        const bool block_changed = __syncthreads_or(changed) != 0;
+        double* sums = reinterpret_cast<double*>(w.delta) + (size_t)(it % 3) * n * P;
+        int32_t* cnt = w.delta_cnt + (size_t)(it % 3) * n;
+        for (int i = tid; i < n * P; i += kFitThreads)
+            if (block_cnt[i / P]) atomicAdd(&sums[i], block_sums[i]);
+        for (int i = tid; i < n; i += kFitThreads)
+            if (block_cnt[i]) atomicAdd(&cnt[i], block_cnt[i]);
+        const bool any = grid_barrier(w.bar, it, blocks, block_changed, seen[it & 1], &ok);
+        if (!ok) return;
+        if (!any) { done = true; ++it; break; }
+        for (int i = tid; i < n * P; i += kFitThreads) {
+            const int size = __ldcg(&cnt[i / P]);
+            if (size > 0) sc[i] = (float)(__ldcg(&sums[i]) / (double)size);      // (an empty cell keeps its centre)
+        }
+        if (blockIdx.x == 0) {
+            const int old = (it + 2) % 3;
+            for (int i = tid; i < n * P; i += kFitThreads) w.delta[(size_t)old * n * P + i] = 0;
+            for (int i = tid; i < n; i += kFitThreads) w.delta_cnt[(size_t)old * n + i] = 0;
+        }
+        __syncthreads();
+    }
+    write_result(w, sc, n * P, err, done, it, s_err);
+}
+
 __host__ __device__ inline bool fit_lists(int n) { return n >= kMinNearCentres && n <= kMaxNearCentres; }
 inline size_t fit_smem(int p, int n) {
     return (size_t)n * p * (sizeof(long long) + sizeof(float)) + (size_t)n * sizeof(int) +
@@ -125,7 +281,8 @@ inline size_t fit_smem(int p, int n) {
 //     one at a time; many scans are done one per lane.
 //   * Update.  Only samples that changed cell touch the sums.  The sums are 64-bit fixed point, scaled so that m times the
 //     largest |coordinate| stays below 2^62: for N(0, I) samples all but the tiniest coordinates are represented
-//     exactly, and integer sums do not depend on the order of the atomics.  Every block adds the iteration's changes to
+//     exactly, and integer sums do not depend on the order of the atomics.  (Sample sets that this does not suit go to
+//     plain_fit_kernel.)  Every block adds the iteration's changes to
 //     its own copy of the sums and computes the new centres itself, so no second barrier is needed.  Three buffers take
 //     turns: the changes of iteration i are read after its barrier; block 0 clears those of i - 1, which every block has
 //     read before it arrived there, for iteration i + 2.
@@ -133,7 +290,7 @@ inline size_t fit_smem(int p, int n) {
 // p = 2, n = 256, 2^18 samples: 37 -> 9 us per iteration (before: every sample scanned all centres every time, sums by
 // fp64 atomics in shared memory, two barriers).  One barrier and movement bounds without lists: 12.4 us.
 template <int P>
-__global__ void __launch_bounds__(kFitThreads, 1) grid_fit_kernel(GridWs w, const float* __restrict__ samples, int n, int64_t m, int max_iters) {
+__global__ void __launch_bounds__(kFitThreads, 1) grid_fit_kernel(GridWs w, const float* __restrict__ samples, int n, int64_t m, int slots, int max_iters) {
     extern __shared__ __align__(16) unsigned char grid_smem[];
     const bool shared_sums = n * P <= kMaxSharedSums, lists = fit_lists(n);
     long long* sums = reinterpret_cast<long long*>(grid_smem);         // [n][P]
@@ -167,24 +324,16 @@ __global__ void __launch_bounds__(kFitThreads, 1) grid_fit_kernel(GridWs w, cons
     if (tid < 2) s_move[tid] = 0u;
     if (tid < 2) s_queued[tid] = 0;
     int qi = 0;
-    // scale of the fixed-point sums
-    unsigned top = 0u;
-    for (int64_t c = chunk0; c < chunks; c += chunk_step) {
-        const int64_t i = c * 32 + lane;
-#pragma unroll
-        for (int k = 0; k < P; ++k)
-            if (i < m) top = max(top, __float_as_uint(fabsf(samples[i * P + k])));
+    const uint2 range = range_of(w, slots);
+    if (range_unsuited(range, m)) {
+        if (blockIdx.x == 0 && tid == 0) w.flags[2] = 1;
+        return;
     }
-    top = __reduce_max_sync(0xffffffffu, top);
-    if (lane == 0) atomicMax(reinterpret_cast<unsigned*>(&w.flags[2]), top);
+    const int shift = sum_shift(range.x, m);
+    const double scale = power_of_two(shift), unscale = power_of_two(-shift);
     int barrier_no = 0;
     unsigned seen[2] = {0u, 0u};
     bool ok;
-    grid_barrier(w.bar, barrier_no++, blocks, false, seen[0], &ok);
-    if (!ok) return;
-    top = (unsigned)__ldcg(&w.flags[2]);
-    const int shift = 62 - (m > 1 ? 64 - __clzll(m - 1) : 0) - (max((int)(top >> 23), 1) - 126);       // |sample| < 2^(exponent - 126)
-    const double scale = __hiloint2double((1023 + shift) << 20, 0), unscale = __hiloint2double((1023 - shift) << 20, 0);
 
     // scanning one sample: n steps of its lane, or ceil(n / 32) steps and a reduction of the whole warp
     const int scan_all = max(1, 9 * n / (9 * ((n + 31) / 32) + 45));
@@ -460,21 +609,10 @@ __global__ void __launch_bounds__(kFitThreads, 1) grid_fit_kernel(GridWs w, cons
             err += (double)centre_distance<P>(x, sc + w.assign[i] * P);
         }
     }
-#pragma unroll
-    for (int k = 16; k > 0; k >>= 1) err += __shfl_xor_sync(0xffffffffu, err, k);
-    if (lane == 0) s_err[warp] = err;
-    __syncthreads();
-    if (tid == 0) {
-        double total = 0.0;
-        for (int i = 0; i < kFitThreads / 32; ++i) total += s_err[i];
-        w.err[blockIdx.x] = total;
-        if (blockIdx.x == 0) { w.flags[0] = done ? 1 : 0; w.flags[1] = it; }
-    }
-    if (blockIdx.x == 0)
-        for (int i = tid; i < n * P; i += kFitThreads) w.centres[i] = sc[i];
+    write_result(w, sc, n * P, err, done, it, s_err);
 }
 
-__global__ void __launch_bounds__(256) grid_finalize_kernel(GridWs w, int p, int n, int64_t m, int blocks, float* __restrict__ grid_out,
+__global__ void __launch_bounds__(256) grid_finalize_kernel(GridWs w, int p, int n, int64_t m, int fit_blocks, int plain_blocks, float* __restrict__ grid_out,
                                                             float* __restrict__ mse_out, int32_t* __restrict__ iters_out) {
     // lexicographic sort by rank counting, one warp per centre (coordinate 0 first; equal points keep their index order)
     const int lane = threadIdx.x & 31, c = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
@@ -492,6 +630,7 @@ __global__ void __launch_bounds__(256) grid_finalize_kernel(GridWs w, int p, int
         if (lane < p) grid_out[rank * p + lane] = w.centres[c * p + lane];
     }
     if (c == 0) {
+        const int blocks = w.flags[2] ? plain_blocks : fit_blocks;
         double e = 0.0;
         for (int i = lane; i < blocks; i += 32) e += w.err[i];
 #pragma unroll
@@ -581,13 +720,26 @@ static int sm_count_of_device() {
 
 // One cooperative launch for the whole iteration, a block per SM (fewer when there are fewer than 32 samples for each); where
 // the device does not allow it, one ordinary block, whose barriers are trivial.
+template <typename... Args>
+static int launch_resident(void (*kernel)(Args...), int* blocks, size_t smem, cudaStream_t st, Args... args) {
+    if (*blocks > 1) {
+        void* ptrs[] = {&args...};
+        if (cudaLaunchCooperativeKernel((const void*)kernel, dim3((unsigned)*blocks), dim3(kFitThreads), ptrs, smem, st) == cudaSuccess) return HIGGS_OK;
+        (void)cudaGetLastError();
+        *blocks = 1;
+    }
+    kernel<<<1, kFitThreads, smem, st>>>(args...);
+    return cuda_status(cudaGetLastError());
+}
+
 template <int P>
-static int launch_fit(GridWs w, const float* samples, int n, int64_t m, int max_iters, int* blocks_out, cudaStream_t st) {
+static int launch_fit(GridWs w, const float* samples, int n, int64_t m, int slots, int max_iters, int (&blocks_out)[2], cudaStream_t st) {
     constexpr size_t kMaxSmem = (P * (sizeof(long long) + sizeof(float)) + sizeof(int)) * kMaxGridPoints;     // (n = 4096: no lists)
     static int state[64] = {0};           // 1 = cooperative launch possible, 2 = not, -1 = failed
     const int how = device_once(state, [] {
         int dev = 0, coop = 0, v = 0;
-        if (cudaFuncSetAttribute(grid_fit_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxSmem > 73728 ? kMaxSmem : 73728)) != cudaSuccess)
+        if (cudaFuncSetAttribute(grid_fit_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxSmem > 73728 ? kMaxSmem : 73728)) != cudaSuccess ||
+            cudaFuncSetAttribute(plain_fit_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) != cudaSuccess)
             return -1;
         if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, grid_fit_kernel<P>, kFitThreads, kMaxSmem) != cudaSuccess || v < 1)
@@ -595,37 +747,31 @@ static int launch_fit(GridWs w, const float* samples, int n, int64_t m, int max_
         return 1;
     });
     if (how < 0) return HIGGS_ERR_CUDA;
-    const size_t smem = fit_smem(P, n);
-    if (how == 1) {
-        int64_t blocks = (m + 31) / 32;
-        if (blocks > sm_count_of_device()) blocks = sm_count_of_device();
-        if (blocks > kMaxFitBlocks) blocks = kMaxFitBlocks;
-        void* args[] = {&w, &samples, &n, &m, &max_iters};
-        if (cudaLaunchCooperativeKernel((const void*)grid_fit_kernel<P>, dim3((unsigned)blocks), dim3(kFitThreads), args, smem, st) == cudaSuccess) {
-            *blocks_out = (int)blocks;
-            return HIGGS_OK;
-        }
-        (void)cudaGetLastError();
-    }
-    grid_fit_kernel<P><<<1, kFitThreads, smem, st>>>(w, samples, n, m, max_iters);
-    *blocks_out = 1;
-    return cuda_status(cudaGetLastError());
+    int64_t blocks = how == 1 ? (m + 31) / 32 : 1;
+    if (blocks > sm_count_of_device()) blocks = sm_count_of_device();
+    if (blocks > kMaxFitBlocks) blocks = kMaxFitBlocks;
+    blocks_out[0] = blocks_out[1] = (int)blocks;
+    const int rc = launch_resident(grid_fit_kernel<P>, &blocks_out[0], fit_smem(P, n), st, w, samples, n, m, slots, max_iters);
+    if (rc != HIGGS_OK) return rc;
+    return launch_resident(plain_fit_kernel<P>, &blocks_out[1], (size_t)n * (P * (sizeof(double) + sizeof(float)) + sizeof(int)), st, w, samples, n, m, max_iters);
 }
 
 int launch_make_grid(int p, int n, const float* samples, int64_t m, int max_iters, float* grid_out, float* mse_out,
                      int32_t* iters_out, void* ws, cudaStream_t st) {
     GridWs w = carve(ws, p, n, m);
-    const int64_t init_threads = m > (int64_t)3 * n * p ? m : (int64_t)3 * n * p;
-    grid_init_kernel<<<(unsigned)((init_threads + 255) / 256), 256, 0, st>>>(w, p, n, m);
-    int blocks = 0, rc = HIGGS_ERR_UNSUPPORTED;
+    const int64_t most = (m + kRangeThreads - 1) / kRangeThreads;
+    const int slots = (int)(most < kMaxFitBlocks ? most : kMaxFitBlocks);
+    grid_init_kernel<<<(unsigned)slots, kRangeThreads, 0, st>>>(w, samples, p, n, m);
+    grid_range_kernel<<<(unsigned)slots, kRangeThreads, 0, st>>>(w, samples, p, m, slots);
+    int blocks[2] = {0, 0}, rc = HIGGS_ERR_UNSUPPORTED;
     switch (p) {
-        case 1: rc = launch_fit<1>(w, samples, n, m, max_iters, &blocks, st); break;
-        case 2: rc = launch_fit<2>(w, samples, n, m, max_iters, &blocks, st); break;
-        case 3: rc = launch_fit<3>(w, samples, n, m, max_iters, &blocks, st); break;
-        case 4: rc = launch_fit<4>(w, samples, n, m, max_iters, &blocks, st); break;
+        case 1: rc = launch_fit<1>(w, samples, n, m, slots, max_iters, blocks, st); break;
+        case 2: rc = launch_fit<2>(w, samples, n, m, slots, max_iters, blocks, st); break;
+        case 3: rc = launch_fit<3>(w, samples, n, m, slots, max_iters, blocks, st); break;
+        case 4: rc = launch_fit<4>(w, samples, n, m, slots, max_iters, blocks, st); break;
     }
     if (rc != HIGGS_OK) return rc;
-    grid_finalize_kernel<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(w, p, n, m, blocks, grid_out, mse_out, iters_out);
+    grid_finalize_kernel<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(w, p, n, m, blocks[0], blocks[1], grid_out, mse_out, iters_out);
     return cuda_status(cudaGetLastError());
 }
 

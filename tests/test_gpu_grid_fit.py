@@ -10,7 +10,7 @@ from tests import gpu_util as U
 pytestmark = pytest.mark.gpu
 
 
-def plain_lloyd(p, n, x, max_iters):
+def plain_lloyd(p, n, x, max_iters, cells=None):
     c = x[:n].copy()
     old = np.full(len(x), -1)
     for it in range(1, max_iters + 1):
@@ -21,13 +21,18 @@ def plain_lloyd(p, n, x, max_iters):
             d = (e[..., 0] ** 2).astype(np.float32)
             for k in range(1, p):
                 d = (e[..., k] ** 2 + d).astype(np.float32)                    # one rounding, as a fused multiply-add
+            d = np.where(np.isnan(d), np.float32(np.inf), d)                       # (never below infinity: index 0 when all are)
             a[i:i + 4096] = d.argmin(1)
             err += float(d.min(1).astype(np.float64).sum())
         if np.array_equal(a, old):
             return c, err, it
         old = a
         size = np.bincount(a, minlength=n)
+        if cells is not None:                                                      # sizes and sums of magnitudes behind the centres
+            cells[0][:] = size
         for k in range(p):
+            if cells is not None:
+                cells[1][:, k] = np.bincount(a, weights=np.abs(x[:, k].astype(np.float64)), minlength=n)
             s = np.bincount(a, weights=x[:, k].astype(np.float64), minlength=n)
             c[size > 0, k] = (s[size > 0] / size[size > 0]).astype(np.float32)
     return c, err, -max_iters
@@ -60,6 +65,38 @@ def test_samples_without_a_nearest_centre(p, n, m, bad):
     """A sample whose distances are all NaN or infinite belongs to cell 0, whichever way it is scanned."""
     x = np.random.default_rng(n).standard_normal((m, p)).astype(np.float32)
     x[n + 3, p - 1] = x[m - 1, 0] = bad
-    _, _, it = hb.higgs_make_grid(p, n, torch.from_numpy(x).to(U.dev()), max_iters=12)
+    grid, mse, it = hb.higgs_make_grid(p, n, torch.from_numpy(x).to(U.dev()), max_iters=12)
     assert hb.higgs_device_status() == hb.HIGGS_OK
     assert 1 <= abs(int(it)) <= 12
+    with np.errstate(all="ignore"):
+        c, err, iters = plain_lloyd(p, n, x, 12)
+    assert int(it) == iters
+    assert np.isinf(float(mse)) if np.isinf(err) else abs(float(mse) - err / (m * p)) <= 1e-6 * err / (m * p)
+    if not np.isnan(bad):                                   # (a NaN has no place in the order of the centres)
+        want = c[np.lexsort(c.T[::-1])]
+        assert np.allclose(grid.cpu().numpy(), want, rtol=2.0 ** -22, atol=2.0 ** -22)
+
+
+@pytest.mark.parametrize("p,n,m,case", [(1, 16, 4000, "outlier"), (2, 256, 70000, "outlier"), (2, 256, 33, "few"), (2, 600, 5000, "spread"),
+                                        (4, 100, 9000, "spread"), (1, 64, 3000, "tiny"), (3, 300, 4000, "huge")])
+def test_samples_of_another_range(p, n, m, case):
+    """Sets that 64-bit fixed-point sums would round: their means are those of fp64 sums."""
+    if case == "few":
+        n = 16
+    rng = np.random.default_rng(n)
+    x = rng.standard_normal((m, p))
+    if case == "spread":
+        x *= 10.0 ** rng.uniform(-12, 12, (m, 1))
+    x = (x * {"tiny": 1e-25, "huge": 1e18}.get(case, 1.0)).astype(np.float32)
+    if case in ("outlier", "few"):
+        x[m - 2, 0], x[n + 2, p - 1] = 3e15, -1e15
+    size, mag = np.zeros(n), np.zeros((n, p))
+    c, err, iters = plain_lloyd(p, n, x, 40, cells=(size, mag))
+    grid, mse, it = hb.higgs_make_grid(p, n, torch.from_numpy(x).to(U.dev()), max_iters=40)
+    assert hb.higgs_device_status() == hb.HIGGS_OK
+    assert int(it) == iters
+    # per cell: fp64 sums of its samples in another order, the sum of magnitudes over the size, then one rounding to fp32
+    bound = size[:, None] * 2.0 ** -53 * mag / np.maximum(size, 1)[:, None] + 2.0 ** -23 * np.abs(c)
+    order = np.lexsort(c.T[::-1])
+    assert np.all(np.abs(grid.cpu().numpy().astype(np.float64) - c[order]) <= bound[order])
+    assert abs(float(mse) - err / (m * p)) <= 1e-6 * err / (m * p) + 1e-30
