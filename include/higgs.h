@@ -150,6 +150,8 @@ int higgs_make_uniform_grid(int n, float* grid_out, float* step_out, float* mse_
  *                the samples
  *   iters_out    device, optional: iterations run (int32), negative if
  *                max_iters was reached without convergence
+ * If a wait of the fit runs out (higgs_device_status), mse_out is NaN, iters_out
+ * negative and the grid made of the first n samples.
  * Distances are fp32, sums 64-bit fixed point in steps of 2^-62 times
  * num_samples times the largest |coordinate|, both rounded up to powers of two
  * (exact for N(0, 1) samples but the tiniest), independent of the order of
@@ -446,6 +448,10 @@ int higgs_device_status(void* stream, int clear);
  */
 int higgs_launch_floor(int32_t blocks, int32_t threads, size_t shared_bytes, void* stream);
 int higgs_selftest_wait(int32_t which, uint32_t polls, int32_t* result_out, void* stream);
+/* higgs_make_grid (p <= 2, up to 2^20 samples) whose barrier waits for one arrival more than there are blocks, about 2^10 polls long: every
+ * block gives up and returns, higgs_device_status() reports HIGGS_ERR_TIMEOUT and the outputs are those of a wait that ran out. */
+int higgs_selftest_grid_fit(int p, int n, const float* samples, int64_t num_samples, float* grid_out, float* mse_out,
+                            int32_t* iters_out, void* workspace, size_t workspace_bytes, void* stream);
 
 /* Number of K ranges the product kernel assigns to different thread blocks for this shape and
  * batch (1 = not split), and whether those ranges meet in fp32 atomics.  For batches up to 16 two ranges are taken

@@ -30,7 +30,7 @@ EXPORTS = [
     "higgs_rotated_layout", "higgs_dequantize", "higgs_make_uniform_grid", "higgs_layer_error",
     "higgs_allocate_bits", "higgs_general_tuples", "higgs_quantize_general", "higgs_linear_host_batch",
     "higgs_linear_gather", "higgs_linear_share", "higgs_make_grid_seeded", "higgs_gaussian_samples", "higgs_shard_rows",
-    "higgs_launch_floor", "higgs_selftest_wait", "higgs_linear_uses_atomics", "higgs_shard_seed", "higgs_linear_kshard", "higgs_reduce_slots", "higgs_linear_multi", "higgs_linear_multi_workspace_bytes",
+    "higgs_launch_floor", "higgs_selftest_wait", "higgs_selftest_grid_fit", "higgs_linear_uses_atomics", "higgs_shard_seed", "higgs_linear_kshard", "higgs_reduce_slots", "higgs_linear_multi", "higgs_linear_multi_workspace_bytes",
     "higgs_linear_multi_launch_count", "higgs_linear_host_block", "higgs_linear_host_block_workspace_bytes",
 ]
 
@@ -149,6 +149,8 @@ def _load() -> ctypes.CDLL:
     lib.higgs_reduce_slots.argtypes = [vp, i32, i64, vp, i32, vp]
     lib.higgs_launch_floor.restype = i32
     lib.higgs_launch_floor.argtypes = [i32, i32, sz, vp]
+    lib.higgs_selftest_grid_fit.restype = i32
+    lib.higgs_selftest_grid_fit.argtypes = [i32, i32, vp, i64, vp, vp, vp, vp, sz, vp]
     lib.higgs_selftest_wait.restype = i32
     lib.higgs_selftest_wait.argtypes = [i32, ctypes.c_uint32, vp, vp]
     return lib
@@ -268,6 +270,18 @@ def higgs_selftest_wait(which: int, polls: int, device=None) -> torch.Tensor:
     out = torch.full((2,), -1, dtype=torch.int32, device=device)
     _check(lib.higgs_selftest_wait(which, polls, _ptr(out), _stream()), "higgs_selftest_wait")
     return out
+
+
+def higgs_selftest_grid_fit(p: int, n: int, samples: torch.Tensor):
+    """A grid fit whose barrier runs out; returns (grid, mse, iters) like higgs_make_grid."""
+    assert samples.is_cuda and samples.dtype == torch.float32 and samples.is_contiguous()
+    m = samples.numel() // p
+    d = higgs_desc(p, n, 0, HIGGS_F16, 0, 0, m, HIGGS_LAYOUT_VERSION, 0)
+    workspace = _workspace(higgs_workspace_bytes(d, HIGGS_OP_MAKE_GRID), samples.device)
+    grid, mse, iters = samples.new_empty((n, p)), samples.new_empty(()), samples.new_empty((), dtype=torch.int32)
+    _check(lib.higgs_selftest_grid_fit(p, n, _ptr(samples), m, _ptr(grid), _ptr(mse), _ptr(iters), _ptr(workspace), workspace.numel(), _stream()),
+           "higgs_selftest_grid_fit")
+    return grid, mse, iters
 
 
 def higgs_make_encoder_table(p: int, n: int, grid: torch.Tensor) -> torch.Tensor:

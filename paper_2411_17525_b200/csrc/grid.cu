@@ -23,7 +23,7 @@ struct GridWs {
     int32_t* delta_cnt;           // [3][n]    changes of the cells' sizes
     double* err;                  // [kMaxFitBlocks] squared error of a block's samples; before the fit the range of the samples, as uint2
     unsigned long long* bar;      // [2] grid barrier: arrivals (low half), blocks with a changed assignment (high half)
-    int32_t* flags;               // [0] done, [1] iterations, [2] the samples are left to plain_fit_kernel
+    int32_t* flags;               // [0] done, [1] iterations, [2] the samples are left to plain_fit_kernel, [3] a barrier ran out
     uint16_t* near_idx;           // [kMaxNearCentres][kNear] neighbour lists
     float* excl;                  // [kMaxNearCentres]
     int32_t* assign;              // [m]
@@ -55,6 +55,7 @@ __global__ void __launch_bounds__(kRangeThreads) grid_init_kernel(GridWs w, cons
     const int64_t first = (int64_t)blockIdx.x * kRangeThreads + threadIdx.x, step = (int64_t)gridDim.x * kRangeThreads;
     for (int64_t i = first; i < (int64_t)3 * n * p; i += step) w.delta[i] = 0;
     for (int64_t i = first; i < 3 * n; i += step) w.delta_cnt[i] = 0;
+    for (int64_t i = first; i < n * p; i += step) w.centres[i] = samples[i];       // (the result if a barrier runs out)
     if (first < 2) w.bar[first] = 0;
     if (first < 8) w.flags[first] = 0;
     unsigned top = 0u;
@@ -126,31 +127,36 @@ __device__ __forceinline__ bool range_unsuited(uint2 range, int64_t m) {
 
 // Every block is resident (a cooperative launch, or one block), so the blocks can meet at a barrier: a counter in the
 // workspace that every block's first thread adds to and then polls, with a limit on the polls - a barrier that runs out
-// raises the grid-fit status word and every block leaves.  The same addition counts the blocks that report `changed`.
+// raises the grid-fit status word and the fit's own flag, and every block leaves.  The same addition counts the blocks that report `changed`.
 // Two counters take turns (barrier number `no` uses no % 2), so a block that reads late cannot see the next barrier's.
 __device__ int g_grid_status = 0;
 constexpr unsigned kGridBarrierLimit = 1u << 22;
 
-// returns whether any block reported a change in this barrier; *ok = false if it ran out
-__device__ __forceinline__ bool grid_barrier(unsigned long long* bar, int no, int blocks, bool changed, unsigned& seen, bool* ok) {
+// returns whether any block reported a change in this barrier; *ok = false if it ran out.  RUN_OUT (a test): one arrival more is
+// waited for than there are blocks, for a short time.
+template <bool RUN_OUT>
+__device__ __forceinline__ bool grid_barrier(const GridWs& w, int no, bool changed, unsigned& seen, bool* ok) {
     __shared__ unsigned s_high;
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        unsigned long long* counter = bar + (no & 1);
-        const unsigned target = (unsigned)(no / 2 + 1) * (unsigned)blocks;
+        unsigned long long* counter = w.bar + (no & 1);
+        const unsigned target = (unsigned)(no / 2 + 1) * (gridDim.x + (RUN_OUT ? 1u : 0u));
         __threadfence();
         atomicAdd(counter, 1ull | (changed ? 1ull << 32 : 0ull));
         unsigned it = 0;
         unsigned long long v;
         for (;;) {
             asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(counter) : "memory");
-            if ((unsigned)v >= target || ++it > kGridBarrierLimit) break;
+            if ((unsigned)v >= target || ++it > (RUN_OUT ? 1u << 10 : kGridBarrierLimit)) break;
         }
         __threadfence();
         s_high = (unsigned)(v >> 32);
         s_ok = (unsigned)v >= target;
-        if ((unsigned)v < target) atomicExch(&g_grid_status, (int)HIGGS_ERR_TIMEOUT);
+        if ((unsigned)v < target) {
+            atomicExch(&g_grid_status, (int)HIGGS_ERR_TIMEOUT);
+            w.flags[3] = 1;
+        }
     }
     __syncthreads();
     *ok = s_ok != 0;
@@ -204,7 +210,7 @@ __device__ __forceinline__ void write_result(const GridWs& w, const float* sc, i
 // The iteration as it stands, without bounds and with fp64 sums over all samples, for the sample sets that grid_fit_kernel leaves
 // untouched (it is launched after that kernel every time; a kernel of its own because a call in there takes registers from the
 // other path: 2 % of its time).  The sums of an iteration are in w.delta (as doubles), three buffers in turn as there.
-template <int P>
+template <int P, bool RUN_OUT>
 __global__ void __launch_bounds__(kFitThreads, 1) plain_fit_kernel(GridWs w, const float* __restrict__ samples, int n, int64_t m, int max_iters) {
     if (!w.flags[2]) return;
     extern __shared__ __align__(16) unsigned char grid_smem[];
@@ -243,7 +249,7 @@ __global__ void __launch_bounds__(kFitThreads, 1) plain_fit_kernel(GridWs w, con
             if (block_cnt[i / P]) atomicAdd(&sums[i], block_sums[i]);
         for (int i = tid; i < n; i += kFitThreads)
             if (block_cnt[i]) atomicAdd(&cnt[i], block_cnt[i]);
-        const bool any = grid_barrier(w.bar, it, blocks, block_changed, seen[it & 1], &ok);
+        const bool any = grid_barrier<RUN_OUT>(w, it, block_changed, seen[it & 1], &ok);
         if (!ok) return;
         if (!any) { done = true; ++it; break; }
         for (int i = tid; i < n * P; i += kFitThreads) {
@@ -289,7 +295,7 @@ inline size_t fit_smem(int p, int n) {
 // Bound: latency - per iteration about 2.5 us of barrier, 2 us of update, 2.5 us to test the samples and 1 to 2 us of scans.
 // p = 2, n = 256, 2^18 samples: 37 -> 9 us per iteration (before: every sample scanned all centres every time, sums by
 // fp64 atomics in shared memory, two barriers).  One barrier and movement bounds without lists: 12.4 us.
-template <int P>
+template <int P, bool RUN_OUT>
 __global__ void __launch_bounds__(kFitThreads, 1) grid_fit_kernel(GridWs w, const float* __restrict__ samples, int n, int64_t m, int slots, int max_iters) {
     extern __shared__ __align__(16) unsigned char grid_smem[];
     const bool shared_sums = n * P <= kMaxSharedSums, lists = fit_lists(n);
@@ -376,7 +382,7 @@ __global__ void __launch_bounds__(kFitThreads, 1) grid_fit_kernel(GridWs w, cons
                 if (lane == 0) w.excl[a] = __fsqrt_rd(__fmul_rd(__uint_as_float(out), 0.999996f));
             }
             if (tid == 0) s_min_excl = 0x7f800000u;
-            grid_barrier(w.bar, barrier_no, blocks, false, seen[barrier_no & 1], &ok);
+            grid_barrier<RUN_OUT>(w, barrier_no, false, seen[barrier_no & 1], &ok);
             ++barrier_no;
             if (!ok) return;
             for (int i = tid; i < n * kNear / 8; i += kFitThreads)
@@ -552,7 +558,7 @@ __global__ void __launch_bounds__(kFitThreads, 1) grid_fit_kernel(GridWs w, cons
             for (int q = tid; q < n; q += kFitThreads)
                 if (d_cnt[q]) { atomicAdd(&delta_cnt[q], d_cnt[q]); d_cnt[q] = 0; }
         }
-        const bool any = grid_barrier(w.bar, barrier_no, blocks, block_changed, seen[barrier_no & 1], &ok);
+        const bool any = grid_barrier<RUN_OUT>(w, barrier_no, block_changed, seen[barrier_no & 1], &ok);
         ++barrier_no;
         if (!ok) return;
         if (!any) { done = true; ++it; break; }          // no assignment changed: a fixed point
@@ -636,8 +642,9 @@ __global__ void __launch_bounds__(256) grid_finalize_kernel(GridWs w, int p, int
 #pragma unroll
         for (int k = 16; k > 0; k >>= 1) e += __shfl_xor_sync(0xffffffffu, e, k);
         if (lane == 0) {
-            if (mse_out) *mse_out = (float)(e / ((double)m * p));
-            if (iters_out) *iters_out = w.flags[0] ? w.flags[1] : -w.flags[1];
+            const bool ran_out = w.flags[3] != 0;
+            if (mse_out) *mse_out = ran_out ? NAN : (float)(e / ((double)m * p));
+            if (iters_out) *iters_out = ran_out ? -1 : w.flags[0] ? w.flags[1] : -w.flags[1];
         }
     }
 }
@@ -732,17 +739,17 @@ static int launch_resident(void (*kernel)(Args...), int* blocks, size_t smem, cu
     return cuda_status(cudaGetLastError());
 }
 
-template <int P>
+template <int P, bool RUN_OUT>
 static int launch_fit(GridWs w, const float* samples, int n, int64_t m, int slots, int max_iters, int (&blocks_out)[2], cudaStream_t st) {
     constexpr size_t kMaxSmem = (P * (sizeof(long long) + sizeof(float)) + sizeof(int)) * kMaxGridPoints;     // (n = 4096: no lists)
     static int state[64] = {0};           // 1 = cooperative launch possible, 2 = not, -1 = failed
     const int how = device_once(state, [] {
         int dev = 0, coop = 0, v = 0;
-        if (cudaFuncSetAttribute(grid_fit_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxSmem > 73728 ? kMaxSmem : 73728)) != cudaSuccess ||
-            cudaFuncSetAttribute(plain_fit_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) != cudaSuccess)
+        if (cudaFuncSetAttribute(grid_fit_kernel<P, RUN_OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxSmem > 73728 ? kMaxSmem : 73728)) != cudaSuccess ||
+            cudaFuncSetAttribute(plain_fit_kernel<P, RUN_OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) != cudaSuccess)
             return -1;
         if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, grid_fit_kernel<P>, kFitThreads, kMaxSmem) != cudaSuccess || v < 1)
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, grid_fit_kernel<P, RUN_OUT>, kFitThreads, kMaxSmem) != cudaSuccess || v < 1)
             return 2;
         return 1;
     });
@@ -751,24 +758,26 @@ static int launch_fit(GridWs w, const float* samples, int n, int64_t m, int slot
     if (blocks > sm_count_of_device()) blocks = sm_count_of_device();
     if (blocks > kMaxFitBlocks) blocks = kMaxFitBlocks;
     blocks_out[0] = blocks_out[1] = (int)blocks;
-    const int rc = launch_resident(grid_fit_kernel<P>, &blocks_out[0], fit_smem(P, n), st, w, samples, n, m, slots, max_iters);
+    const int rc = launch_resident(grid_fit_kernel<P, RUN_OUT>, &blocks_out[0], fit_smem(P, n), st, w, samples, n, m, slots, max_iters);
     if (rc != HIGGS_OK) return rc;
-    return launch_resident(plain_fit_kernel<P>, &blocks_out[1], (size_t)n * (P * (sizeof(double) + sizeof(float)) + sizeof(int)), st, w, samples, n, m, max_iters);
+    return launch_resident(plain_fit_kernel<P, RUN_OUT>, &blocks_out[1], (size_t)n * (P * (sizeof(double) + sizeof(float)) + sizeof(int)), st, w, samples, n, m, max_iters);
 }
 
 int launch_make_grid(int p, int n, const float* samples, int64_t m, int max_iters, float* grid_out, float* mse_out,
-                     int32_t* iters_out, void* ws, cudaStream_t st) {
+                     int32_t* iters_out, void* ws, cudaStream_t st, bool run_out) {
     GridWs w = carve(ws, p, n, m);
     const int64_t most = (m + kRangeThreads - 1) / kRangeThreads;
     const int slots = (int)(most < kMaxFitBlocks ? most : kMaxFitBlocks);
     grid_init_kernel<<<(unsigned)slots, kRangeThreads, 0, st>>>(w, samples, p, n, m);
     grid_range_kernel<<<(unsigned)slots, kRangeThreads, 0, st>>>(w, samples, p, m, slots);
     int blocks[2] = {0, 0}, rc = HIGGS_ERR_UNSUPPORTED;
-    switch (p) {
-        case 1: rc = launch_fit<1>(w, samples, n, m, slots, max_iters, blocks, st); break;
-        case 2: rc = launch_fit<2>(w, samples, n, m, slots, max_iters, blocks, st); break;
-        case 3: rc = launch_fit<3>(w, samples, n, m, slots, max_iters, blocks, st); break;
-        case 4: rc = launch_fit<4>(w, samples, n, m, slots, max_iters, blocks, st); break;
+    switch (2 * p + (run_out ? 1 : 0)) {
+        case 2: rc = launch_fit<1, false>(w, samples, n, m, slots, max_iters, blocks, st); break;
+        case 3: rc = launch_fit<1, true>(w, samples, n, m, slots, max_iters, blocks, st); break;
+        case 4: rc = launch_fit<2, false>(w, samples, n, m, slots, max_iters, blocks, st); break;
+        case 5: rc = launch_fit<2, true>(w, samples, n, m, slots, max_iters, blocks, st); break;
+        case 6: rc = launch_fit<3, false>(w, samples, n, m, slots, max_iters, blocks, st); break;
+        case 8: rc = launch_fit<4, false>(w, samples, n, m, slots, max_iters, blocks, st); break;
     }
     if (rc != HIGGS_OK) return rc;
     grid_finalize_kernel<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(w, p, n, m, blocks[0], blocks[1], grid_out, mse_out, iters_out);

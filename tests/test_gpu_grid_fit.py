@@ -100,3 +100,19 @@ def test_samples_of_another_range(p, n, m, case):
     order = np.lexsort(c.T[::-1])
     assert np.all(np.abs(grid.cpu().numpy().astype(np.float64) - c[order]) <= bound[order])
     assert abs(float(mse) - err / (m * p)) <= 1e-6 * err / (m * p) + 1e-30
+
+
+@pytest.mark.parametrize("p,n,m", [(1, 4, 31), (2, 256, 30000), (2, 600, 5000)])
+@pytest.mark.parametrize("value", [0.5, float("inf")])
+def test_a_barrier_that_runs_out(p, n, m, value):
+    """Blocks that wait for one arrival too many give up: a reported timeout and defined outputs, and the next fit is none the worse."""
+    x = np.random.default_rng(m).standard_normal((m, p)).astype(np.float32)
+    x[m - 1, 0] = value                                     # (infinite: the kernel for sample sets of any range)
+    t = torch.from_numpy(x).to(U.dev())
+    grid, mse, it = hb.higgs_selftest_grid_fit(p, n, t)
+    assert hb.higgs_device_status() == hb.HIGGS_ERR_TIMEOUT
+    assert int(it) < 0 and np.isnan(float(mse))
+    assert np.array_equal(grid.cpu().numpy(), x[:n][np.lexsort(x[:n].T[::-1])])
+    _, mse, it = hb.higgs_make_grid(p, n, t, max_iters=20)
+    assert hb.higgs_device_status() == hb.HIGGS_OK
+    assert int(it) != 0 and not np.isnan(float(mse))
