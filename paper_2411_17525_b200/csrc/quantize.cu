@@ -222,7 +222,8 @@ __global__ void __launch_bounds__(128) encode_kernel(const T* __restrict__ W, co
 // The same nearest-point rule as above, evaluated only on the grid points that can win.  The plane (the line for
 // p = 1) is cut into square cells; cell i of an axis covers the values whose scaled coordinate x * cells / 2R + cells / 2
 // rounds to i.  The encoder finds it with two fused multiply-adds: onto [0, 1] with saturation, then onto 2^23, where the
-// integer is the low bits of the float; values beyond the table (and NaN) fall into the outermost cells, which are marked.  A cell's
+// integer is the low bits of the float; values beyond the table (and NaN) fall into the outermost cells, which the encoder marks
+// in its own copy (a table may be older than that rule).  A cell's
 // candidate list is built in two steps.  (1) U = min over grid points of the distance to the cell's farthest corner
 // bounds the winner's distance from any point of the cell, so only points whose distance to the cell is at most U (+ a
 // slack far above fp32 rounding) can be nearest.  (2) Of those, c is dropped if another candidate c' is nearer at all
@@ -286,8 +287,7 @@ __global__ void __launch_bounds__(256) build_cells_kernel(const float* __restric
         }
         __syncwarp();
         uint32_t word = kCellScan;
-        const bool border = cx == 0 || cx == CELLS - 1 || (P == 2 && (cy == 0 || cy == CELLS - 1));
-        if (k <= kPrefilter && !border) {
+        if (k <= kPrefilter) {
             // step (2): lane i judges candidate i against every candidate j
             const bool have = lane < k;
             const int mine = have ? slist[wi][lane] : 0;
@@ -451,8 +451,14 @@ __global__ void __launch_bounds__(kEncThreads, 1) encode_pruned_kernel(const T* 
     uint8_t* tiles_base = rep + (size_t)n * 128 + 32 * kEncExchange + half * (kEncTiles * 16 * RS);
     const uint32_t bar = enc_smem_u32(rep + (size_t)n * 128 + 32 * kEncExchange + 2 * kEncTiles * 16 * RS) + 8u * half;   // one arrival per warp and turn
     if (wib == 0 && lane == 0) enc_mbar_init(bar, 16);
-    for (int i = threadIdx.x; i < NC / 4; i += blockDim.x)
-        reinterpret_cast<uint4*>(cells)[i] = reinterpret_cast<const uint4*>(table)[i];
+    for (int i = threadIdx.x; i < NC / 4; i += blockDim.x) {
+        uint4 c = reinterpret_cast<const uint4*>(table)[i];
+        const int cy = P == 2 ? i / (CELLS / 4) : 1, cx = i % (CELLS / 4);
+        if (P == 2 && (cy == 0 || cy == CELLS - 1)) c = make_uint4(kCellScan, kCellScan, kCellScan, kCellScan);
+        if (cx == 0) c.x = kCellScan;
+        if (cx == CELLS / 4 - 1) c.w = kCellScan;
+        reinterpret_cast<uint4*>(cells)[i] = c;
+    }
     for (int i = threadIdx.x; i < n * 32; i += blockDim.x)
         reinterpret_cast<float*>(rep)[i] = -grid[P == 2 ? 2 * (i >> 5) + (i & 1) : (i >> 5)];
     __syncthreads();

@@ -27,3 +27,21 @@ def test_turns_equal_the_exhaustive_scan(p, n, N, K, dtype):
         ds = hb.make_desc(p, n, rows, K, 13)
         _, sc, ca = hb.higgs_quantize(ds, W[r:r + rows].contiguous(), gt, want_canonical=True)
         assert torch.equal(canon[r:r + rows], ca) and torch.equal(scales[r // 16:(r + rows) // 16], sc)
+
+
+@pytest.mark.parametrize("p,n", [(2, 256), (2, 16), (1, 16)])
+def test_outermost_cells_of_the_search_table_are_never_used(p, n):
+    """Points beyond the table fall into its outermost cells, so these are always scanned, whatever a table (an older one, say) lists there."""
+    _, grid = U.grid32(p, n)
+    W = torch.randn(2048, 4096, device=U.dev(), generator=torch.Generator(device="cuda").manual_seed(p))
+    d = hb.make_desc(p, n, 2048, 4096, 3)
+    table = hb.higgs_make_encoder_table(p, n, grid)
+    cells = table.view(torch.int32).view(128, 128) if p == 2 else table.view(torch.int32).view(1, 1024)
+    if p == 2:
+        cells[[0, -1]] = 0
+    cells[:, [0, -1]] = 0
+    packed, scales, codes = hb.higgs_quantize(d, W, grid, want_canonical=True, table=table)
+    few = hb.make_desc(p, n, 16, 4096, 3)                   # (small layers are scanned exhaustively)
+    ref = torch.cat([hb.higgs_quantize(few, W[r:r + 16].contiguous(), grid, want_canonical=True)[2] for r in range(0, 2048, 16)])
+    assert hb.higgs_device_status() == hb.HIGGS_OK
+    assert torch.equal(codes, ref)
