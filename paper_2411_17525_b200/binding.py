@@ -150,7 +150,7 @@ def _load() -> ctypes.CDLL:
     lib.higgs_launch_floor.restype = i32
     lib.higgs_launch_floor.argtypes = [i32, i32, sz, vp]
     lib.higgs_selftest_grid_fit.restype = i32
-    lib.higgs_selftest_grid_fit.argtypes = [i32, i32, vp, i64, vp, vp, vp, vp, sz, vp]
+    lib.higgs_selftest_grid_fit.argtypes = [i32, i32, i32, vp, i64, vp, vp, vp, vp, sz, vp]
     lib.higgs_selftest_wait.restype = i32
     lib.higgs_selftest_wait.argtypes = [i32, ctypes.c_uint32, vp, vp]
     return lib
@@ -272,14 +272,14 @@ def higgs_selftest_wait(which: int, polls: int, device=None) -> torch.Tensor:
     return out
 
 
-def higgs_selftest_grid_fit(p: int, n: int, samples: torch.Tensor):
-    """A grid fit whose barrier runs out; returns (grid, mse, iters) like higgs_make_grid."""
+def higgs_selftest_grid_fit(which: int, p: int, n: int, samples: torch.Tensor):
+    """A grid fit whose barrier runs out (which = 0) or whose first launch is refused (1); returns (grid, mse, iters) like higgs_make_grid."""
     assert samples.is_cuda and samples.dtype == torch.float32 and samples.is_contiguous()
     m = samples.numel() // p
     d = higgs_desc(p, n, 0, HIGGS_F16, 0, 0, m, HIGGS_LAYOUT_VERSION, 0)
     workspace = _workspace(higgs_workspace_bytes(d, HIGGS_OP_MAKE_GRID), samples.device)
     grid, mse, iters = samples.new_empty((n, p)), samples.new_empty(()), samples.new_empty((), dtype=torch.int32)
-    _check(lib.higgs_selftest_grid_fit(p, n, _ptr(samples), m, _ptr(grid), _ptr(mse), _ptr(iters), _ptr(workspace), workspace.numel(), _stream()),
+    _check(lib.higgs_selftest_grid_fit(which, p, n, _ptr(samples), m, _ptr(grid), _ptr(mse), _ptr(iters), _ptr(workspace), workspace.numel(), _stream()),
            "higgs_selftest_grid_fit")
     return grid, mse, iters
 

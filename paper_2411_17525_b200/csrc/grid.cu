@@ -725,22 +725,22 @@ static int sm_count_of_device() {
     return v;
 }
 
-// One cooperative launch for the whole iteration, a block per SM (fewer when there are fewer than 32 samples for each); where
-// the device does not allow it, one ordinary block, whose barriers are trivial.
+// One cooperative launch for the whole iteration, a block per SM (fewer when there are fewer than 32 samples for each).  Where fewer
+// are resident (a context that owns a part of the SMs), half as many are tried until they are; the last resort is one ordinary
+// block, whose barriers are trivial.
 template <typename... Args>
 static int launch_resident(void (*kernel)(Args...), int* blocks, size_t smem, cudaStream_t st, Args... args) {
-    if (*blocks > 1) {
-        void* ptrs[] = {&args...};
+    void* ptrs[] = {&args...};
+    for (; *blocks > 1; *blocks /= 2) {
         if (cudaLaunchCooperativeKernel((const void*)kernel, dim3((unsigned)*blocks), dim3(kFitThreads), ptrs, smem, st) == cudaSuccess) return HIGGS_OK;
         (void)cudaGetLastError();
-        *blocks = 1;
     }
     kernel<<<1, kFitThreads, smem, st>>>(args...);
     return cuda_status(cudaGetLastError());
 }
 
 template <int P, bool RUN_OUT>
-static int launch_fit(GridWs w, const float* samples, int n, int64_t m, int slots, int max_iters, int (&blocks_out)[2], cudaStream_t st) {
+static int launch_fit(GridWs w, const float* samples, int n, int64_t m, int slots, int max_iters, int crowd, int (&blocks_out)[2], cudaStream_t st) {
     constexpr size_t kMaxSmem = (P * (sizeof(long long) + sizeof(float)) + sizeof(int)) * kMaxGridPoints;     // (n = 4096: no lists)
     static int state[64] = {0};           // 1 = cooperative launch possible, 2 = not, -1 = failed
     const int how = device_once(state, [] {
@@ -757,27 +757,28 @@ static int launch_fit(GridWs w, const float* samples, int n, int64_t m, int slot
     int64_t blocks = how == 1 ? (m + 31) / 32 : 1;
     if (blocks > sm_count_of_device()) blocks = sm_count_of_device();
     if (blocks > kMaxFitBlocks) blocks = kMaxFitBlocks;
-    blocks_out[0] = blocks_out[1] = (int)blocks;
+    blocks_out[0] = blocks_out[1] = (int)blocks * crowd;
     const int rc = launch_resident(grid_fit_kernel<P, RUN_OUT>, &blocks_out[0], fit_smem(P, n), st, w, samples, n, m, slots, max_iters);
     if (rc != HIGGS_OK) return rc;
     return launch_resident(plain_fit_kernel<P, RUN_OUT>, &blocks_out[1], (size_t)n * (P * (sizeof(double) + sizeof(float)) + sizeof(int)), st, w, samples, n, m, max_iters);
 }
 
 int launch_make_grid(int p, int n, const float* samples, int64_t m, int max_iters, float* grid_out, float* mse_out,
-                     int32_t* iters_out, void* ws, cudaStream_t st, bool run_out) {
+                     int32_t* iters_out, void* ws, cudaStream_t st, FitTest test) {
     GridWs w = carve(ws, p, n, m);
     const int64_t most = (m + kRangeThreads - 1) / kRangeThreads;
     const int slots = (int)(most < kMaxFitBlocks ? most : kMaxFitBlocks);
     grid_init_kernel<<<(unsigned)slots, kRangeThreads, 0, st>>>(w, samples, p, n, m);
     grid_range_kernel<<<(unsigned)slots, kRangeThreads, 0, st>>>(w, samples, p, m, slots);
     int blocks[2] = {0, 0}, rc = HIGGS_ERR_UNSUPPORTED;
-    switch (2 * p + (run_out ? 1 : 0)) {
-        case 2: rc = launch_fit<1, false>(w, samples, n, m, slots, max_iters, blocks, st); break;
-        case 3: rc = launch_fit<1, true>(w, samples, n, m, slots, max_iters, blocks, st); break;
-        case 4: rc = launch_fit<2, false>(w, samples, n, m, slots, max_iters, blocks, st); break;
-        case 5: rc = launch_fit<2, true>(w, samples, n, m, slots, max_iters, blocks, st); break;
-        case 6: rc = launch_fit<3, false>(w, samples, n, m, slots, max_iters, blocks, st); break;
-        case 8: rc = launch_fit<4, false>(w, samples, n, m, slots, max_iters, blocks, st); break;
+    const int crowd = test == FitTest::kTooManyBlocks ? 4 : 1;
+    switch (2 * p + (test == FitTest::kRunOut ? 1 : 0)) {
+        case 2: rc = launch_fit<1, false>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
+        case 3: rc = launch_fit<1, true>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
+        case 4: rc = launch_fit<2, false>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
+        case 5: rc = launch_fit<2, true>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
+        case 6: rc = launch_fit<3, false>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
+        case 8: rc = launch_fit<4, false>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
     }
     if (rc != HIGGS_OK) return rc;
     grid_finalize_kernel<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(w, p, n, m, blocks[0], blocks[1], grid_out, mse_out, iters_out);

@@ -109,10 +109,26 @@ def test_a_barrier_that_runs_out(p, n, m, value):
     x = np.random.default_rng(m).standard_normal((m, p)).astype(np.float32)
     x[m - 1, 0] = value                                     # (infinite: the kernel for sample sets of any range)
     t = torch.from_numpy(x).to(U.dev())
-    grid, mse, it = hb.higgs_selftest_grid_fit(p, n, t)
+    grid, mse, it = hb.higgs_selftest_grid_fit(0, p, n, t)
     assert hb.higgs_device_status() == hb.HIGGS_ERR_TIMEOUT
     assert int(it) < 0 and np.isnan(float(mse))
     assert np.array_equal(grid.cpu().numpy(), x[:n][np.lexsort(x[:n].T[::-1])])
     _, mse, it = hb.higgs_make_grid(p, n, t, max_iters=20)
     assert hb.higgs_device_status() == hb.HIGGS_OK
     assert int(it) != 0 and not np.isnan(float(mse))
+
+
+@pytest.mark.parametrize("p,n,m", [(1, 16, 8192), (2, 256, 70000)])
+@pytest.mark.parametrize("value", [0.5, 1e15])
+def test_fewer_resident_blocks_than_asked_for(p, n, m, value):
+    """A launch that the runtime refuses because not all its blocks are resident is repeated with fewer: same result."""
+    x = np.random.default_rng(m).standard_normal((m, p)).astype(np.float32)
+    x[m - 1, 0] = value
+    t = torch.from_numpy(x).to(U.dev())
+    got, want = hb.higgs_selftest_grid_fit(1, p, n, t), hb.higgs_make_grid(p, n, t, max_iters=100)
+    assert hb.higgs_device_status() == hb.HIGGS_OK
+    assert int(got[2]) == int(want[2])
+    if value < 1:
+        assert torch.equal(got[0], want[0])
+    else:                                                   # (fp64 sums in any order, one rounding to fp32)
+        assert torch.allclose(got[0], want[0], rtol=2.0 ** -22, atol=2.0 ** -22)
