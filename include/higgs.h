@@ -451,7 +451,7 @@ int higgs_selftest_wait(int32_t which, uint32_t polls, int32_t* result_out, void
 /* higgs_make_grid (p <= 2, up to 2^20 samples, 100 iterations at most).  which = 0: its barrier waits for one arrival more than there
  * are blocks, about 2^10 polls long; every block gives up and returns, higgs_device_status() reports HIGGS_ERR_TIMEOUT and the outputs
  * are those of a wait that ran out.  which = 1: it first asks for more blocks than the device holds, which the runtime refuses, and runs
- * with as many as there is room for; the outputs are the usual ones. */
+ * with as many as there is room for; which = 2: the variant for sets of 2^20 samples and more; the outputs of both are the usual ones. */
 int higgs_selftest_grid_fit(int32_t which, int p, int n, const float* samples, int64_t num_samples, float* grid_out, float* mse_out,
                             int32_t* iters_out, void* workspace, size_t workspace_bytes, void* stream);
 

@@ -273,7 +273,7 @@ def higgs_selftest_wait(which: int, polls: int, device=None) -> torch.Tensor:
 
 
 def higgs_selftest_grid_fit(which: int, p: int, n: int, samples: torch.Tensor):
-    """A grid fit whose barrier runs out (which = 0) or whose first launch is refused (1); returns (grid, mse, iters) like higgs_make_grid."""
+    """A grid fit whose barrier runs out (which = 0), whose first launch is refused (1), or the variant for large sets (2); returns (grid, mse, iters) like higgs_make_grid."""
     assert samples.is_cuda and samples.dtype == torch.float32 and samples.is_contiguous()
     m = samples.numel() // p
     d = higgs_desc(p, n, 0, HIGGS_F16, 0, 0, m, HIGGS_LAYOUT_VERSION, 0)

@@ -90,12 +90,12 @@ int higgs_make_grid(int p, int n, const float* samples, int64_t num_samples, int
 
 int higgs_selftest_grid_fit(int32_t which, int p, int n, const float* samples, int64_t num_samples, float* grid_out, float* mse_out, int32_t* iters_out,
                             void* workspace, size_t workspace_bytes, void* stream) {
-    if (which < 0 || which > 1 || !samples || !grid_out || !mse_out || !iters_out || !workspace || !aligned(workspace, 256)) return HIGGS_ERR_INVALID_ARG;
+    if (which < 0 || which > 2 || !samples || !grid_out || !mse_out || !iters_out || !workspace || !aligned(workspace, 256)) return HIGGS_ERR_INVALID_ARG;
     if (p < 1 || p > 2 || n < 1 || n > kMaxGridPoints) return HIGGS_ERR_UNSUPPORTED;
     if (num_samples < n || num_samples > (1 << 20)) return HIGGS_ERR_INVALID_ARG;
     if (workspace_bytes < make_grid_workspace(p, n, num_samples)) return HIGGS_ERR_WORKSPACE;
     return launch_make_grid(p, n, samples, num_samples, 100, grid_out, mse_out, iters_out, workspace, as_stream(stream),
-                            which == 0 ? FitTest::kRunOut : FitTest::kTooManyBlocks);
+                            which == 0 ? FitTest::kRunOut : which == 1 ? FitTest::kTooManyBlocks : FitTest::kAdapt);
 }
 
 int higgs_make_grid_seeded(int p, int n, uint64_t sample_seed, int log2_samples, int max_iters, float* grid_out,

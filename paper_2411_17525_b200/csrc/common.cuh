@@ -399,8 +399,8 @@ bool linear_fused_possible(const higgs_desc& d, int64_t B);
 bool linear_fused_eligible(const higgs_desc& d, int64_t B);
 int launch_convert_out(const float* y32, void* y, int y_dtype, size_t count, cudaStream_t st);
 size_t make_grid_workspace(int p, int n, int64_t m);
-// self-checks of the fit: a barrier that runs out; a first launch that asks for more blocks than are resident
-enum class FitTest { kNone, kRunOut, kTooManyBlocks };
+// self-checks of the fit: a barrier that runs out; a first launch that asks for more blocks than are resident; the variant for large sets
+enum class FitTest { kNone, kRunOut, kTooManyBlocks, kAdapt };
 int launch_make_grid(int p, int n, const float* samples, int64_t m, int max_iters, float* grid_out, float* mse_out,
                      int32_t* iters_out, void* ws, cudaStream_t st, FitTest test = FitTest::kNone);
 // partials: scratch of at least kErrorPartials pairs of doubles

@@ -16,6 +16,7 @@ constexpr int kMinNearCentres = 65;    // grids with lists: below, a scan is no 
 constexpr int kMaxNearCentres = 512;   // ... above, building the lists costs as much as the scans they save
 constexpr int kMaxSharedSums = 1024;   // coordinates whose changes a block collects in shared memory first
 constexpr int kQueueRounds = 4;        // samples a lane tests before the block scans those that need it
+constexpr int64_t kAdaptSamples = 1 << 20;   // sets from which on the fit decides by measured work whether bounds pay
 
 struct GridWs {
     float* centres;               // [n][p]
@@ -23,6 +24,7 @@ struct GridWs {
     int32_t* delta_cnt;           // [3][n]    changes of the cells' sizes
     double* err;                  // [kMaxFitBlocks] squared error of a block's samples; before the fit the range of the samples, as uint2
     unsigned long long* bar;      // [2] grid barrier: arrivals (low half), blocks with a changed assignment (high half)
+    unsigned long long* work;     // [3] scans of an iteration in steps of a warp (three in turn)
     int32_t* flags;               // [0] done, [1] iterations, [2] the samples are left to plain_fit_kernel, [3] a barrier ran out
     uint16_t* near_idx;           // [kMaxNearCentres][kNear] neighbour lists
     float* excl;                  // [kMaxNearCentres]
@@ -40,7 +42,8 @@ GridWs carve(void* ws, int p, int n, int64_t m) {
     w.delta_cnt = reinterpret_cast<int32_t*>(b); b += up256(sizeof(int32_t) * 3 * n);
     w.err = reinterpret_cast<double*>(b); b += up256(sizeof(double) * kMaxFitBlocks);
     w.bar = reinterpret_cast<unsigned long long*>(b);
-    w.flags = reinterpret_cast<int32_t*>(b + 16); b += 256;
+    w.flags = reinterpret_cast<int32_t*>(b + 16);
+    w.work = reinterpret_cast<unsigned long long*>(b + 64); b += 256;
     w.near_idx = reinterpret_cast<uint16_t*>(b); b += sizeof(uint16_t) * kMaxNearCentres * kNear;
     w.excl = reinterpret_cast<float*>(b); b += sizeof(float) * kMaxNearCentres;
     w.assign = reinterpret_cast<int32_t*>(b); b += up256(sizeof(int32_t) * (size_t)m);
@@ -58,6 +61,7 @@ __global__ void __launch_bounds__(kRangeThreads) grid_init_kernel(GridWs w, cons
     for (int64_t i = first; i < n * p; i += step) w.centres[i] = samples[i];       // (the result if a barrier runs out)
     if (first < 2) w.bar[first] = 0;
     if (first < 8) w.flags[first] = 0;
+    if (first < 3) w.work[first] = 0;
     unsigned top = 0u;
     for (int64_t i = first; i < m; i += step) {
         w.assign[i] = -1;
@@ -292,10 +296,16 @@ inline size_t fit_smem(int p, int n) {
 //     its own copy of the sums and computes the new centres itself, so no second barrier is needed.  Three buffers take
 //     turns: the changes of iteration i are read after its barrier; block 0 clears those of i - 1, which every block has
 //     read before it arrived there, for iteration i + 2.
+//   * Large sets (ADAPT) are bound by the scans, not by latency, and bounds then have to pay for themselves: keeping the second-best
+//     distance makes a scan 1.3 times as long, and while the centres still move much, or without lists, most samples are scanned all the
+//     same.  The fit starts with four iterations of plain scans (one with lists of a sixth of the centres); then one that sets the bounds, then bounded ones, whose scans are
+//     counted.  When they cost more than 0.85 of scanning everything, plain iterations follow, 8, 16, 32, 64, and another try.  (2^24 samples,
+//     30 iterations, plain scans with fp64 sums / bounds always / this, in ms: p = 2, n = 16 9.3 / 7.5 / 4.8, n = 64 11.1 / 17.3 / 11.2, n = 65
+//     11.5 / 13.0 / 11.4, n = 256 34.8 / 14.9 / 15.1, n = 600 84.9 / 88.6 / 75.8.  Below 2^20 samples bounds are ahead from the start.)
 // Bound: latency - per iteration about 2.5 us of barrier, 2 us of update, 2.5 us to test the samples and 1 to 2 us of scans.
 // p = 2, n = 256, 2^18 samples: 37 -> 9 us per iteration (before: every sample scanned all centres every time, sums by
 // fp64 atomics in shared memory, two barriers).  One barrier and movement bounds without lists: 12.4 us.
-template <int P, bool RUN_OUT>
+template <int P, bool RUN_OUT, bool ADAPT>
 __global__ void __launch_bounds__(kFitThreads, 1) grid_fit_kernel(GridWs w, const float* __restrict__ samples, int n, int64_t m, int slots, int max_iters) {
     extern __shared__ __align__(16) unsigned char grid_smem[];
     const bool shared_sums = n * P <= kMaxSharedSums, lists = fit_lists(n);
@@ -344,7 +354,10 @@ __global__ void __launch_bounds__(kFitThreads, 1) grid_fit_kernel(GridWs w, cons
     // scanning one sample: n steps of its lane, or ceil(n / 32) steps and a reduction of the whole warp
     const int scan_all = max(1, 9 * n / (9 * ((n + 31) / 32) + 45));
     float moved = 0.f, moved_at_build = 0.f;    // sum over the iterations of the largest movement of any centre
-    bool fresh = lists;                         // the lists have to be (have just been) built
+    bool fresh = lists && !ADAPT;               // the lists have to be (have just been) built
+    int plain_left = lists && n >= 192 ? 1 : 4, plain_next = 8;         // ADAPT: plain iterations until bounds are set, and after the next futile try
+    bool set_bounds = false;                    // ADAPT: this iteration scans everything and sets the bounds
+    unsigned work = 0u;                         // ADAPT: this warp's scans
     double err = 0.0;
     int it = 0;
     bool done = false;
@@ -413,10 +426,7 @@ __global__ void __launch_bounds__(kFitThreads, 1) grid_fit_kernel(GridWs w, cons
                 atomicAdd(reinterpret_cast<unsigned long long*>(&delta[cell * P + k]), (unsigned long long)v);
             }
         };
-        // the outcome of a scan: the bound on every other centre, and the cell if it changed
-        auto settle = [&](int64_t i, const float (&x)[P], int a, int to, float second) {
-            w.lower[i] = __fadd_rd(second, lists ? near_moved[to] : moved);
-            if (to == a) return;
+        auto move = [&](int64_t i, const float (&x)[P], int a, int to) {
             w.assign[i] = to;
             changed = 1;
 #pragma unroll
@@ -429,7 +439,25 @@ __global__ void __launch_bounds__(kFitThreads, 1) grid_fit_kernel(GridWs w, cons
             atomicAdd(&dc[to], 1);
             if (a >= 0) atomicAdd(&dc[a], -1);
         };
-        for (int64_t batch = 0; batch * chunk_step < chunks; batch += kQueueRounds) {
+        // the outcome of a scan: the bound on every other centre, and the cell if it changed
+        auto settle = [&](int64_t i, const float (&x)[P], int a, int to, float second) {
+            w.lower[i] = __fadd_rd(second, lists ? near_moved[to] : moved);
+            if (to != a) move(i, x, a, to);
+        };
+        const bool plain = ADAPT && plain_left > 0;
+        if (plain) {
+            for (int64_t c = chunk0; c < chunks; c += chunk_step) {
+                const int64_t i = c * 32 + lane;
+                if (i >= m) continue;
+                float x[P], best;
+#pragma unroll
+                for (int k = 0; k < P; ++k) x[k] = samples[i * P + k];
+                const int a = w.assign[i], to = nearest_centre<P>(x, sc, n, best);
+                if (to != a) move(i, x, a, to);
+                if (last) err += (double)best;
+            }
+        }
+        for (int64_t batch = 0; !plain && batch * chunk_step < chunks; batch += kQueueRounds) {
             for (int r = 0; r < kQueueRounds; ++r) {
                 const int64_t c = chunk0 + (batch + r) * chunk_step;
                 if (c >= chunks) break;
@@ -440,9 +468,9 @@ __global__ void __launch_bounds__(kFitThreads, 1) grid_fit_kernel(GridWs w, cons
                 for (int k = 0; k < P; ++k) x[k] = valid ? samples[i * P + k] : 0.f;
                 const int a = valid ? w.assign[i] : 0;
                 const float lower = valid ? w.lower[i] : 0.f;           // (not yet written in the first iteration, and not used)
-                bool need = valid && a < 0, listed = false;
+                bool need = valid && (ADAPT ? set_bounds : a < 0), listed = false;
                 float best = 0.f;
-                if (valid && a >= 0) {
+                if (valid && (ADAPT ? !set_bounds : a >= 0)) {
                     best = centre_distance<P>(x, sc + a * P);
                     const float u = __fsqrt_ru(__fmul_ru(best, 1.000004f));
                     if (lists) {
@@ -470,8 +498,10 @@ __global__ void __launch_bounds__(kFitThreads, 1) grid_fit_kernel(GridWs w, cons
                         best = b;
                         settle(i, x, a, bi, __fsqrt_rd(__fmul_rd(s2, 0.999996f)));
                     }
+                    if (ADAPT) work += (unsigned)n + (unsigned)n / 4u;
                     if (last && valid) err += (double)best;
                 } else {
+                    if (ADAPT) work += 10u + (unsigned)__popc(by_list) * 3u + (unsigned)__popc(todo & ~by_list) * ((unsigned)n / 32u + 8u);
                     int at = 0;
                     if (lane == 0 && todo) at = atomicAdd(&s_queued[qi], __popc(todo));
                     at = __shfl_sync(0xffffffffu, at, 0);
@@ -549,6 +579,10 @@ __global__ void __launch_bounds__(kFitThreads, 1) grid_fit_kernel(GridWs w, cons
             }
             if ((batch + kQueueRounds) * chunk_step < chunks) __syncthreads();      // (the queue is written again)
         }
+        if (ADAPT && !plain) {
+            if (lane == 0) atomicAdd(&w.work[buf], (unsigned long long)work);
+            work = 0u;
+        }
         const bool block_changed = __syncthreads_or(changed) != 0;
         if (shared_sums && block_changed) {
             for (int q = tid; q < n * P; q += kFitThreads) {
@@ -584,11 +618,22 @@ __global__ void __launch_bounds__(kFitThreads, 1) grid_fit_kernel(GridWs w, cons
             const int old = (it + 2) % 3;
             for (int i = tid; i < n * P; i += kFitThreads) w.delta[(size_t)old * n * P + i] = 0;
             for (int i = tid; i < n; i += kFitThreads) w.delta_cnt[(size_t)old * n + i] = 0;
+            if (ADAPT && tid == 0) w.work[old] = 0;
         }
         __syncthreads();
         moved = __fadd_ru(moved, __uint_as_float(s_move[it & 1]));
         if (tid == 0) s_move[(it + 1) & 1] = 0u;       // (last read before the barrier of this iteration)
-        if (lists) {
+        if (ADAPT) {
+            const bool tried = !plain && !set_bounds;
+            set_bounds = plain && --plain_left == 0;
+            if (tried && __ldcg(&w.work[buf]) * 20 > (unsigned long long)chunks * (unsigned)n * 17) {
+                plain_left = plain_next;
+                plain_next = min(2 * plain_next, 64);
+            }
+        }
+        if (ADAPT && (plain || plain_left > 0)) {
+            fresh = lists && set_bounds;
+        } else if (lists) {
             fresh = __fsub_ru(moved, moved_at_build) > 0.15f * __uint_as_float(s_min_excl);
             // four threads per cell: the largest movement among its list
             for (int q = tid; q < ((4 * n + 31) & ~31); q += kFitThreads) {
@@ -739,17 +784,17 @@ static int launch_resident(void (*kernel)(Args...), int* blocks, size_t smem, cu
     return cuda_status(cudaGetLastError());
 }
 
-template <int P, bool RUN_OUT>
+template <int P, bool RUN_OUT, bool ADAPT>
 static int launch_fit(GridWs w, const float* samples, int n, int64_t m, int slots, int max_iters, int crowd, int (&blocks_out)[2], cudaStream_t st) {
     constexpr size_t kMaxSmem = (P * (sizeof(long long) + sizeof(float)) + sizeof(int)) * kMaxGridPoints;     // (n = 4096: no lists)
     static int state[64] = {0};           // 1 = cooperative launch possible, 2 = not, -1 = failed
     const int how = device_once(state, [] {
         int dev = 0, coop = 0, v = 0;
-        if (cudaFuncSetAttribute(grid_fit_kernel<P, RUN_OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxSmem > 73728 ? kMaxSmem : 73728)) != cudaSuccess ||
+        if (cudaFuncSetAttribute(grid_fit_kernel<P, RUN_OUT, ADAPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxSmem > 73728 ? kMaxSmem : 73728)) != cudaSuccess ||
             cudaFuncSetAttribute(plain_fit_kernel<P, RUN_OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) != cudaSuccess)
             return -1;
         if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, grid_fit_kernel<P, RUN_OUT>, kFitThreads, kMaxSmem) != cudaSuccess || v < 1)
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, grid_fit_kernel<P, RUN_OUT, ADAPT>, kFitThreads, kMaxSmem) != cudaSuccess || v < 1)
             return 2;
         return 1;
     });
@@ -758,7 +803,7 @@ static int launch_fit(GridWs w, const float* samples, int n, int64_t m, int slot
     if (blocks > sm_count_of_device()) blocks = sm_count_of_device();
     if (blocks > kMaxFitBlocks) blocks = kMaxFitBlocks;
     blocks_out[0] = blocks_out[1] = (int)blocks * crowd;
-    const int rc = launch_resident(grid_fit_kernel<P, RUN_OUT>, &blocks_out[0], fit_smem(P, n), st, w, samples, n, m, slots, max_iters);
+    const int rc = launch_resident(grid_fit_kernel<P, RUN_OUT, ADAPT>, &blocks_out[0], fit_smem(P, n), st, w, samples, n, m, slots, max_iters);
     if (rc != HIGGS_OK) return rc;
     return launch_resident(plain_fit_kernel<P, RUN_OUT>, &blocks_out[1], (size_t)n * (P * (sizeof(double) + sizeof(float)) + sizeof(int)), st, w, samples, n, m, max_iters);
 }
@@ -772,13 +817,17 @@ int launch_make_grid(int p, int n, const float* samples, int64_t m, int max_iter
     grid_range_kernel<<<(unsigned)slots, kRangeThreads, 0, st>>>(w, samples, p, m, slots);
     int blocks[2] = {0, 0}, rc = HIGGS_ERR_UNSUPPORTED;
     const int crowd = test == FitTest::kTooManyBlocks ? 4 : 1;
-    switch (2 * p + (test == FitTest::kRunOut ? 1 : 0)) {
-        case 2: rc = launch_fit<1, false>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
-        case 3: rc = launch_fit<1, true>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
-        case 4: rc = launch_fit<2, false>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
-        case 5: rc = launch_fit<2, true>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
-        case 6: rc = launch_fit<3, false>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
-        case 8: rc = launch_fit<4, false>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
+    switch (4 * p + (test == FitTest::kRunOut ? 1 : test == FitTest::kAdapt || m >= kAdaptSamples ? 2 : 0)) {
+        case 4: rc = launch_fit<1, false, false>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
+        case 5: rc = launch_fit<1, true, false>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
+        case 6: rc = launch_fit<1, false, true>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
+        case 8: rc = launch_fit<2, false, false>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
+        case 9: rc = launch_fit<2, true, false>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
+        case 10: rc = launch_fit<2, false, true>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
+        case 12: rc = launch_fit<3, false, false>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
+        case 14: rc = launch_fit<3, false, true>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
+        case 16: rc = launch_fit<4, false, false>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
+        case 18: rc = launch_fit<4, false, true>(w, samples, n, m, slots, max_iters, crowd, blocks, st); break;
     }
     if (rc != HIGGS_OK) return rc;
     grid_finalize_kernel<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(w, p, n, m, blocks[0], blocks[1], grid_out, mse_out, iters_out);

@@ -147,7 +147,7 @@ def test_seeded_grid_and_helper_arguments():
     assert L.higgs_launch_floor(148, 2048, 0, None) == hb.HIGGS_ERR_INVALID_ARG
     assert L.higgs_selftest_wait(0, 100, None, None) == hb.HIGGS_ERR_INVALID_ARG
     assert L.higgs_selftest_wait(2, 100, a, None) == hb.HIGGS_ERR_INVALID_ARG
-    assert L.higgs_selftest_grid_fit(2, 2, 256, a, 1000, a, a, a, a, 1 << 30, None) == hb.HIGGS_ERR_INVALID_ARG
+    assert L.higgs_selftest_grid_fit(3, 2, 256, a, 1000, a, a, a, a, 1 << 30, None) == hb.HIGGS_ERR_INVALID_ARG
     assert L.higgs_selftest_grid_fit(0, 3, 256, a, 1000, a, a, a, a, 1 << 30, None) == hb.HIGGS_ERR_UNSUPPORTED
     assert L.higgs_selftest_grid_fit(0, 2, 256, a, 1000, a, a, a, a, 16, None) == hb.HIGGS_ERR_WORKSPACE
 

@@ -132,3 +132,15 @@ def test_fewer_resident_blocks_than_asked_for(p, n, m, value):
         assert torch.equal(got[0], want[0])
     else:                                                   # (fp64 sums in any order, one rounding to fp32)
         assert torch.allclose(got[0], want[0], rtol=2.0 ** -22, atol=2.0 ** -22)
+
+
+@pytest.mark.parametrize("p,n,m", [(1, 4, 31), (2, 16, 8192), (1, 64, 3000), (2, 65, 9000), (1, 256, 4000), (2, 512, 5001), (2, 600, 5000)])
+def test_the_variant_for_large_sets(p, n, m):
+    """Plain iterations in turn with bounded ones, where bounds pay and where they do not."""
+    x = np.random.default_rng(3 * n + m).standard_normal((m, p)).astype(np.float32)
+    c, err, iters = plain_lloyd(p, n, x, 100)
+    grid, mse, it = hb.higgs_selftest_grid_fit(2, p, n, torch.from_numpy(x).to(U.dev()))
+    assert hb.higgs_device_status() == hb.HIGGS_OK
+    assert int(it) == iters
+    assert np.max(np.abs(grid.cpu().numpy() - c[np.lexsort(c.T[::-1])])) <= 2.0 ** -22
+    assert abs(float(mse) - err / (m * p)) <= 1e-6 * err / (m * p) + 1e-30
