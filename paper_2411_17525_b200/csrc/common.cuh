@@ -87,6 +87,8 @@ inline int device_once(int (&state)[64], F&& setup) {
 // touches anything the previous kernel may read or write.  pdl_trigger() lets the next kernel
 // start as early as possible.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Data that the previous kernel may still be writing when this one starts is read with __ldcg after the wait, and its pointer is
+// not __restrict__: the read-only path is for data that nobody writes while the kernel runs.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>

@@ -181,12 +181,12 @@ __global__ void __launch_bounds__(kDqWarps * 32, 2) packed_rows_kernel(const uin
     }
 }
 
-__global__ void __launch_bounds__(64) error_total_kernel(const double* __restrict__ partials, int blocks, double* __restrict__ sums) {
+__global__ void __launch_bounds__(64) error_total_kernel(const double* partials, int blocks, double* __restrict__ sums) {
     __shared__ double total[2];
     const int which = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double s = 0.0;
     pdl_wait();
-    for (int i = lane; i < blocks; i += 32) s += partials[2 * i + which];
+    for (int i = lane; i < blocks; i += 32) s += __ldcg(&partials[2 * i + which]);
 #pragma unroll
     for (int m = 16; m > 0; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
     if (lane == 0) { total[which] = s; sums[which] = s; }

@@ -886,11 +886,11 @@ __global__ void wait_selftest_kernel(uint32_t limit, int* result) {
     if ((threadIdx.x & 31) == 0) result[threadIdx.x >> 5] = ok ? 1 : 0;
 }
 
-__global__ void convert_out_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, size_t count) {
+__global__ void convert_out_kernel(const float* src, __nv_bfloat16* __restrict__ dst, size_t count) {
     size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     pdl_trigger();
     pdl_wait();
-    if (i < count) dst[i] = __float2bfloat16_rn(src[i]);
+    if (i < count) dst[i] = __float2bfloat16_rn(__ldcg(src + i));
 }
 
 int sm_count() {
@@ -1100,13 +1100,13 @@ int launch_linear_mma(const higgs_desc& d, const __half* xdag, int64_t B, const 
 
 // A K-split product accumulates into a contiguous fp32 [B][N]; this spreads it to the gathered destinations.
 struct ScatterDst { void* y[kMaxGather]; int n; };
-__global__ void scatter_out_kernel(const float* __restrict__ src, int64_t B, int64_t N, ScatterDst dst, int64_t ldy, int bf16) {
+__global__ void scatter_out_kernel(const float* src, int64_t B, int64_t N, ScatterDst dst, int64_t ldy, int bf16) {
     pdl_trigger();
     pdl_wait();
     const int64_t quads = N / 4;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < B * quads; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = i / quads, c = (i % quads) * 4;
-        const float4 v = *reinterpret_cast<const float4*>(src + b * N + c);
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(src + b * N + c));
         for (int pd = 0; pd < dst.n; ++pd) {
             if (bf16) {
                 const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);

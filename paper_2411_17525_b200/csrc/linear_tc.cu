@@ -698,7 +698,7 @@ namespace {
 // one warp's transform.  1999 tokens x 4096: 22 -> 10.0 us, x 14336: 69 -> 29.7 us (before: four warps per group with five
 // shuffle stages, 16-byte stores 128 bytes apart).
 constexpr int kRotWarps = 8;
-__global__ void __launch_bounds__(kRotWarps * 32) rht_activations_tc_kernel(const __nv_bfloat16* __restrict__ x, __half* __restrict__ xdag,
+__global__ void __launch_bounds__(kRotWarps * 32) rht_activations_tc_kernel(const __nv_bfloat16* x, __half* __restrict__ xdag,
                                                                             int64_t B, int64_t K, uint64_t xi, int BN) {
     __shared__ __align__(16) float ex[kRotWarps][kFwhtExchange];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -715,7 +715,7 @@ __global__ void __launch_bounds__(kRotWarps * 32) rht_activations_tc_kernel(cons
         const uint4* src = reinterpret_cast<const uint4*>(x + b * K + (int64_t)gi * kGroup) + lane;
         uint4 raw[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) raw[c] = __ldg(src + c * 32);
+        for (int c = 0; c < 4; ++c) raw[c] = __ldcg(src + c * 32);
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             const uint32_t w[4] = {raw[c].x, raw[c].y, raw[c].z, raw[c].w};

@@ -53,7 +53,7 @@ __device__ __forceinline__ void load_group<float>(const float* __restrict__ src,
 // bit, as the rotation fused into the product kernel.)
 // Threads also clear `zero_ptr` (the fp32 accumulation target of a K-split product) so that no separate memset launch
 // is needed.
-__global__ void __launch_bounds__(32) rht_activations_kernel(const __nv_bfloat16* __restrict__ x, __half* __restrict__ xdag,
+__global__ void __launch_bounds__(32) rht_activations_kernel(const __nv_bfloat16* x, __half* __restrict__ xdag,
                                                              int64_t B, int64_t K, uint64_t xi,
                                                              float* __restrict__ zero_ptr, size_t zero_floats) {
     __shared__ __align__(16) uint8_t ex[2048];
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(32) rht_activations_kernel(const __nv_bfloat16
     {
         uint4 raw[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) raw[c] = reinterpret_cast<const uint4*>(src)[c];
+        for (int c = 0; c < 4; ++c) raw[c] = __ldcg(reinterpret_cast<const uint4*>(src) + c);
 #pragma unroll
         for (int t = 0; t < 16; ++t) {
             const uint4 r = raw[t >> 2];

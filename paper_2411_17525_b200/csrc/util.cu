@@ -24,14 +24,14 @@ __global__ void gaussian_samples_kernel(int p, uint64_t seed, int64_t count, flo
 }
 
 // Sums `world` fp32 slots of `count` values in slot order (a fixed order: the result is reproducible) into y.
-__global__ void reduce_slots_kernel(const float* __restrict__ slots, int world, int64_t count, void* __restrict__ y, int bf16) {
+__global__ void reduce_slots_kernel(const float* slots, int world, int64_t count, void* __restrict__ y, int bf16) {
     pdl_trigger();
     pdl_wait();
     const int64_t quads = count / 4;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < quads; i += (int64_t)gridDim.x * blockDim.x) {
-        float4 acc = *reinterpret_cast<const float4*>(slots + 4 * i);
+        float4 acc = __ldcg(reinterpret_cast<const float4*>(slots + 4 * i));
         for (int r = 1; r < world; ++r) {
-            const float4 v = *reinterpret_cast<const float4*>(slots + (int64_t)r * count + 4 * i);
+            const float4 v = __ldcg(reinterpret_cast<const float4*>(slots + (int64_t)r * count + 4 * i));
             acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
         }
         if (bf16) {

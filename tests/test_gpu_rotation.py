@@ -45,3 +45,36 @@ def test_a_call_without_workspace(N, K, B, one_launch):
     ref = hb.higgs_linear(d, x, packed, scales, grid, workspace=torch.empty(hb.higgs_workspace_bytes(d, hb.HIGGS_OP_LINEAR, B), dtype=torch.uint8, device=U.dev()))
     assert torch.equal(y, ref) if one_launch else y.isnan().all()
     assert torch.equal(hb.higgs_linear(d, x, packed, scales, grid), ref)
+
+
+@pytest.mark.parametrize("B", [1, 2, 5, 16, 40])
+@pytest.mark.parametrize("N,K", [(1024, 1024), (2048, 2048), (8192, 2048)])
+def test_a_chain_reads_what_the_product_before_it_wrote(N, K, B):
+    """Every kernel starts while the one before it runs; activations that it has just written, over older ones that were read a moment
+    ago, are what the next product sees."""
+    g = torch.Generator(device="cuda").manual_seed(B)
+    _, grid = U.grid32(2, 256)
+    down, up = hb.make_desc(2, 256, K, N, 7), hb.make_desc(2, 256, N, K, 8)
+    weights = [(torch.randint(0, 256, (N * K // 2,), dtype=torch.uint8, device="cuda", generator=g),
+                (torch.rand(N * K // 1024, device="cuda", generator=g) * (2.0 / inputs) ** 0.5).half()) for inputs in (K, N)]
+    x0 = torch.randn(B, K, device="cuda", generator=g).to(torch.bfloat16)
+    ws = torch.empty(max(hb.higgs_workspace_bytes(d, hb.HIGGS_OP_LINEAR, B) for d in (up, down)), dtype=torch.uint8, device="cuda")
+
+    def run(steps, wait):
+        x, h, seen = x0.clone(), torch.zeros(B, N, dtype=torch.bfloat16, device="cuda"), []
+        for _ in range(steps):
+            hb.higgs_linear(up, x, *weights[0], grid, workspace=ws, y=h)
+            if wait:
+                torch.cuda.synchronize()
+            hb.higgs_linear(down, h, *weights[1], grid, workspace=ws, y=x)
+            if wait:
+                torch.cuda.synchronize()
+                seen.append(x.clone())
+        return seen if wait else x
+
+    seen = run(12, True)
+    assert torch.isfinite(seen[-1].float()).all() and seen[-1].float().abs().max() > 1e-3
+    if any(hb.higgs_linear_uses_atomics(d, B) for d in (up, down)):
+        pytest.skip("K ranges that meet in atomics: no two runs are alike")
+    for steps in (1, 2, 5, 12):
+        assert torch.equal(run(steps, False), seen[steps - 1])
