@@ -8,8 +8,8 @@ effective weight bandwidth (packed codes + scales bytes of the layer set / time 
 (Algorithm 1) and the grid fit (Algorithm 2) run once during set-up, on the GPU, and are reported separately.
 
 The default workload is the largest single-GPU configuration: the Llama-3.1-70B layer shapes with the seeded 3/4-bit
-assignment (3.5 bits per weight on average), batch 1.  The same run reports, under "detail", one row per layer, grid
-and batch of the other configurations (8B shapes at three grids and batches 1/4/16, and at batches 64/256 with
+assignment (3.5 bits per weight on average), batch 1.  The same run reports, under "detail" in bench_detail.json (the
+printed line holds the results alone and stays short), one row per layer, grid and batch of the other configurations (8B shapes at three grids and batches 1/4/16, and at batches 64/256 with
 log-normal channel scales; 1B shapes at batches 1/16), each with its share of the roofline and a parity check of the
 timed output against the fp64 oracle on sampled rows.
 
@@ -293,6 +293,32 @@ def cpu_baseline(layers, pn, cfg, xi, grids64, B):
 
 
 # --------------------------------------------------------------------------------------------- our arm: helpers
+DETAIL_FILE = "bench_detail.json"
+
+
+def headline(line: dict) -> dict:
+    """The printed line: what readers of the last few KB of the output need.  The rows of the other configurations and the notes on how
+    things were measured made it 28 KB, of which such a reader saw the end without the value."""
+    short = {k: v for k, v in line.items() if k not in ("detail", "per_replay", "quantize", "cpu_baseline")}
+    if line.get("quantize"):
+        short["quantize"] = {k: line["quantize"][k] for k in ("weights_per_s", "ms", "weights")}
+    if line.get("cpu_baseline"):
+        short["cpu_baseline"] = {k: line["cpu_baseline"][k] for k in ("value", "unit", "cores", "kind")}
+    return short
+
+
+def report(line: dict) -> None:
+    """The whole record into DETAIL_FILE beside this script, its headline to stdout."""
+    short = headline(line)
+    try:
+        with open(os.path.join(ROOT, DETAIL_FILE), "w") as f:
+            json.dump(line, f)
+        short["detail_file"] = DETAIL_FILE
+    except OSError as e:
+        short["detail_file"] = f"not written: {e.strerror}"
+    print(json.dumps(short))
+
+
 def divisor_at_most(steps: int, cap: int) -> int:
     """Largest divisor of `steps` that is <= cap (>= 1): `steps` steps then run from steps / d equal graphs."""
     for d in range(max(1, min(cap, steps)), 0, -1):
@@ -918,7 +944,7 @@ def run_ours(args):
                        "global_batch": B * world, "parallelism": f"replicas x{world}",
                        "l2": f"rotating {copies} weight copies ({copies * set_bytes / 1e6:.0f} MB > 126 MB L2)",
                        "launch": "direct" if args.no_graph else f"CUDA graphs of {spg} consecutive steps over rotating weight copies ({args.steps // spg} replays timed)",
-                       "step": "one transformer block, 7 matrices: layers that read the same input and share a grid (here: " + merged_names + ") run as one product over their concatenated rows (higgs_linear_multi); other sharing layers share one rotation (higgs_linear_share + higgs_linear_prerotated); a layer with its own input goes through higgs_linear; for 1-2 tokens the rotation runs inside the product kernel"},
+                       "step": "one transformer block, 7 matrices: layers that read the same input and share a grid (here: " + merged_names + ") run as one product over their concatenated rows (higgs_linear_multi); other sharing layers share one rotation (higgs_linear_share + higgs_linear_prerotated); a layer with its own input goes through higgs_linear; for 1-2 tokens the rotation of a small layer runs inside the product kernel"},
             "us_per_layer": ms_per_step * 1e3 / len(layers),
             "per_replay": per_replay,
             "weight_bytes_per_step": set_bytes,
@@ -934,7 +960,7 @@ def run_ours(args):
                          "rooflines": encoder_rooflines(wps, pn, [N * K for _, N, K in layers], clocks, peak, peak_src)},
             "detail": detail,
         }
-        print(json.dumps(line))
+        report(line)
     if world > 1:
         dist.destroy_process_group()
 

@@ -1,5 +1,6 @@
 """world_size-2 gloo test of the benchmark's multi-rank logic (replicas only: no data-path collective): the timed
 region's duration is the MAX over ranks, the reported value the sum of all ranks' bytes over that time."""
+import json
 import os
 import socket
 
@@ -202,3 +203,19 @@ def test_reference_arm_prints_the_contract_line():
     assert line["e2e"]["h2d_bytes_per_step"] == 0 and line["e2e"]["d2h_bytes_per_step"] == 0
     assert line["config"]["workload"].startswith("llama-3.1-70b layer set (7 matrices), grid mixed ")
     assert line["config"]["workload"].endswith("g=1024, batch 1")
+
+
+def test_the_printed_line_is_short_and_complete():
+    """The full record has tens of KB; what is printed keeps every result and fits the last 3 KB of an output."""
+    note = "x" * 600
+    line = {"metric": "m", "value": 1.0 / 3, "unit": "GB/s", "n_gpus": 1, "steps": 200, "warmup": 10, "ms_per_step": 0.1234567890123, "higher_is_better": True,
+            "scaling": "weak", "vs_baseline": None, "dtype": "f16xf16->f32", "data": "synthetic", "config": {"workload": note, "step": note},
+            "e2e": {"value": 1.0, "unit": "GB/s", "h2d_bytes_per_step": 1, "d2h_bytes_per_step": 2}, "gpu_launches": 5,
+            "clocks": {"sm_mhz": 1965, "sm_max_mhz": 1965, "reasons": []}, "roofline": {"bound": "hbm", "frac": 0.5, "note": note},
+            "per_replay": [0.1] * 500, "cpu_baseline": {"value": 1.0, "unit": "GB/s", "cores": 16, "kind": "oracle", "sample": note},
+            "quantize": {"weights_per_s": 1e11, "ms": 2.0, "weights": 10 ** 9, "calls": note, "rooflines": [note] * 3}, "detail": {"layers": [{"us": 1.0}] * 1000}}
+    short = bench.headline(line)
+    assert len(json.dumps(short)) < 3000
+    for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline", "dtype", "data",
+              "config", "e2e", "gpu_launches", "clocks", "roofline"):
+        assert short[k] == line[k]
