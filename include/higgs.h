@@ -464,6 +464,9 @@ int higgs_selftest_grid_fit(int32_t which, int p, int n, const float* samples, i
  * (larger batches) sums the ranges of a tile in a fixed order inside a cluster too. */
 int higgs_linear_uses_atomics(const higgs_desc* desc, int64_t B);
 int higgs_linear_k_splits(const higgs_desc* desc, int64_t B);
+/* Tokens that one block of the tensor-core path's product takes (0 where another kernel runs).  It may be narrower than the token tile of
+ * the rotated activations (higgs_rotated_layout), to fill the last wave of blocks. */
+int higgs_linear_token_tile(const higgs_desc* desc, int64_t B);
 
 /* Number of kernels one higgs_linear call enqueues for this shape and batch. */
 int higgs_linear_launch_count(const higgs_desc* desc, int64_t B, int y_dtype);

@@ -26,7 +26,7 @@ EXPORTS = [
     "higgs_encoder_table_bytes", "higgs_make_encoder_table", "higgs_quantize_prepared",
     "higgs_pack_codes", "higgs_unpack_codes", "higgs_rotate_activations", "higgs_linear_prerotated",
     "higgs_linear_host", "higgs_linear_host_workspace_bytes", "higgs_linear_launch_count", "higgs_device_status",
-    "higgs_linear_static", "higgs_linear_static_capacity", "higgs_linear_k_splits", "higgs_rotated_bytes",
+    "higgs_linear_static", "higgs_linear_static_capacity", "higgs_linear_k_splits", "higgs_linear_token_tile", "higgs_rotated_bytes",
     "higgs_rotated_layout", "higgs_dequantize", "higgs_make_uniform_grid", "higgs_layer_error",
     "higgs_allocate_bits", "higgs_general_tuples", "higgs_quantize_general", "higgs_linear_host_batch",
     "higgs_linear_gather", "higgs_linear_share", "higgs_make_grid_seeded", "higgs_gaussian_samples", "higgs_shard_rows",
@@ -95,6 +95,8 @@ def _load() -> ctypes.CDLL:
     lib.higgs_rotated_bytes.argtypes = [P, i64]
     lib.higgs_rotated_layout.restype = i32
     lib.higgs_rotated_layout.argtypes = [P, i64]
+    lib.higgs_linear_token_tile.restype = i32
+    lib.higgs_linear_token_tile.argtypes = [P, i64]
     lib.higgs_linear_k_splits.restype = i32
     lib.higgs_linear_k_splits.argtypes = [P, i64]
     lib.higgs_linear_uses_atomics.restype = i32
@@ -642,6 +644,10 @@ def higgs_rotated_layout(desc: higgs_desc, B: int) -> int:
 
 def higgs_linear_k_splits(desc: higgs_desc, B: int) -> int:
     return int(lib.higgs_linear_k_splits(ctypes.byref(desc), int(B)))
+
+
+def higgs_linear_token_tile(desc: higgs_desc, B: int) -> int:
+    return int(lib.higgs_linear_token_tile(ctypes.byref(desc), int(B)))
 
 
 def higgs_linear_uses_atomics(desc: higgs_desc, B: int) -> bool:

@@ -722,6 +722,11 @@ int higgs_linear_k_splits(const higgs_desc* d, int64_t B) {
     return linear_k_chunks(*d, B);
 }
 
+int higgs_linear_token_tile(const higgs_desc* d, int64_t B) {
+    if (check_desc(d) != HIGGS_OK || B < 1 || d->N == 0 || d->K == 0 || !tc_eligible(*d, B)) return 0;
+    return tc_product_tile(*d, B);
+}
+
 int higgs_linear_uses_atomics(const higgs_desc* d, int64_t B) {
     if (check_desc(d) != HIGGS_OK || B < 1 || d->N == 0 || d->K == 0) return 0;
     if (tc_eligible(*d, B)) return 0;

@@ -868,6 +868,9 @@ static int tc_token_tile(const higgs_desc& d, int64_t B) {
     return best_bn;
 }
 
+// the token tile of a product's launch
+int tc_product_tile(const higgs_desc& d, int64_t B) { return tc_k_split(d, B) == 1 ? tc_token_tile(d, B) : tc_batch_tile(B); }
+
 namespace {
 
 // cuTensorMapEncodeTiled through the runtime's driver-entry-point query (the library does not link libcuda).
@@ -913,7 +916,7 @@ int launch_linear_tc(const higgs_desc& d, const __half* xdag_tc, int64_t B, cons
                      const MultiSegments* segs) {
     if (more && more->count > kMaxGather - 1) return HIGGS_ERR_INVALID_ARG;
     if (segs && (segs->count < 1 || segs->count > kMaxMulti || more)) return HIGGS_ERR_INVALID_ARG;
-    const int ksplit = tc_k_split(d, B), BN = ksplit == 1 ? tc_token_tile(d, B) : tc_batch_tile(B);
+    const int ksplit = tc_k_split(d, B), BN = tc_product_tile(d, B);
     const int64_t tiles = (B + BN - 1) / BN;
     static int configured[64] = {0};
     const int conf = device_once(configured, [] {
