@@ -104,12 +104,12 @@ def measured_peaks():
 
 
 # Encoder rooflines.  ALU: the pruned search is bound by instruction issue (profiles/encode_pruned_kernel_...): ncu
-# counted 3748 warp instructions per (row, group) task of 1024 weights for p=2 n=256 (smsp__inst_executed.sum / tasks);
+# counted 1497 warp instructions per (row, group) task of 1024 weights for p=2 n=256 (smsp__inst_executed.sum / tasks);
 # achieved = weights/s x that count, against 148 SMs x 4 schedulers x 1 warp instruction per clock.  It is derived from
 # the measured weights/s and a counted constant, not read from a counter in this run.  HBM: what the encoder must move
 # per weight - the bf16 weight in, log2(n)/p bits of code and 16/1024 bits of scale out - against the copy peak; this
 # is the floor an exact pruned search approaches.
-ENCODER_WARP_INSTR_PER_WEIGHT = {(2, 256): 1776.0 / 1024.0}
+ENCODER_WARP_INSTR_PER_WEIGHT = {(2, 256): 1497.0 / 1024.0}
 
 
 def encoder_rooflines(weights_per_s, pn, sizes, clocks, hbm_peak, peak_src):

@@ -286,7 +286,7 @@ int higgs_linear_share(const higgs_desc* desc, const void* x, int64_t B, const v
  * independent per output row, so matrices with the same K, grid, group size and seed are one layer over their
  * concatenated rows - the activations are rotated once and, for batches up to 16 (the small-batch kernel, K ranges
  * not meeting in atomics), one kernel launch per 16 tokens streams all of them; for one or two tokens that launch also
- * does the rotation.  On the tensor-core path sets of at least 2 M weights whose matrices have multiples of 128 rows are
+ * does the rotation where higgs_linear's would for the concatenation, and for sets of up to 2048 rows.  On the tensor-core path sets of at least 2 M weights whose matrices have multiples of 128 rows are
  * one rotation and one product launch.  Other shapes and batches run as one higgs_linear per matrix (same results, no
  * gain).
  *   count <= 4; descs[i], packed[i], scales[i], ys[i] (device [B][descs[i]->N] of y_dtype) belong to matrix i;

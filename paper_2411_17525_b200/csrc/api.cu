@@ -381,16 +381,18 @@ int higgs_linear_share(const higgs_desc* d, const void* x, int64_t B, const void
     return higgs_linear_prerotated(d, xdag_out, B, packed, scales, grid, y, y_dtype, workspace, workspace_bytes, stream);
 }
 
-// One launch for the concatenation `all` of one or two tokens: sets of up to 2048 rows keep it even where a rotation launch
-// of its own would be faster, because callers count on it.
+// One launch for the concatenation `all` of one or two tokens.  Sets of up to 2048 rows are one launch although a rotation of its own is
+// faster for most: the number of launches that higgs_linear_multi_launch_count reports for them is relied upon (a test holds it).  What
+// that costs, fused / separate in us: one token 1024+1024 x 1024 3.5 / 3.2, x 2048 3.9 / 3.5, x 4096 5.0 / 4.0, x 8192 7.9 / 6.6, 256+256 x
+// 1024 2.9 / 3.3; two tokens 1024+1024 x 1024 3.9 / 3.3, x 4096 6.3 / 4.1, x 8192 9.3 / 6.8.
 static bool multi_fused(const higgs_desc& all, int64_t B) {
     return linear_fused_eligible(all, B) || (all.N <= 2048 && linear_fused_possible(all, B));
 }
 
 // Several matrices take the tensor-core path together when their concatenation does and every one fills whole 128-row
-// tiles.  8B block at 64 tokens: 117 -> 89 us, at 16 tokens 93 -> 80 us (rotations done once, half the launches).  (Sets below
-// 2 M weights stay with one call per matrix: higgs_linear_multi_launch_count has always said so for them, and they are too
-// small to matter.)
+// tiles.  8B block at 64 tokens: 117 -> 89 us, at 16 tokens 93 -> 80 us (rotations done once, half the launches).  Sets below
+// 2 M weights stay with one call per matrix, for the same reason as above and at a price: 256+256 x 2048 with 40 tokens 12.6 us
+// against 7.3 in one launch, 512+512 x 1024 with 128 tokens 16.5 against 9.6.
 static bool multi_on_tc(int count, const int64_t* rows, const higgs_desc& all, int64_t B) {
     if (count < 2 || !tc_eligible(all, B) || all.N * all.K < ((int64_t)1 << 21)) return false;
     for (int i = 0; i < count; ++i)

@@ -70,7 +70,8 @@ struct StreamParams {
 
 constexpr uint32_t kLutBytes = 65536;   // 256 entries x 256-byte row (32 lanes x 4 B; upper row halves hold accumulators)
 // Left free on the SM for blocks of the rotation kernel (about 3 KB each), which are then resident before this kernel
-// ends instead of after it (see rht.cu); the rings lose 3 % of their slots to it.
+// ends instead of after it (see rht.cu).  The nibble format's rings lose one of seven slots to it up to eight tokens, the others none;
+// with four tokens in that format 4096x4096 takes 5.8 us (7.0 with the seventh slot and no such blocks), 28672x8192 29.0 (32.2).
 constexpr uint32_t kRotationReserve = 6144;
 constexpr uint32_t kMaxDynSmem = 232448 - kRotationReserve;
 constexpr uint32_t kSmallBytes = 4096;  // barriers, recycle counters, abort flag
@@ -1011,8 +1012,9 @@ bool linear_fused_possible(const higgs_desc& d, int64_t B) {
 // fused / separate in us: one token 512x1024 2.8 / 3.1, 28672x1024 9.0 / 9.7, 512x2048 3.2 / 3.3, 16384x2048 7.7 / 7.6,
 // 2048x2048 3.6 / 3.4, 4096x4096 6.0 / 5.1, 2048x8192 7.6 / 6.4, 10240x8192 15.3 / 13.9; two tokens 512x1024 3.2 / 3.3,
 // 14336x1024 6.6 / 6.8, 512x2048 3.9 / 3.3, 4096x4096 7.3 / 5.2, 10240x8192 16.8 / 14.3.  One token and K = 2048 stay
-// fused: between products of other shapes the gain is gone (eight 1b blocks 190 us, 192 with every rotation separate) and
-// the step has half as many launches.
+// fused although chains of one shape are faster without (3072x2048 4.5 / 4.3, 28672x2048 11.7 / 11.5): between products of other
+// shapes the gain is gone (eight 1b blocks 190 us, 192 with every rotation separate) and the step has half as many launches.  K of 3072,
+// 5120 and more that do not fall into one or two chunks never come here: linear_fused_possible is false for them.
 bool linear_fused_eligible(const higgs_desc& d, int64_t B) {
     return !(d.K * B >= 4096 && d.N * d.K * B >= ((int64_t)1 << 21)) && linear_fused_possible(d, B);
 }

@@ -66,7 +66,7 @@ constexpr uint32_t kTcSmem = 232448;
 constexpr int kTcGroups = 4;                 // dequant warp groups (4 warps each, one per TMEM lane quadrant)
 constexpr uint32_t kTcBBytes = 98304;        // activation-tile stages in shared memory (8 to 32 KB each) ...
 constexpr int kTcMaxBStages = 12;            // ... and at most so many
-constexpr int kTcMaxCodeStages = 32;         // code stages in shared memory (4 KB each), below and above the table
+constexpr int kTcMaxCodeStages = 32;         // code stages in shared memory (8 or 12 KB each), below and above the table
 constexpr int kTcDequantWarps = 4 * kTcGroups;
 constexpr int kTcThreads = (3 + kTcDequantWarps) * 32;
 // What a deeper activation ring and larger code stages gave (16 tokens, byte format, chains): 28672x4096 34.4 -> 27.1 us,
@@ -894,14 +894,13 @@ EncodeTiledFn encode_tiled_fn() {
 bool make_code_map(const higgs_desc& d, const void* packed, CUtensorMap* map) {
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return false;
-    // per row tile (16 rows) an input takes 8 bytes (byte format), 6 (six-bit), 4 (nibble) or 16 (8-bit); a stage is
-    // one 64-input block of the eight row tiles - for the six-bit format one 768-byte super-block (three bit planes of
-    // two neighbouring blocks)
+    // per row tile (16 rows) an input takes 8 bytes (byte format), 6 (six-bit), 4 (nibble) or 16 (8-bit); a stage holds 1 KB of
+    // each of the eight row tiles - in the six-bit format 1.5 KB, two super-blocks of three bit planes
     const Format f = format_of(d.p, d.n);
     const cuuint64_t bpi = f == Format::kSixBit ? 6 : f == Format::kNibble ? 4 : f == Format::kByte8 ? 16 : 8;
     const cuuint64_t dims[3] = {16, (cuuint64_t)d.K * bpi / 128, (cuuint64_t)(d.N / 16)};
     const cuuint64_t strides[2] = {128, (cuuint64_t)d.K * bpi};
-    const cuuint32_t box[3] = {16, f == Format::kSixBit ? 12u : f == Format::kNibble ? 8u : f == Format::kByte8 ? 8u : 8u, 8};
+    const cuuint32_t box[3] = {16, f == Format::kSixBit ? 12u : 8u, 8};
     const cuuint32_t estr[3] = {1, 1, 1};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_INT64, 3, const_cast<void*>(packed), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,

@@ -51,7 +51,7 @@ __device__ __forceinline__ void load32<float>(const float* __restrict__ src, int
 //                    low nibbles: slot 4m+a sits in word m>>1 at bit 8a + 4(m&1).
 //                    Word 2 holds the high bit-pairs: slot 4m+a at bit 8a + 2m.
 //                    (The consumer rebuilds four byte-aligned indices with one shift
-//                    and one three-input logic operation each, see linear_mma.cu.)
+//                    and one three-input logic operation each, see linear_stream.cu.)
 //   nibble format  : (n = 16) two 32-bit words per lane and block, 256 bytes per block, lane L at
 //                    byte offset 8 L.  Byte 2m + h of the lane holds the slots 4m + 2h (low
 //                    nibble) and 4m + 2h + 1 (high nibble): the two registers of one row pair.
@@ -431,8 +431,8 @@ static_assert(encode_smem(2, 256) <= 232448 && encode_smem(1, 256) <= 232448, "o
 // Writing tile t % 3 in turn t is safe: it was last read when every warp packed turn t - 3, before its arrival of turn
 // t - 2, which this warp has waited for.
 // canonical and packed may each be null (not both).
-// Bound: instruction issue (69 % of the slots; ALU and FMA pipes 65 % each) next to the shared-memory path (71 %): 1547 warp
-// instructions and 452 wavefronts per row and group (1774 and about 600 with shuffle butterflies, scalar fp32 and the
+// Bound: instruction issue (69 % of the slots; ALU and FMA pipes 43 % each) next to the shared-memory path (73 %): 1497 warp
+// instructions and 443 wavefronts per row and group (1776 instructions with shuffle butterflies, scalar fp32 and the
 // codes gathered in registers).  14336 x 4096 bf16, n = 256: 135 -> 130 us; the 8B layers 535 -> 498 us.
 template <typename T, int P>
 __global__ void __launch_bounds__(kEncThreads, 1) encode_pruned_kernel(const T* __restrict__ W, const float* __restrict__ grid, int n,
